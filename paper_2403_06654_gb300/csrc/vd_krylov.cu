@@ -9,6 +9,7 @@
 // iteration return at once when the flag is set, so iterations enqueued ahead cost a launch
 // each and change nothing.
 #include "vd_krylov.cuh"
+#include "vd_dd.cuh"
 #include "vd_prof.h"
 
 #include <algorithm>
@@ -35,63 +36,117 @@ __device__ __forceinline__ cpx<double> ld(const cpx<T>* p, long long e) {
   return mk<double>((double)v.x, (double)v.y);
 }
 
-// Block-sum v[0..NV) into per-block partials; the last block gets the totals in thread 0.
-// Returns true (in every thread of the last block) when the caller must run the epilogue.
+// float -> double on the integer pipes (exact; subnormals take the conversion instruction).  The
+// FP64 pipe of GB300, which also converts, takes ~17 cycles per warp instruction and SM, and a
+// reduction's tail is bound by it.
+__device__ __forceinline__ double widen(float f) {
+  const unsigned u = __float_as_uint(f);
+  return ((u & 0x7f800000u) == 0u && (u & 0x7fffffu) != 0u) ? (double)f : f2d_bits(f);
+}
+
+__host__ __device__ constexpr int log2_ceil(int n) { return n <= 1 ? 0 : 1 + log2_ceil((n + 1) / 2); }
+
+// Sums of v[0..NV) (NV <= 32) over the block, one value per group of 8 threads: on return
+// thread 8 i holds the total of value i (other threads nothing).  Within a warp the values are
+// exchanged and halved (lanes whose bit is set keep the upper half of the values, the others the
+// lower half), so NV values cost about NV + 5 - log2 NV additions per lane instead of 5 NV: the
+// tail of a reduction kernel is its FP64 additions (8 values with one butterfly each, 608 blocks:
+// k_gm_mdot 31 us on 87k points, 6 us this way).
 template <int NV>
-__device__ bool reduce_last(double (&v)[NV], double* partials, unsigned* counter, double (&tot)[NV]) {
+__device__ __forceinline__ double block_sums(const double (&v)[NV], double (*sm)[kRedThreads / 32]) {
+  constexpr int L = log2_ceil(NV), P = 1 << L;
+  static_assert(NV >= 1 && P <= 32 && kRedThreads == 256, "one exchange step per lane bit");
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  double a[P];
+#pragma unroll
+  for (int i = 0; i < P; ++i) a[i] = i < NV ? v[i < NV ? i : 0] : 0.0;
+#pragma unroll
+  for (int s = 0; s < 5; ++s) {
+    const int o = 16 >> s, cnt = P >> (s + 1);   // values kept after this step
+    if (cnt >= 1) {
+      const bool up = (lane & o) != 0;
+#pragma unroll
+      for (int i = 0; i < cnt; ++i) {
+        const double give = up ? a[i] : a[i + cnt], keep = up ? a[i + cnt] : a[i];
+        a[i] = keep + __shfl_xor_sync(0xffffffffu, give, o);
+      }
+    } else {
+      a[0] += __shfl_xor_sync(0xffffffffu, a[0], o);
+    }
+  }
+  const int mine = lane >> (5 - L);   // the value this lane ended with
+  if ((lane & ((32 >> L) - 1)) == 0 && mine < NV) sm[mine][warp] = a[0];
+  __syncthreads();
+  double s = 0.0;
+  if (warp * 4 < NV) {   // warps holding a thread t with t / 8 < NV
+    const int i = threadIdx.x >> 3;
+    if (i < NV) s = sm[i][threadIdx.x & 7];
+    s += __shfl_xor_sync(0xffffffffu, s, 4);
+    s += __shfl_xor_sync(0xffffffffu, s, 2);
+    s += __shfl_xor_sync(0xffffffffu, s, 1);
+  }
+  return s;
+}
+
+// Block-sum v[0..NV) into per-block partials (partials[i * blocks + block]); the last block gets
+// the totals in tot (every thread).  Returns true (in every thread of the last block) when the
+// caller must run the epilogue.  Fixed order: deterministic.
+template <int NV>
+__device__ bool reduce_last(const double (&v)[NV], double* partials, unsigned* counter, double (&tot)[NV]) {
   __shared__ double sm[NV][kRedThreads / 32];
   __shared__ int am_last;
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-#pragma unroll
-  for (int i = 0; i < NV; ++i) {
-    double s = v[i];
-    for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
-    if (lane == 0) sm[i][warp] = s;
-  }
-  __syncthreads();
-  if (threadIdx.x == 0) {
-#pragma unroll
-    for (int i = 0; i < NV; ++i) {
-      double s = 0.0;
-      for (int w = 0; w < kRedThreads / 32; ++w) s += sm[i][w];
-      partials[blockIdx.x * NV + i] = s;
+  const int nb = (int)gridDim.x;
+  const int vi = threadIdx.x >> 3;
+  const double s = block_sums<NV>(v, sm);
+  if (nb > 1) {
+    if ((threadIdx.x & 7) == 0 && vi < NV) {
+      partials[vi * nb + blockIdx.x] = s;
+      __threadfence();
     }
+    __syncthreads();
+    if (threadIdx.x == 0) am_last = (atomicAdd(counter, 1u) == (unsigned)nb - 1u) ? 1 : 0;
+    __syncthreads();
+    if (!am_last) return false;
     __threadfence();
-    const unsigned t = atomicAdd(counter, 1u);
-    am_last = (t == gridDim.x - 1) ? 1 : 0;
-  }
-  __syncthreads();
-  if (!am_last) return false;
-  __threadfence();
-  double a[NV];
+    double a[NV];
+    if constexpr (NV < 8) {
 #pragma unroll
-  for (int i = 0; i < NV; ++i) a[i] = 0.0;
-  for (int b = threadIdx.x; b < (int)gridDim.x; b += blockDim.x) {
+      for (int i = 0; i < NV; ++i) a[i] = 0.0;
+      for (int b = threadIdx.x; b < nb; b += kRedThreads) {
 #pragma unroll
-    for (int i = 0; i < NV; ++i) a[i] += __ldcg(partials + b * NV + i);
-  }
-  __syncthreads();
+        for (int i = 0; i < NV; ++i) a[i] += __ldcg(partials + i * nb + b);
+      }
+      const double f = block_sums<NV>(a, sm);
+      if ((threadIdx.x & 7) == 0 && vi < NV) sm[vi][0] = f;
+    } else {
+      // warp w sums the values w, w + 8, ...
+      const int lane = threadIdx.x & 31;
+      for (int i = threadIdx.x >> 5; i < NV; i += kRedThreads / 32) {
+        double f = 0.0;
+        for (int b = lane; b < nb; b += 32) f += __ldcg(partials + i * nb + b);
 #pragma unroll
-  for (int i = 0; i < NV; ++i) {
-    double s = a[i];
-    for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
-    if (lane == 0) sm[i][warp] = s;
-  }
-  __syncthreads();
-  if (threadIdx.x == 0) {
-#pragma unroll
-    for (int i = 0; i < NV; ++i) {
-      double s = 0.0;
-      for (int w = 0; w < kRedThreads / 32; ++w) s += sm[i][w];
-      tot[i] = s;
+        for (int o = 16; o > 0; o >>= 1) f += __shfl_xor_sync(0xffffffffu, f, o);
+        if (lane == 0) sm[i][0] = f;
+      }
     }
-    *counter = 0u;
+    if (threadIdx.x == 0) *counter = 0u;
+  } else {
+    __syncthreads();   // sm is read by block_sums' last step
+    if ((threadIdx.x & 7) == 0 && vi < NV) sm[vi][0] = s;
   }
+  __syncthreads();
+#pragma unroll
+  for (int i = 0; i < NV; ++i) tot[i] = sm[i][0];
   return true;
 }
 
+// Blocks of a reduction over len elements: up to one per SM while that leaves a thread at most
+// kRedPerThread elements, then up to four (the tail's FP64 work grows with the blocks of an SM).
 static inline int red_blocks(long long len) {
-  return (int)std::max<long long>(1, std::min<long long>(kRedBlocks, (len + kRedThreads - 1) / kRedThreads));
+  constexpr long long kRedPerThread = 8, one = kRedBlocks / 4;
+  const long long need = (len + kRedThreads - 1) / kRedThreads;
+  if (need <= one * kRedPerThread) return (int)std::max<long long>(1, std::min(one, need));
+  return (int)std::min<long long>(kRedBlocks, (need + kRedPerThread - 1) / kRedPerThread);
 }
 
 #define GRID_STRIDE(e, len) \
@@ -263,23 +318,29 @@ __device__ void epilogue(int epi, const double (&t)[NV], KState* ks, double* his
     case EPI_GM_NORM: {
       const int m = ks->m;
       const double hn = sqrt(t[0]);
-      double* col = ks->H + (size_t)j * (m + 1);
-      for (int i = 0; i <= j; ++i) col[i] = ks->h1[i] + ks->h2[i];
-      col[j + 1] = hn;
+      double* __restrict__ col = ks->H + (size_t)j * (m + 1);
+      const double* __restrict__ h1 = ks->h1;
+      const double* __restrict__ h2 = ks->h2;
+      const double* __restrict__ cs = ks->cs;
+      const double* __restrict__ sn = ks->sn;
+      // the entry a rotation passes on stays in a register; the loads of the next rotations
+      // (unrolled) do not wait for it
+      double cur = h1[0] + h2[0];
+#pragma unroll 4
       for (int i = 0; i < j; ++i) {
-        const double a = ks->cs[i] * col[i] + ks->sn[i] * col[i + 1];
-        col[i + 1] = -ks->sn[i] * col[i] + ks->cs[i] * col[i + 1];
-        col[i] = a;
+        const double nx = h1[i + 1] + h2[i + 1], ci = cs[i], si = sn[i];
+        col[i] = ci * cur + si * nx;
+        cur = -si * cur + ci * nx;
       }
       double c = 1.0, s = 0.0;
-      if (col[j + 1] != 0.0) {
-        const double h = hypot(col[j], col[j + 1]);
-        c = col[j] / h;
-        s = col[j + 1] / h;
+      if (hn != 0.0) {
+        const double h = hypot(cur, hn);
+        c = cur / h;
+        s = hn / h;
       }
       ks->cs[j] = c;
       ks->sn[j] = s;
-      col[j] = c * col[j] + s * col[j + 1];
+      col[j] = c * cur + s * hn;
       col[j + 1] = 0.0;
       ks->gv[j + 1] = -s * ks->gv[j];
       ks->gv[j] = c * ks->gv[j];
@@ -348,6 +409,7 @@ template <typename T>
 struct Acc {
   double a = 0.0;
   __device__ __forceinline__ void add(T v) { a += (double)v; }
+  __device__ __forceinline__ void dot(cpx<T> u, cpx<T> v) { a = fma(u.x, v.x, fma(u.y, v.y, a)); }   // += Re(u conj v)
   __device__ __forceinline__ double total() const { return a; }
 };
 template <>
@@ -359,7 +421,8 @@ struct Acc<float> {
     c += (s - (t - bp)) + (v - bp);
     s = t;
   }
-  __device__ __forceinline__ double total() const { return (double)s + (double)c; }
+  __device__ __forceinline__ void dot(cpx<float> u, cpx<float> v) { add(u.x * v.x + u.y * v.y); }
+  __device__ __forceinline__ double total() const { return widen(s) + widen(c); }
 };
 
 // CG start: p = S r, reduce [bb, rr, rz]
@@ -392,10 +455,9 @@ __global__ void __launch_bounds__(kRedThreads) k_dot(Ix ix, const cpx<T>* __rest
   if (*done) return;
   Acc<T> a0, a1;
   IX_LOOP(ix) {
-    const T w = pweight<T>(kx, ix.h0);
-    const cpx<T> uu = u[e], vv = v[e];
-    a0.add(w * (uu.x * vv.x + uu.y * vv.y));
-    if (NV > 1) a1.add(w * (vv.x * vv.x + vv.y * vv.y));
+    const cpx<T> vv = v[e], wv = scal(vv, pweight<T>(kx, ix.h0));   // the weight is 1 or 2: exact
+    a0.dot(wv, u[e]);
+    if (NV > 1) a1.dot(wv, vv);
   }
   double a[NV];
   a[0] = a0.total();
@@ -534,30 +596,59 @@ __global__ void k_gm_scale(Ix ix, cpx<T>* __restrict__ dst, const cpx<T>* __rest
     dst[e] = scal(src[e], s);
 }
 
-// GMRES: h[off + i] = (w, V_{off+i})_w for i < nv (<= 8)
-template <typename T>
+// GMRES orthogonalisation (classical Gram-Schmidt twice).  k_gm_mdot: h1[off + i] =
+// (w, V_{off+i})_w for i < nv <= NB.  k_gm_step: w -= sum_{i<nv} h1_i V_i, then h2_i = (w, V_i)_w in
+// the same pass: every vector is local to an element, so V is read once, into registers, for both
+// (the pair was two kernels and, at 8 vectors per dot kernel, up to nine launches per iteration).
+// Up to 32 basis vectors; past that the dots run 32 at a time and the update apart.
+template <typename T, int NB>
 __global__ void __launch_bounds__(kRedThreads) k_gm_mdot(Ix ix, const cpx<T>* __restrict__ w,
                                                          const cpx<T>* __restrict__ V, int off, int nv, int epi, int j,
                                                          RedArgs ra) {
   if (ra.ks->cycle_done) return;
-  Acc<T> a[8];
+  Acc<T> a[NB];
   IX_LOOP(ix) {
-    const T wt = pweight<T>(kx, ix.h0);
-    const cpx<T> wv = w[e];
+    const cpx<T> wv = scal(w[e], pweight<T>(kx, ix.h0));   // the weight is 1 or 2: exact
 #pragma unroll
-    for (int i = 0; i < 8; ++i) {
-      if (i < nv) {
-        const cpx<T> vv = V[(size_t)(off + i) * ix.len + e];
-        a[i].add(wt * (wv.x * vv.x + wv.y * vv.y));
-      }
-    }
+    for (int i = 0; i < NB; ++i)
+      if (i < nv) a[i].dot(wv, V[(size_t)(off + i) * ix.len + e]);
   }
-  double v[8];
+  double v[NB];
 #pragma unroll
-  for (int i = 0; i < 8; ++i) v[i] = a[i].total();
-  double t[8];
-  if (reduce_last<8>(v, ra.partials, ra.counter, t) && threadIdx.x == 0)
-    epilogue<8>(epi, t, ra.ks, ra.hist, ra.tol, off, j);
+  for (int i = 0; i < NB; ++i) v[i] = a[i].total();
+  double t[NB];
+  if (reduce_last<NB>(v, ra.partials, ra.counter, t) && threadIdx.x == 0)
+    epilogue<NB>(epi, t, ra.ks, ra.hist, ra.tol, off, j);
+}
+
+template <typename T, int NB>
+__global__ void __launch_bounds__(kRedThreads) k_gm_step(Ix ix, cpx<T>* __restrict__ w, const cpx<T>* __restrict__ V,
+                                                         int nv, RedArgs ra) {
+  if (ra.ks->cycle_done) return;
+  __shared__ T hs[NB];
+  for (int i = threadIdx.x; i < NB; i += blockDim.x) hs[i] = (i < nv) ? (T)ra.ks->h1[i] : T(0);
+  __syncthreads();
+  Acc<T> a[NB];
+  IX_LOOP(ix) {
+    cpx<T> wv = w[e], vv[NB];
+#pragma unroll
+    for (int i = 0; i < NB; ++i)
+      if (i < nv) vv[i] = V[(size_t)i * ix.len + e];
+#pragma unroll
+    for (int i = 0; i < NB; ++i)
+      if (i < nv) wv = mk<T>(fma(-hs[i], vv[i].x, wv.x), fma(-hs[i], vv[i].y, wv.y));
+    w[e] = wv;
+    wv = scal(wv, pweight<T>(kx, ix.h0));
+#pragma unroll
+    for (int i = 0; i < NB; ++i)
+      if (i < nv) a[i].dot(wv, vv[i]);
+  }
+  double v[NB];
+#pragma unroll
+  for (int i = 0; i < NB; ++i) v[i] = a[i].total();
+  double t[NB];
+  if (reduce_last<NB>(v, ra.partials, ra.counter, t) && threadIdx.x == 0)
+    epilogue<NB>(EPI_GM_H2, t, ra.ks, ra.hist, ra.tol, 0, nv - 1);
 }
 
 // GMRES: w -= sum_{i<=j} h_i V_i (h = h1 or h2); with_norm: reduce [(w,w)] -> EPI_GM_NORM
@@ -573,13 +664,14 @@ __global__ void __launch_bounds__(kRedThreads) k_gm_maxpy(Ix ix, cpx<T>* __restr
   Acc<T> a0;
   IX_LOOP(ix) {
     cpx<T> wv = w[e];
+#pragma unroll 8
     for (int i = 0; i <= j; ++i) {
       const T c = hs[i];
       const cpx<T> vv = V[(size_t)i * ix.len + e];
       wv = mk<T>(fma(-c, vv.x, wv.x), fma(-c, vv.y, wv.y));
     }
     w[e] = wv;
-    a0.add(pweight<T>(kx, ix.h0) * (wv.x * wv.x + wv.y * wv.y));
+    a0.dot(scal(wv, pweight<T>(kx, ix.h0)), wv);
   }
   if (!with_norm) return;
   double v[1] = {a0.total()};
@@ -588,14 +680,69 @@ __global__ void __launch_bounds__(kRedThreads) k_gm_maxpy(Ix ix, cpx<T>* __restr
     epilogue<1>(EPI_GM_NORM, t, ra.ks, ra.hist, ra.tol, 0, j);
 }
 
-// GMRES: back substitution H(0:k,0:k) y = g (one thread)
-__global__ void k_gm_solve(KState* ks) {
-  if (ks->done || threadIdx.x != 0 || blockIdx.x != 0) return;
-  const int k = ks->k, m = ks->m;
-  for (int i = k - 1; i >= 0; --i) {
-    double s = ks->gv[i];
-    for (int l = i + 1; l < k; ++l) s -= ks->H[i + (size_t)l * (m + 1)] * ks->y[l];
-    ks->y[i] = s / ks->H[i + (size_t)i * (m + 1)];
+static inline Ix mkix(long long len, int h0, long long nc, int blocks, int threads);
+
+// NB vectors per thread: the least of 2, 4, 8, 16, 32 that holds nv
+#define GM_BY_COUNT(nv, CALL)       \
+  do {                              \
+    if ((nv) <= 2) CALL(2);         \
+    else if ((nv) <= 4) CALL(4);    \
+    else if ((nv) <= 8) CALL(8);    \
+    else if ((nv) <= 16) CALL(16);  \
+    else CALL(32);                  \
+  } while (0)
+
+// the orthogonalisation of w against V_0..V_j on st: h1, h2, w and |w| (EPI_GM_NORM)
+template <typename T>
+static void gm_orthogonalise(const SpecSystem& sys, cpx<T>* w, const cpx<T>* V, int j, const RedArgs& ra,
+                             cudaStream_t st) {
+  const int n = j + 1;
+  const int cls = sizeof(T) == 4 ? PC_VEC32 : PC_VEC64;
+  const double el = (double)sys.len * sizeof(cpx<T>);
+  // the partials hold 8 kRedBlocks values: fewer blocks for more values
+  auto blocks = [&](int nb) { return std::min(red_blocks(sys.len), kRedBlocks * 8 / nb); };
+  auto index = [&](int rb) { return mkix(sys.len, sys.h0, sys.G->g.ncplx, rb, kRedThreads); };
+  auto mdot = [&](int off, int nv, int epi) {
+    ProfScope ps_(cls, st, (nv + 1) * el, 0.0);
+#define GM_MDOT(NB) \
+  k_gm_mdot<T, NB><<<blocks(NB), kRedThreads, 0, st>>>(index(blocks(NB)), w, V, off, nv, epi, j, ra)
+    GM_BY_COUNT(nv, GM_MDOT);
+#undef GM_MDOT
+  };
+  auto maxpy = [&](int which) {
+    ProfScope ps_(cls, st, (n + 2) * el, 0.0);
+    k_gm_maxpy<T><<<blocks(1), kRedThreads, 0, st>>>(index(blocks(1)), w, V, j, which, which, ra);
+  };
+  for (int off = 0; off < n; off += 32) mdot(off, std::min(32, n - off), EPI_GM_H1);
+  if (n <= 32) {
+    ProfScope ps_(cls, st, (n + 2) * el, 0.0);
+#define GM_STEP(NB) k_gm_step<T, NB><<<blocks(NB), kRedThreads, 0, st>>>(index(blocks(NB)), w, V, n, ra)
+    GM_BY_COUNT(n, GM_STEP);
+#undef GM_STEP
+  } else {
+    maxpy(0);
+    for (int off = 0; off < n; off += 32) mdot(off, std::min(32, n - off), EPI_GM_H2);
+  }
+  maxpy(1);
+}
+#undef GM_BY_COUNT
+
+// GMRES: back substitution H(0:k,0:k) y = g: one warp, column by column, the triangle in shared
+// memory (one thread reading it from global memory took 35 us at k = 30)
+__global__ void __launch_bounds__(32) k_gm_solve(KState* ks) {
+  if (ks->done) return;
+  __shared__ double tri[kMaxRestart * kMaxRestart], g[kMaxRestart];
+  const int k = ks->k, m = ks->m, lane = threadIdx.x;
+  for (int l = 0; l < k; ++l)
+    for (int i = lane; i <= l; i += 32) tri[i + l * kMaxRestart] = ks->H[i + (size_t)l * (m + 1)];
+  for (int i = lane; i < k; i += 32) g[i] = ks->gv[i];
+  __syncwarp();
+  for (int l = k - 1; l >= 0; --l) {
+    const double y = g[l] / tri[l + l * kMaxRestart];
+    __syncwarp();
+    for (int i = lane; i < l; i += 32) g[i] -= tri[i + l * kMaxRestart] * y;
+    if (lane == 0) ks->y[l] = y;
+    __syncwarp();
   }
 }
 
@@ -992,13 +1139,7 @@ vd_status krylov_solve(const SpecSystem& sys, const SolveOpts& o, const void* b,
       for (int j = 0; j < m; ++j) {
         cpx<T>* Vj = V + (size_t)j * len;
         sys.apply(sys, Vj, w, true, cdone, st);
-        for (int pass = 0; pass < 2; ++pass) {
-          for (int off = 0; off <= j; off += 8) {
-            const int nv = std::min(8, j + 1 - off);
-            { ProfScope ps_(sizeof(T) == 4 ? PC_VEC32 : PC_VEC64, st, (double)(nv + 1) * len * sizeof(cpx<T>), 0.0); k_gm_mdot<T><<<rb, kRedThreads, 0, st>>>(ixr, w, V, off, nv, pass ? EPI_GM_H2 : EPI_GM_H1, j, ra); }
-          }
-          { ProfScope ps_(sizeof(T) == 4 ? PC_VEC32 : PC_VEC64, st, (double)(j + 3) * len * sizeof(cpx<T>), 0.0); k_gm_maxpy<T><<<rb, kRedThreads, 0, st>>>(ixr, w, V, j, pass, pass, ra); }
-        }
+        gm_orthogonalise<T>(sys, w, V, j, ra, st);
         { ProfScope ps_(sizeof(T) == 4 ? PC_VEC32 : PC_VEC64, st, (double)2 * len * sizeof(cpx<T>), 0.0); k_gm_scale<T><<<eb, 256, 0, st>>>(ixe, V + (size_t)(j + 1) * len, w, kw.ks, 0); }
         if ((j + 1) % check == 0 || j + 1 == m) {
           vd_status e = read_head(kw, &hd, st);
@@ -1006,7 +1147,7 @@ vd_status krylov_solve(const SpecSystem& sys, const SolveOpts& o, const void* b,
           if (hd.cycle_done || hd.done) break;
         }
       }
-      { k_gm_solve<<<1, 1, 0, st>>>(kw.ks); count_launch(); }
+      { k_gm_solve<<<1, 32, 0, st>>>(kw.ks); count_launch(); }
       { ProfScope ps_(sizeof(T) == 4 ? PC_VEC32 : PC_VEC64, st, (double)(m + 2) * len * sizeof(cpx<T>) + (double)nc * sizeof(T), 0.0); k_gm_update<T><<<eb, 256, 0, st>>>(ixe, X, V, sym, kw.ks); }
       { k_gm_close<<<1, 1, 0, st>>>(kw.ks); count_launch(); }
       vd_status e = read_head(kw, &hd, st);
@@ -1192,19 +1333,11 @@ vd_status krylov_enqueue_graph(const SpecSystem& sys, const SolveOpts& o, const 
     for (int j = 0; j < m; ++j) {
       cpx<T>* Vj = V + (size_t)j * len;
       sys.apply(sys, Vj, w, true, cdone, body_st);
-      for (int pass = 0; pass < 2; ++pass) {
-        for (int off = 0; off <= j; off += 8) {
-          const int nv = std::min(8, j + 1 - off);
-          k_gm_mdot<T><<<rb, kRedThreads, 0, body_st>>>(ixr, w, V, off, nv, pass ? EPI_GM_H2 : EPI_GM_H1, j, ra);
-          count_launch();
-        }
-        k_gm_maxpy<T><<<rb, kRedThreads, 0, body_st>>>(ixr, w, V, j, pass, pass, ra);
-        count_launch();
-      }
+      gm_orthogonalise<T>(sys, w, V, j, ra, body_st);
       k_gm_scale<T><<<eb, 256, 0, body_st>>>(ixe, V + (size_t)(j + 1) * len, w, kw.ks, 0);
       count_launch();
     }
-    k_gm_solve<<<1, 1, 0, body_st>>>(kw.ks);
+    k_gm_solve<<<1, 32, 0, body_st>>>(kw.ks);
     k_gm_update<T><<<eb, 256, 0, body_st>>>(ixe, X, V, sym, kw.ks);
     k_gm_close<<<1, 1, 0, body_st>>>(kw.ks);
     count_launch();
