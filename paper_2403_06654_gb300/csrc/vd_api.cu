@@ -47,6 +47,39 @@ static bool make_plan(int n, FftPlan* p) {
   return p->nst <= kMaxStages;
 }
 
+// Plan of vd_wide.cuh in radices up to `most`: the fewest stages, then the smallest largest radix,
+// then powers of two first (the index k = i mod p of a middle stage is then a mask).
+static void wide_search(int n, int least, int most, WidePlan* cur, WidePlan* best) {
+  static const int rads[] = {2, 3, 4, 5, 6, 8, 9, 10, 12, 15, 16};
+  if (n == 1) {
+    auto top = [](const WidePlan& p) { return *std::max_element(p.rad, p.rad + p.nst); };
+    if (best->nst == 0 || cur->nst < best->nst || (cur->nst == best->nst && top(*cur) < top(*best))) *best = *cur;
+    return;
+  }
+  if (cur->nst == 8 || (best->nst > 0 && cur->nst >= best->nst)) return;
+  for (int r : rads)
+    if (r >= least && r <= most && n % r == 0) {
+      cur->rad[cur->nst++] = (int8_t)r;
+      wide_search(n / r, r, most, cur, best);
+      --cur->nst;
+    }
+}
+bool make_wide_plans(int n, int tw_off, WidePlan p[kWideClasses]) {
+  for (int k = 0; k < kWideClasses; ++k) {
+    WidePlan cur{}, best{};
+    wide_search(n, 2, kWideMost[k], &cur, &best);
+    if (best.nst == 0) return false;
+    std::sort(best.rad, best.rad + best.nst, [](int a, int b) {
+      const bool pa = (a & (a - 1)) == 0, pb = (b & (b - 1)) == 0;
+      return pa != pb ? pa : a > b;
+    });
+    p[k] = best;
+    p[k].n = (int16_t)n;
+    p[k].tw_off = tw_off;
+  }
+  return true;
+}
+
 // exp(-2 pi i j / n) evaluated in extended precision
 static void twiddle_ld(long long j, long long n, long double* re, long double* im) {
   j %= n;
@@ -108,9 +141,9 @@ bool grid_desc_only(int ndim, const int n[3], const double L[3], vd_grid* G) {
   g.nreal = (long long)nn[0] * nn[1] * nn[2];
   g.ncplx = (long long)g.h0 * nn[1] * nn[2];
   for (int j = 0; j < 3; ++j) G->L[j] = (j < ndim) ? L[j] : 1.0;
-  bool ok = make_plan(nn[0] / 2, &g.px);
-  if (ndim >= 2) ok = ok && make_plan(nn[1], &g.py);
-  if (ndim == 3) ok = ok && make_plan(nn[2], &g.pz);
+  bool ok = make_plan(nn[0] / 2, &g.px) && make_wide_plans(nn[0] / 2, 0, g.wx);
+  if (ndim >= 2) ok = ok && make_plan(nn[1], &g.py) && make_wide_plans(nn[1], 0, g.wy);
+  if (ndim == 3) ok = ok && make_plan(nn[2], &g.pz) && make_wide_plans(nn[2], 0, g.wz);
   return ok && g.ncplx * 3 < (1ll << 31);
 }
 }  // namespace vd
@@ -148,10 +181,10 @@ vd_status vd_grid_create(int ndim, const int n[3], const double L[3], vd_grid** 
     split_ld(kl, &g.kfac_dd[j][0], &g.kfac_dd[j][1]);
     g.kfac_f[j] = (float)g.kfac[j];
   }
-  bool ok = make_plan(nn[0] / 2, &g.px);
-  if (ndim >= 2) ok = ok && make_plan(nn[1], &g.py);
+  bool ok = make_plan(nn[0] / 2, &g.px) && make_wide_plans(nn[0] / 2, 0, g.wx);
+  if (ndim >= 2) ok = ok && make_plan(nn[1], &g.py) && make_wide_plans(nn[1], 0, g.wy);
   else g.py = g.px;
-  if (ndim == 3) ok = ok && make_plan(nn[2], &g.pz);
+  if (ndim == 3) ok = ok && make_plan(nn[2], &g.pz) && make_wide_plans(nn[2], 0, g.wz);
   else g.pz = g.py;
   if (!ok) {
     delete G;
@@ -173,6 +206,11 @@ vd_status vd_grid_create(int ndim, const int n[3], const double L[3], vd_grid** 
   else g.py.tw_off = g.px.tw_off;
   if (ndim == 3) add(g.pz);
   else g.pz.tw_off = g.py.tw_off;
+  for (int k = 0; k < kWideClasses; ++k) {
+    g.wx[k].tw_off = g.px.tw_off;
+    g.wy[k].tw_off = g.py.tw_off;
+    g.wz[k].tw_off = g.pz.tw_off;
+  }
   g.pk_off = (int)(tw.size() / 2);
   for (int k = 0; k <= nn[0] / 2; ++k) {
     double re, im;

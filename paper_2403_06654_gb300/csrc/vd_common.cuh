@@ -74,6 +74,16 @@ struct FftPlan {
   int tw_off;
 };
 
+// The same length for the passes of vd_wide.cuh, radices 2, 3, 4, 5, 6, 8, 9, 10, 12, 15 and 16 up to
+// the largest of its class (kWideMost), on the same table.
+struct WidePlan {
+  int16_t n, nst;
+  int8_t rad[8];
+  int tw_off;
+};
+constexpr int kWideClasses = 3;
+constexpr int kWideMost[kWideClasses] = {5, 8, 16};
+
 // Plans of one grid.  The x axis is transformed as a complex FFT of length m = n0/2 plus the
 // real-data packing step, which needs W_{n0}^k for k in [0, m] (table at pk_off).
 struct GridDesc {
@@ -88,6 +98,7 @@ struct GridDesc {
   FftPlan px;        // length n0/2
   FftPlan py;        // length n1 (ndim >= 2)
   FftPlan pz;        // length n2 (ndim == 3)
+  WidePlan wx[kWideClasses], wy[kWideClasses], wz[kWideClasses];
   int pk_off;        // packing twiddles W_{n0}^k, k = 0..n0/2
   int* dev_err = nullptr;   // device error word of the grid (a bounded wait gave up), or null
 };

@@ -105,6 +105,15 @@ __device__ __forceinline__ cpx<dd> csub_lazy(cpx<dd> a, cpx<dd> b) {
   return mk<dd>(dd_add_lazy(a.x, -b.x), dd_add_lazy(a.y, -b.y));
 }
 
+// z * (wh + wl) rounded once to float: the product with the high part is split exactly by an
+// FMA (Dekker's two-product), the low part's product is added to its error term before the
+// final rounding
+__device__ __forceinline__ float mul_pair(float z, float wh, float wl) {
+  const float p = z * wh;
+  const float e = fmaf(z, wh, -p);
+  return p + fmaf(z, wl, e);
+}
+
 // Conversions to and from double, on the integer pipes.  The FP64 pipe of GB300 runs at ~1/64
 // of the float rate, so the conversions are done on the IEEE bit patterns.
 //

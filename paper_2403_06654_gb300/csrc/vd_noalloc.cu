@@ -153,6 +153,10 @@ extern "C" vd_status vd_apply_pressure_noalloc(int ndim, const int n[3], const d
   } else {
     g.pz = g.py;
   }
+  // the transform passes' plans, on the same twiddle tables
+  const FftPlan* narrow[3] = {&g.px, &g.py, &g.pz};
+  WidePlan* wide[3] = {g.wx, g.wy, g.wz};
+  for (int j = 0; j < ndim; ++j) ok = ok && make_wide_plans(narrow[j]->n, narrow[j]->tw_off, wide[j]);
   if (!ok) return fail(VD_ERR_INVALID_ARG, "axis lengths must factor into 2, 3 and 5");
   g.pk_off = off;
   const size_t ntw = (size_t)off + g.n0 / 2 + 1;

@@ -19,11 +19,6 @@
 #include <mutex>
 
 namespace vd {
-static void ensure_smem(const void* func, size_t smem);
-static int sm_count();
-}
-
-namespace vd {
 
 // Element load / store of a pass.  The float-pair instantiation (T = dd) may read its input
 // from, and write its output to, double fields (the Krylov vectors), converting on the fly.
@@ -69,15 +64,6 @@ __device__ __forceinline__ T scale_t(double s, float hi, float lo) {
   else return s;
 }
 
-// z * (wh + wl) rounded once to float: the product with the high part is split exactly by an
-// FMA (Dekker's two-product), the low part's product is added to its error term before the
-// final rounding
-__device__ __forceinline__ float mul_pair(float z, float wh, float wl) {
-  const float p = z * wh;
-  const float e = fmaf(z, wh, -p);
-  return p + fmaf(z, wl, e);
-}
-
 // Hint: bring [p, p + bytes) into L2 (p and bytes multiples of 16), in pieces of at most 32 KB.
 __device__ __forceinline__ void prefetch_l2(const void* p, unsigned bytes) {
   const size_t ga = __cvta_generic_to_global(p);
@@ -93,23 +79,53 @@ __device__ __forceinline__ void prefetch_line_l2(const void* p) {
 }
 
 constexpr int kThreads = 256;
-template <typename T>
-constexpr int kEPT = (sizeof(T) == 4) ? 16 : 8;   // tile elements per thread (float: 16; double, dd: 8)
+static inline int ilog2(int v) { return wide_log2(v); }
+static inline int pow2_at_least(int v) { return (1 << ilog2(v)) < v ? 2 << ilog2(v) : 1 << ilog2(v); }
 
-static inline int tile_width(int n, int ept) {
-  int w = 1;
-  while (w < 64 && (2 * w) * n <= ept * kThreads) w *= 2;
-  return w;
+// Lines per block of the passes without a tuned shape: the widest block that still gives every SM
+// its share.  A block's time hardly depends on its width while its warps have issue slots to spare,
+// so a grid of few lines takes narrow blocks (a 96 x 96 double y pass: 4 blocks of 16 lines 23 us,
+// 25 of 2 lines 9 us; below 2 lines in double, 4 in float, the tables of a block outweigh its lines).
+static int spread(int lines, int least, long long total, int blocks_per_sm) {
+  const long long want = (long long)blocks_per_sm * sm_count();
+  while (lines > least && (total + lines - 1) / lines < want) lines /= 2;
+  return lines;
 }
-static inline int ilog2(int v) {
-  int l = 0;
-  while ((1 << (l + 1)) <= v) ++l;
-  return l;
+
+// y/z pass: 128-byte rows per tile (coalesced) where shared memory allows them
+static int axis_lines(int type, const FftPlan& pl, const WidePlan& wide, long long total) {
+  int w = type == 1 ? 16 : 8;
+  if (type == 2) {   // float pairs: 8 elements per thread at 256 threads
+    w = 1;
+    while (w < 64 && 2 * w * pl.n <= 8 * kThreads) w *= 2;
+    return spread(w, 1, total, 1);
+  }
+  while (w > 1 && shape_smem(0, type, pl, wide, w) > (type == 1 ? 72 : 100) * 1024) w /= 2;
+  return spread(w, type == 1 ? 4 : 2, total, 2);
 }
-static inline int lines_per_cta(int m, int ept) {
+
+// x pass: about 256 butterflies of the widest stage per block
+static int x_lines(int type, const FftPlan& pl, const WidePlan& wide, long long total) {
   int l = 1;
-  while (l < 64 && (2 * l) * m <= ept * kThreads / 2) l *= 2;
-  return l;
+  if (type == 2) {   // one radix-8 butterfly per thread
+    while (l < 64 && 2 * l * pow2_at_least((pl.n + 7) / 8) <= kThreads) l *= 2;
+    while (l > 1 && shape_smem(1, type, pl, wide, l) > 76 * 1024) l /= 2;
+    return spread(l, 1, total, 1);
+  }
+  int nb = 1;
+  for (int s = 0; s < wide.nst; ++s) nb = std::max(nb, wide.n / wide.rad[s]);
+  while (l < 64 && 2 * l * nb <= kThreads) l *= 2;
+  while (l > 1 && shape_smem(1, type, pl, wide, l) > (type == 1 ? 72 : 100) * 1024) l /= 2;
+  return spread(l, 1, total, 2);
+}
+
+size_t shape_smem(int kind, int type, const FftPlan& pl, const WidePlan& wide, int lines) {
+  const size_t n = (size_t)pl.n, w = (size_t)lines;
+  if (type != 2) {
+    const size_t el = type == 1 ? sizeof(float) : sizeof(double);
+    return kind == 0 ? wide_axis_smem(wide, lines, el) : wide_xpass_smem(wide, lines, el);
+  }
+  return sizeof(cpx<dd>) * (kind == 0 ? 2 * n + 2 * w * n : 5 * n + 2 + 2 * w * (n + 1));   // packed: two tables
 }
 
 // ---------------------------------------------------------------------------------------
@@ -120,7 +136,7 @@ static inline int lines_per_cta(int m, int ept) {
 // complex float pairs (vd_pdd.cuh), bit-identical to the unpacked engine; its twiddle table
 // holds two entries per twiddle.
 template <typename T, int S, bool CV, bool PK = false>
-__global__ void __launch_bounds__(kThreads, (std::is_same<T, double>::value ? 2 : (std::is_same<T, dd>::value ? 4 : 3))) k_axis(const AxisProg P, const GridDesc g,
+__global__ void __launch_bounds__(kThreads, 4) k_axis(const AxisProg P, const GridDesc g,
                                                    const cpx<T>* __restrict__ twg, int lw) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   if (P.done && *P.done) return;
@@ -133,8 +149,8 @@ __global__ void __launch_bounds__(kThreads, (std::is_same<T, double>::value ? 2 
   E* tw2 = tw + n;   // PK: the second table
   E* A = tw + (PK ? 2 : 1) * n;
   E* B = A + W * n;
-  const int tid = threadIdx.x;
-  for (int j = tid; j < n; j += kThreads) {
+  const int tid = threadIdx.x, nthr = blockDim.x;
+  for (int j = tid; j < n; j += nthr) {
     if constexpr (PK) p_tw_entry<S>(twg[pl.tw_off + j], &tw[j], &tw2[j]);
     else tw[j] = twg[pl.tw_off + j];
   }
@@ -156,7 +172,7 @@ __global__ void __launch_bounds__(kThreads, (std::is_same<T, double>::value ? 2 
   // this thread's line (column) and its first element / butterfly
   const int w = tid & (W - 1);
   const int ib = tid >> lw;
-  const int istep = kThreads >> lw;
+  const int istep = nthr >> lw;
   const int col = col0 + w;
   const bool colok = col < inner_n;
   const int g0 = o * outer_stride + col + ib * line_stride;   // offset of element ib
@@ -765,9 +781,9 @@ __global__ void __launch_bounds__(kRLines * N2, (N2 == 16 ? 3 : 6))
 // PK (float pairs, radices 2 / 4 / 8 only): the transforms and the (un)packing of the real
 // transform run on packed complex float pairs (vd_pdd.cuh), bit-identical to the unpacked
 // code, with packed twiddle tables for both directions and the packing twiddles W_{n0}^k.
-template <typename T, bool CV, bool PK = false, int MINB = (std::is_same<T, dd>::value ? 3 : 1)>
+template <typename T, bool CV, bool PK = false, int MINB = 3>
 __global__ void __launch_bounds__(kThreads, MINB) k_xpass(const XProg P, const GridDesc g,
-                                                    const cpx<T>* __restrict__ twg, int llpc) {
+                                                    const cpx<T>* __restrict__ twg, int llpc, int ltpl) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   if (P.done && *P.done) return;
   const int m = g.n0 / 2;
@@ -784,8 +800,8 @@ __global__ void __launch_bounds__(kThreads, MINB) k_xpass(const XProg P, const G
   E* pkx = twx + 3 * m;
   E* A = PK ? pkx + 2 * (m + 1) : reinterpret_cast<E*>(pk + (m + 2));
   E* B = A + LPC * ls;
-  const int tid = threadIdx.x;
-  for (int j = tid; j < m; j += kThreads) {
+  const int tid = threadIdx.x, nthr = blockDim.x;
+  for (int j = tid; j < m; j += nthr) {
     if constexpr (PK) {
       const cpx<T> w = twg[g.px.tw_off + j];
       p_tw_entry<-1>(w, &twx[j], &twx[m + j]);
@@ -795,7 +811,7 @@ __global__ void __launch_bounds__(kThreads, MINB) k_xpass(const XProg P, const G
       twm[j] = twg[g.px.tw_off + j];
     }
   }
-  for (int j = tid; j <= m; j += kThreads) {
+  for (int j = tid; j <= m; j += nthr) {
     if constexpr (PK) p_tw_entry<-1>(twg[g.pk_off + j], &pkx[j], &pkx[m + 1 + j]);
     else pk[j] = twg[g.pk_off + j];
   }
@@ -804,8 +820,7 @@ __global__ void __launch_bounds__(kThreads, MINB) k_xpass(const XProg P, const G
   const long long line0 = (long long)blockIdx.x * LPC;
   const int nl = (int)min((long long)LPC, nlines - line0);
   // this thread's line and its position in the line
-  const int ltpl = 8 - llpc;   // log2(threads per line), kThreads = 256
-  const int TPL = 1 << ltpl;
+  const int TPL = 1 << ltpl;   // threads per line
   const int line = tid >> ltpl;
   const int t0 = tid & (TPL - 1);
   const bool lok = line < nl;
@@ -910,17 +925,6 @@ __global__ void __launch_bounds__(kThreads, MINB) k_xpass(const XProg P, const G
 #pragma unroll 4
           for (int j = t0; j < m; j += TPL) res[lofs + j] = p_scal(res[lofs + j], pdd_of(wf[j]));
           done_pair = true;
-        } else if constexpr (std::is_same<T, float>::value) {
-          if (P.wf_dd) {
-            const float4* __restrict__ wf4 = reinterpret_cast<const float4*>(P.wfield) + (line0 + line) * m;
-#pragma unroll 4
-            for (int j = t0; j < m; j += TPL) {
-              const cpx<T> z = res[lofs + j];
-              const float4 w = wf4[j];
-              res[lofs + j] = mk<T>(mul_pair(z.x, w.x, w.y), mul_pair(z.y, w.z, w.w));
-            }
-            done_pair = true;
-          }
         }
         if constexpr (!PK) {
           if (!done_pair) {
@@ -1435,13 +1439,19 @@ void tune_set(int kind, int type, int n, int axis, int dir, int choice) {
   else g_tune[tune_key(kind, type, n, axis, dir)] = choice;
 }
 
-int default_shape(int kind, int type, int n, int axis) {
-  const int ept = (type == 1) ? 16 : 8;
-  // float z passes of length 128/256: the TMA-staged kernel (its gain is largest on the
-  // multi-transform programs of the operators, which the tuner's single transform understates)
-  if (kind == 0 && type == 1 && axis == 2 && (n == 128 || n == 256)) return kChoiceStaged;
-  if (kind == 0) return (type == 1 && (n == 128 || n == 256)) ? 0 : tile_width(n, ept);
-  return (type == 1 && (n == 64 || n == 128 || n == 256)) ? 0 : lines_per_cta(n, ept);
+int default_shape(int kind, int type, const FftPlan& pl, const WidePlan& wide, int axis, long long lines) {
+  const int n = pl.n;
+  // The register kernels (float) where their blocks fill the GPU twice: 16 lines per block in y and
+  // z, 256 threads of n / 8 or n / 16 elements in x.  z passes: with TMA-staged input (its gain is
+  // largest on the multi-transform programs of the operators, which the tuner's single transform
+  // understates).
+  if (kind == 0) {
+    if (type == 1 && (n == 128 || n == 256) && lines >= 32LL * sm_count()) return axis == 2 ? kChoiceStaged : 0;
+    return axis_lines(type, pl, wide, lines);
+  }
+  const int reg_lines = n == 256 ? 16 : 32;
+  if (type == 1 && (n == 64 || n == 128 || n == 256) && lines >= 2LL * reg_lines * sm_count()) return 0;
+  return x_lines(type, pl, wide, lines);
 }
 
 int tune_table(int* out, int max) {
@@ -1481,7 +1491,7 @@ void tune_save() {
 // Opt a kernel into more than 48 KB of dynamic shared memory.  The limit only grows, under a
 // lock: launches from several host threads (server slots) must never lower it below the
 // size another thread is about to launch with.
-static void ensure_smem(const void* func, size_t smem) {
+void ensure_smem(const void* func, size_t smem) {
   if (smem <= 48 * 1024) return;
   static std::mutex mu;
   static std::map<const void*, size_t> set;
@@ -1493,25 +1503,14 @@ static void ensure_smem(const void* func, size_t smem) {
   }
 }
 
-template <typename T>
-size_t axis_smem_bytes(const GridDesc& g, int axis) {
-  const int n = (axis == 2) ? g.pz.n : g.py.n;
-  const int W = tile_width(n, kEPT<T>);
-  return sizeof(cpx<T>) * (size_t)(n + 2 * W * n);
-}
-
-template <typename T>
-size_t xpass_smem_bytes(const GridDesc& g) {
-  const int m = g.n0 / 2;
-  const int L = lines_per_cta(m, kEPT<T>);
-  return sizeof(cpx<T>) * (size_t)(m + (m + 2) + 2 * L * (m + 1));
-}
-
 template <typename T, int S, bool CV, bool PK>
 static void launch_k_axis(const AxisProg& P, const GridDesc& g, const cpx<T>* tw, int W, long long blocks,
                           size_t smem, cudaStream_t st) {
+  // 8 elements per thread, whole lines' worth of warps
+  const int n = (P.axis == 2) ? g.pz.n : g.py.n;
+  const int threads = std::min(kThreads, std::max(32, W * std::max((n + 7) / 8, (31 + W) / W)));
   ensure_smem(reinterpret_cast<const void*>(k_axis<T, S, CV, PK>), smem);
-  k_axis<T, S, CV, PK><<<(unsigned)blocks, kThreads, smem, st>>>(P, g, tw, ilog2(W));
+  k_axis<T, S, CV, PK><<<(unsigned)blocks, threads, smem, st>>>(P, g, tw, ilog2(W));
 }
 
 template <typename T, int S, int N1, int N2>
@@ -1573,7 +1572,7 @@ static bool encode_tiles(CUtensorMap* m, const void* base, const GridDesc& g, in
              CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-static int sm_count() {
+int sm_count() {
   static int cached[64] = {0};
   int dev = 0;
   cudaGetDevice(&dev);
@@ -1626,11 +1625,6 @@ void launch_axis(const AxisProg& P0, int dir, const GridDesc& g, const void* tw,
   AxisProg P = P0;
   for (int t = 0; t < P.nxf; ++t) split_scale(P.xf[t].scale, &P.xf[t].scale_hi, &P.xf[t].scale_lo);
   const int n = (P.axis == 2) ? g.pz.n : g.py.n;
-  int choice = tune_get(0, type_code<T>(), n, P.axis, dir);
-  const bool reg_ok = std::is_same<T, float>::value && (n == 256 || n == 128);
-  if (choice < 0) choice = default_shape(0, type_code<T>(), n, P.axis);
-  if (choice == kChoiceStaged && !(reg_ok && tma_program_ok(P, g))) choice = 0;   // not applicable: register kernel
-  const int W = (choice > 0 && choice <= 64) ? choice : tile_width(n, kEPT<T>);
   long long inner_n, outer_n;
   if (P.axis == 2) {
     inner_n = (long long)g.n1 * g.h0;
@@ -1639,9 +1633,13 @@ void launch_axis(const AxisProg& P0, int dir, const GridDesc& g, const void* tw,
     inner_n = g.h0;
     outer_n = g.n2;
   }
-  const long long blocks = outer_n * ((inner_n + W - 1) / W);
-  const size_t smem = sizeof(cpx<T>) * (size_t)(n + 2 * W * n);
-  const cpx<T>* twp = reinterpret_cast<const cpx<T>*>(tw);
+  int choice = tune_get(0, type_code<T>(), n, P.axis, dir);
+  const bool reg_ok = std::is_same<T, float>::value && (n == 256 || n == 128);
+  const FftPlan& pl = P.axis == 2 ? g.pz : g.py;
+  const WidePlan& wide = (P.axis == 2 ? g.wz : g.wy)[wide_class(sizeof(T), g.ncplx)];
+  if (choice < 0) choice = default_shape(0, type_code<T>(), pl, wide, P.axis, inner_n * outer_n);
+  if (choice == kChoiceStaged && !(reg_ok && tma_program_ok(P, g))) choice = 0;   // not applicable: register kernel
+  const int W = (choice > 0 && choice <= 64) ? choice : axis_lines(type_code<T>(), pl, wide, inner_n * outer_n);
   // algorithmic traffic: every distinct input and output field once, the symbol array once
   unsigned inmask = 0, outmask = 0;
   int nfft = 0;
@@ -1674,18 +1672,21 @@ void launch_axis(const AxisProg& P0, int dir, const GridDesc& g, const void* tw,
     // register-resident four-step kernel for the common lengths (unless tuned otherwise)
     if (reg_ok && choice <= 0) {
       if (n == 256) {
-        if (dir < 0) launch_axis_r<T, -1, 16, 16>(P, g, twp, inner_n, outer_n, st);
-        else launch_axis_r<T, +1, 16, 16>(P, g, twp, inner_n, outer_n, st);
+        if (dir < 0) launch_axis_r<T, -1, 16, 16>(P, g, twf, inner_n, outer_n, st);
+        else launch_axis_r<T, +1, 16, 16>(P, g, twf, inner_n, outer_n, st);
       } else {
-        if (dir < 0) launch_axis_r<T, -1, 16, 8>(P, g, twp, inner_n, outer_n, st);
-        else launch_axis_r<T, +1, 16, 8>(P, g, twp, inner_n, outer_n, st);
+        if (dir < 0) launch_axis_r<T, -1, 16, 8>(P, g, twf, inner_n, outer_n, st);
+        else launch_axis_r<T, +1, 16, 8>(P, g, twf, inner_n, outer_n, st);
       }
       return;
     }
   }
-  const bool cv = (P.conv_in | P.conv_out) != 0;
   if constexpr (std::is_same<T, dd>::value) {
-    if (choice != kChoiceUnpacked && p_plan_ok(P.axis == 2 ? g.pz : g.py, kThreads / W)) {
+    const bool cv = (P.conv_in | P.conv_out) != 0;
+    const cpx<T>* twp = reinterpret_cast<const cpx<T>*>(tw);
+    const long long blocks = outer_n * ((inner_n + W - 1) / W);
+    const size_t smem = sizeof(cpx<T>) * (size_t)(n + 2 * W * n);
+    if (choice != kChoiceUnpacked && p_plan_ok(pl, kThreads / W)) {
       const size_t psmem = smem + sizeof(pdd) * (size_t)n;   // the second twiddle table
       if (dir < 0 && cv) launch_k_axis<T, -1, true, true>(P, g, twp, W, blocks, psmem, st);
       else if (dir < 0) launch_k_axis<T, -1, false, true>(P, g, twp, W, blocks, psmem, st);
@@ -1693,18 +1694,22 @@ void launch_axis(const AxisProg& P0, int dir, const GridDesc& g, const void* tw,
       else launch_k_axis<T, +1, false, true>(P, g, twp, W, blocks, psmem, st);
       return;
     }
+    if (dir < 0 && cv) launch_k_axis<T, -1, true, false>(P, g, twp, W, blocks, smem, st);
+    else if (dir < 0) launch_k_axis<T, -1, false, false>(P, g, twp, W, blocks, smem, st);
+    else if (cv) launch_k_axis<T, +1, true, false>(P, g, twp, W, blocks, smem, st);
+    else launch_k_axis<T, +1, false, false>(P, g, twp, W, blocks, smem, st);
+  } else {
+    wide_axis<T>(P, dir, g, tw, W, st);
   }
-  if (dir < 0 && cv) launch_k_axis<T, -1, true, false>(P, g, twp, W, blocks, smem, st);
-  else if (dir < 0) launch_k_axis<T, -1, false, false>(P, g, twp, W, blocks, smem, st);
-  else if (cv) launch_k_axis<T, +1, true, false>(P, g, twp, W, blocks, smem, st);
-  else launch_k_axis<T, +1, false, false>(P, g, twp, W, blocks, smem, st);
 }
 
-template <typename T, bool CV, bool PK, int MINB = (std::is_same<T, dd>::value ? 3 : 1)>
+template <typename T, bool CV, bool PK, int MINB = 3>
 static void launch_k_xpass(const XProg& P, const GridDesc& g, const cpx<T>* tw, int L, long long blocks, size_t smem,
                            cudaStream_t st) {
   ensure_smem(reinterpret_cast<const void*>(k_xpass<T, CV, PK, MINB>), smem);
-  k_xpass<T, CV, PK, MINB><<<(unsigned)blocks, kThreads, smem, st>>>(P, g, tw, ilog2(L));
+  // threads per line: a power of two, one radix-8 butterfly each, at least a warp per block
+  const int tpl = std::min(kThreads / L, std::max(pow2_at_least((g.px.n + 7) / 8), pow2_at_least((31 + L) / L)));
+  k_xpass<T, CV, PK, MINB><<<(unsigned)blocks, L * tpl, smem, st>>>(P, g, tw, ilog2(L), ilog2(tpl));
 }
 
 template <typename T>
@@ -1732,11 +1737,9 @@ void launch_xpass(const XProg& P0, const GridDesc& g, const void* tw, cudaStream
   split_scale(P.aux_scale, &P.aux_scale_hi, &P.aux_scale_lo);
   const int m = g.n0 / 2;
   int choice = tune_get(1, type_code<T>(), m, 0, P.mode);
-  const int L = (choice > 0 && choice <= 64) ? choice : lines_per_cta(m, kEPT<T>);
   const long long nlines = (long long)g.n1 * g.n2;
-  const long long blocks = (nlines + L - 1) / L;
-  const size_t smem = sizeof(cpx<T>) * (size_t)(m + (m + 2) + 2 * L * (m + 1));
-  const bool cv = (P.conv_in | P.conv_out | (P.aux_out ? P.aux_conv : 0)) != 0;
+  if (choice < 0) choice = default_shape(1, type_code<T>(), g.px, g.wx[wide_class(sizeof(T), g.ncplx)], 0, nlines);
+  const int L = (choice > 0 && choice <= 64) ? choice : x_lines(type_code<T>(), g.px, g.wx[wide_class(sizeof(T), g.ncplx)], nlines);
   const double fc = (double)g.ncplx * sizeof(cpx<T>), fr = (double)g.nreal * sizeof(T);
   double bytes = 0, flops = 0;
   const double real_fft = (double)g.nreal * 2.5 * std::log2((double)g.n0);   // one real transform of every line
@@ -1781,8 +1784,11 @@ void launch_xpass(const XProg& P0, const GridDesc& g, const void* tw, cudaStream
       return;
     }
   }
-  const cpx<T>* twp = reinterpret_cast<const cpx<T>*>(tw);
   if constexpr (std::is_same<T, dd>::value) {
+    const cpx<T>* twp = reinterpret_cast<const cpx<T>*>(tw);
+    const bool cv = (P.conv_in | P.conv_out | (P.aux_out ? P.aux_conv : 0)) != 0;
+    const long long blocks = (nlines + L - 1) / L;
+    const size_t smem = sizeof(cpx<T>) * (size_t)(m + (m + 2) + 2 * L * (m + 1));
     if (choice != kChoiceUnpacked && p_plan_ok(g.px, kThreads / L)) {
       // the packed twiddle tables: 3 m + 2 (m + 1) entries against 2 m + 2
       const size_t psmem = smem + sizeof(pdd) * (size_t)(3 * m);
@@ -1794,9 +1800,11 @@ void launch_xpass(const XProg& P0, const GridDesc& g, const void* tw, cudaStream
       else launch_k_xpass<T, false, true, 3>(P, g, twp, L, blocks, psmem, st);
       return;
     }
+    if (cv) launch_k_xpass<T, true, false>(P, g, twp, L, blocks, smem, st);
+    else launch_k_xpass<T, false, false>(P, g, twp, L, blocks, smem, st);
+  } else {
+    wide_xpass<T>(P, g, tw, L, st);
   }
-  if (cv) launch_k_xpass<T, true, false>(P, g, twp, L, blocks, smem, st);
-  else launch_k_xpass<T, false, false>(P, g, twp, L, blocks, smem, st);
 }
 
 template void launch_axis<dd>(const AxisProg&, int, const GridDesc&, const void*, cudaStream_t);
@@ -1805,11 +1813,5 @@ template void launch_axis<double>(const AxisProg&, int, const GridDesc&, const v
 template void launch_axis<float>(const AxisProg&, int, const GridDesc&, const void*, cudaStream_t);
 template void launch_xpass<double>(const XProg&, const GridDesc&, const void*, cudaStream_t);
 template void launch_xpass<float>(const XProg&, const GridDesc&, const void*, cudaStream_t);
-template size_t axis_smem_bytes<double>(const GridDesc&, int);
-template size_t axis_smem_bytes<dd>(const GridDesc&, int);
-template size_t xpass_smem_bytes<dd>(const GridDesc&);
-template size_t axis_smem_bytes<float>(const GridDesc&, int);
-template size_t xpass_smem_bytes<double>(const GridDesc&);
-template size_t xpass_smem_bytes<float>(const GridDesc&);
 
 }  // namespace vd

@@ -102,13 +102,53 @@ constexpr int kChoiceUnpacked = 256;
 int tune_get(int kind, int type, int n, int axis, int dir);
 void tune_set(int kind, int type, int n, int axis, int dir, int choice);
 int tune_table(int* out, int max);   // 6 ints per entry; returns the entry count
-int default_shape(int kind, int type, int n, int axis = 0);   // the built-in choice (kind 1: n = n0/2)
+// the built-in choice for a pass of `lines` lines in all (kind 1: n = n0/2)
+int default_shape(int kind, int type, const FftPlan& pl, const WidePlan& wide, int axis, long long lines);
 void tune_save();                    // write the table to $VD_TUNE_FILE (if set)
 
-// shared memory footprint (bytes) of the pass kernels, for the attribute setup
+// opt a kernel into more than 48 KB of dynamic shared memory (once per size)
+void ensure_smem(const void* func, size_t smem);
+int sm_count();
+
+// the float and double passes of any length (vd_wide.cuh): W / L lines per block, powers of two
 template <typename T>
-size_t axis_smem_bytes(const GridDesc& g, int axis);
+void wide_axis(const AxisProg& P, int dir, const GridDesc& g, const void* tw, int W, cudaStream_t st);
 template <typename T>
-size_t xpass_smem_bytes(const GridDesc& g);
+void wide_xpass(const XProg& P, const GridDesc& g, const void* tw, int L, cudaStream_t st);
+// the plans of length n in every radix class, their tables at tw_off
+bool make_wide_plans(int n, int tw_off, WidePlan p[kWideClasses]);
+// The radix class of a pass over a field of ncplx points.  Wide radices make fewer trips through
+// shared memory, narrow ones more and shorter threads.  Double: a warp issues one FP64 instruction
+// per 64 cycles however independent, four warps per SM saturate the pipe, so a small field wants
+// many threads of few operations (96 x 96 double apply: 8 radix-5-and-below stages 78 us, radix 8
+// 96, radix 16 127; 320 x 320: 127, 135; 512 x 1024: 312, 302; 80^3: 411, 393, 16: 504).  Float: latency
+// until the field is large (512 x 1024 forward: radix 8 14.4 us, 16 18.6; 320 x 256 x 160: 145, 108).
+inline int wide_class(size_t el, long long ncplx) {
+  if (el == sizeof(float)) return ncplx >= (1 << 20) ? 2 : 1;
+  return ncplx >= (1 << 21) ? 2 : (ncplx >= (1 << 17) ? 1 : 0);
+}
+inline int wide_log2(int v) {
+  int l = 0;
+  while ((1 << (l + 1)) <= v) ++l;
+  return l;
+}
+// Stockham buffers pad one element in 2^shift, so that the stores of a first stage (a radix apart)
+// spread over the banks: 17 elements apart for radix 16, 9 for 8
+inline int wide_pad_shift(const WidePlan& pl) {
+  int r = 0;
+  for (int s = 0; s < pl.nst; ++s) r = r > pl.rad[s] ? r : pl.rad[s];
+  return r > 10 ? 4 : 3;
+}
+inline int wide_line_stride(const WidePlan& pl) { return (pl.n + (pl.n >> wide_pad_shift(pl)) + 1) | 1; }
+// shared memory of a block of W y/z lines or L x lines; el: bytes of a real
+inline size_t wide_axis_smem(const WidePlan& pl, int W, size_t el) {
+  const size_t rows = (size_t)pl.n + (size_t)(pl.n >> wide_pad_shift(pl));
+  return 2 * el * ((size_t)pl.n + (pl.nst > 2 ? 2 : 1) * (size_t)W * rows) + el * (size_t)pl.n;
+}
+inline size_t wide_xpass_smem(const WidePlan& pl, int L, size_t el) {
+  return 2 * el * ((size_t)pl.n + pl.n / 2 + 1 + 2 * (size_t)L * wide_line_stride(pl)) + el * (size_t)(pl.n + 1);
+}
+// dynamic shared memory a launch of `lines` lines per block takes in type code `type`
+size_t shape_smem(int kind, int type, const FftPlan& pl, const WidePlan& wide, int lines);
 
 }  // namespace vd

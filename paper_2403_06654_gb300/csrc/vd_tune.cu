@@ -76,6 +76,7 @@ template <typename T>
 vd_status tune_type(const vd_grid* G, const void* tw, void* a, void* b, cudaStream_t st, Timer& tm) {
   const GridDesc& g = G->g;
   const int type = tcode<T>();
+  const int cls = wide_class(sizeof(T), g.ncplx);
   // y and z passes
   for (int axis = 1; axis <= 2; ++axis) {
     if (axis == 1 && g.ndim < 2) continue;
@@ -87,7 +88,7 @@ vd_status tune_type(const vd_grid* G, const void* tw, void* a, void* b, cudaStre
     if (reg) cand.push_back(0);
     if (reg) cand.push_back(kChoiceStaged);
     for (int W = 1; W <= 64; W *= 2) {
-      if (sizeof(cpx<T>) * (size_t)(n + 2 * W * n) > kSmemCap) break;
+      if (shape_smem(0, type, axis == 2 ? g.pz : g.py, (axis == 2 ? g.wz : g.wy)[cls], W) > kSmemCap) break;
       if (W > 1 && W > 2 * inner) break;
       cand.push_back(W);
     }
@@ -114,7 +115,8 @@ vd_status tune_type(const vd_grid* G, const void* tw, void* a, void* b, cudaStre
         }
       }
       (void)reg;
-      tune_set(0, type, n, axis, dir, best >= 0 ? best : default_shape(0, type, n, axis));
+      tune_set(0, type, n, axis, dir, best >= 0 ? best : default_shape(0, type, axis == 2 ? g.pz : g.py, (axis == 2 ? g.wz : g.wy)[cls], axis,
+                                                                        inner * (axis == 2 ? 1 : g.n2)));
     }
   }
   // x pass: forward (mode 1), inverse (mode 2), fused (mode 0 with a weight field)
@@ -123,7 +125,7 @@ vd_status tune_type(const vd_grid* G, const void* tw, void* a, void* b, cudaStre
   std::vector<int> cand;
   if (type == 1 && (m == 64 || m == 128 || m == 256)) cand.push_back(0);
   for (int L = 1; L <= 64; L *= 2) {
-    if (sizeof(cpx<T>) * (size_t)(m + (m + 2) + 2 * L * (m + 1)) > kSmemCap) break;
+    if (shape_smem(1, type, g.px, g.wx[cls], L) > kSmemCap) break;
     if (L > 1 && L > nlines) break;
     cand.push_back(L);
   }
@@ -152,7 +154,7 @@ vd_status tune_type(const vd_grid* G, const void* tw, void* a, void* b, cudaStre
         best = c;
       }
     }
-    tune_set(1, type, m, 0, mode, best >= 0 ? best : default_shape(1, type, m));
+    tune_set(1, type, m, 0, mode, best >= 0 ? best : default_shape(1, type, g.px, g.wx[cls], 0, nlines));
   }
   return VD_OK;
 }
