@@ -1,5 +1,6 @@
 // C ABI of the library: grids, density data, operator/preconditioner application and
 // the preconditioned solves (double and mixed precision).
+#include "vd_launch.cuh"
 #include "vd_krylov.cuh"
 #include "vd_dd.cuh"
 #include "vd_internal.h"
@@ -295,6 +296,7 @@ __global__ void k_density_prep(long long n, const double* __restrict__ rho, doub
                                double* __restrict__ rinv_s, float* __restrict__ rinv_f, dd* __restrict__ rinv_dd,
                                double invN,
                                double* __restrict__ stats /* [min, max, bad] via block partials */) {
+  pdl_wait();
   __shared__ double smin[256], smax[256], sbad[256];
   double mn = 1e308, mx = -1e308, bd = 0.0;
   for (long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x; e < n; e += (long long)gridDim.x * blockDim.x) {
@@ -380,6 +382,7 @@ static DensLayout dens_layout(const vd_grid* G, vd_op op, void* base, size_t* by
 // w = rho^-1/2 and per-block partial sums of w^2 (fixed grid: deterministic)
 __global__ void k_krho_w(long long n, const double* __restrict__ rho, double* __restrict__ w,
                          double* __restrict__ part) {
+  pdl_wait();
   __shared__ double sm[256];
   double s = 0.0;
   for (long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x; e < n; e += (long long)gridDim.x * blockDim.x) {
@@ -399,6 +402,7 @@ __global__ void k_krho_w(long long n, const double* __restrict__ rho, double* __
 // c = -Lap(w)/w; stored as c/N in double, float and float-pair (lapw may alias cs)
 __global__ void k_krho_coef(long long n, const double* __restrict__ w, const double* lapw, double invN, double* cs,
                             float* __restrict__ cf, dd* __restrict__ cdd) {
+  pdl_wait();
   for (long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x; e < n; e += (long long)gridDim.x * blockDim.x) {
     const double c = -lapw[e] / w[e] * invN;
     cs[e] = c;
@@ -428,7 +432,7 @@ vd_status vd_density_set(vd_grid* G, vd_op op, const double* rho, void* ws, size
   if (ws_bytes < need) return fail(VD_ERR_OOM, "density workspace too small");
   const GridDesc& g = G->g;
   const int blocks = (int)std::min<long long>(1024, (g.nreal + 255) / 256);
-  { k_density_prep<<<blocks, 256, 0, st>>>(g.nreal, rho, L.rho, L.rinv_s, L.rinv_f, L.rinv_dd, 1.0 / (double)g.nreal,
+  { pdl_launch(k_density_prep, blocks, 256, 0, st, g.nreal, rho, L.rho, L.rinv_s, L.rinv_f, L.rinv_dd, 1.0 / (double)g.nreal,
                                         L.stats); count_launch(); }
   VD_CUDA(cudaGetLastError());
   std::vector<double> stats(3 * blocks);
@@ -482,7 +486,7 @@ vd_status vd_density_set(vd_grid* G, vd_op op, const double* rho, void* ws, size
   G->kw_hat = nullptr;
   if (op == VD_OP_KRHO) {
     const size_t nc = (size_t)g.ncplx;
-    { k_krho_w<<<blocks, 256, 0, st>>>(g.nreal, rho, L.kw, L.stats); count_launch(); }
+    { pdl_launch(k_krho_w, blocks, 256, 0, st, g.nreal, rho, L.kw, L.stats); count_launch(); }
     std::vector<double> part(blocks);
     VD_CUDA(cudaMemcpyAsync(part.data(), L.stats, part.size() * 8, cudaMemcpyDeviceToHost, st));
     VD_CUDA(cudaStreamSynchronize(st));
@@ -497,7 +501,7 @@ vd_status vd_density_set(vd_grid* G, vd_op op, const double* rho, void* ws, size
     m.sym = 1;
     m.symarr = sym;
     inv_transform<double>(G, L.kw_hat, m, L.kc_s, tmp, st);
-    { k_krho_coef<<<blocks, 256, 0, st>>>(g.nreal, L.kw, L.kc_s, 1.0 / (double)g.nreal, L.kc_s, L.kc_f, L.kc_dd);
+    { pdl_launch(k_krho_coef, blocks, 256, 0, st, g.nreal, L.kw, L.kc_s, 1.0 / (double)g.nreal, L.kc_s, L.kc_f, L.kc_dd);
       count_launch(); }
     // unit Parseval norm: sum over the half spectrum with weights = N sum_x w^2
     spec_copy_scale<double>((long long)nc, L.kw_hat, 1.0 / std::sqrt((double)g.nreal * ww), L.kw_hat, st);

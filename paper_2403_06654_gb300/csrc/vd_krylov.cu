@@ -8,6 +8,7 @@
 // behind: it waits for the flag of batch k-1 with batch k already queued.  Kernels of an
 // iteration return at once when the flag is set, so iterations enqueued ahead cost a launch
 // each and change nothing.
+#include "vd_launch.cuh"
 #include "vd_krylov.cuh"
 #include "vd_dd.cuh"
 #include "vd_prof.h"
@@ -430,6 +431,7 @@ template <typename T>
 __global__ void __launch_bounds__(kRedThreads) k_cg_init(Ix ix, const cpx<T>* __restrict__ b,
                                                          const cpx<T>* __restrict__ r, cpx<T>* __restrict__ p,
                                                          const T* __restrict__ sym, RedArgs ra) {
+  pdl_wait();
   Acc<T> a0, a1, a2;
   IX_LOOP(ix) {
     const T w = pweight<T>(kx, ix.h0);
@@ -452,6 +454,7 @@ template <typename T, int NV>
 __global__ void __launch_bounds__(kRedThreads) k_dot(Ix ix, const cpx<T>* __restrict__ u,
                                                      const cpx<T>* __restrict__ v, int epi, RedArgs ra,
                                                      const int* done) {
+  pdl_wait();
   if (*done) return;
   Acc<T> a0, a1;
   IX_LOOP(ix) {
@@ -473,6 +476,7 @@ __global__ void __launch_bounds__(kRedThreads) k_cg_update(Ix ix, cpx<T>* __rest
                                                            const cpx<T>* __restrict__ p, cpx<T>* __restrict__ r,
                                                            const cpx<T>* __restrict__ q, const T* __restrict__ sym,
                                                            RedArgs ra) {
+  pdl_wait();
   if (ra.ks->done) return;
   const T al = (T)ra.ks->alpha;
   Acc<T> a0, a1;
@@ -498,6 +502,7 @@ __global__ void __launch_bounds__(kRedThreads) k_cg_update(Ix ix, cpx<T>* __rest
 template <typename T>
 __global__ void k_cg_p(Ix ix, cpx<T>* __restrict__ p, const cpx<T>* __restrict__ r, const T* __restrict__ sym,
                        const KState* ks) {
+  pdl_wait();
   if (ks->done) return;
   const T be = (T)ks->beta;
   IX_LOOP(ix) {
@@ -512,6 +517,7 @@ template <typename T, int NV>
 __global__ void __launch_bounds__(kRedThreads) k_norms(Ix ix, const cpx<T>* __restrict__ b,
                                                        const cpx<T>* __restrict__ r, int epi, RedArgs ra,
                                                        const int* done) {
+  pdl_wait();
   if (done && *done) return;
   Acc<T> a0, a1;
   IX_LOOP(ix) {
@@ -535,6 +541,7 @@ __global__ void __launch_bounds__(kRedThreads) k_norms(Ix ix, const cpx<T>* __re
 template <typename T>
 __global__ void __launch_bounds__(kRedThreads) k_pdot(Ix ix, const cpx<T>* __restrict__ a,
                                                       const cpx<T>* __restrict__ b, RedArgs ra) {
+  pdl_wait();
   Acc<T> a0;
   IX_LOOP(ix) {
     const cpx<T> u = a[e], v = b[e];
@@ -550,6 +557,7 @@ template <typename T>
 __global__ void __launch_bounds__(kRedThreads) k_sub_norm(Ix ix, const cpx<T>* __restrict__ b,
                                                           const cpx<T>* __restrict__ q, cpx<T>* __restrict__ r,
                                                           RedArgs ra) {
+  pdl_wait();
   Acc<T> a1;
   IX_LOOP(ix) {
     const cpx<T> rv = b[e] - q[e];
@@ -566,6 +574,7 @@ template <typename T>
 __global__ void __launch_bounds__(kRedThreads) k_rmr_update(Ix ix, cpx<T>* __restrict__ x, cpx<T>* __restrict__ r,
                                                             const cpx<T>* __restrict__ wv, const T* __restrict__ sym,
                                                             RedArgs ra) {
+  pdl_wait();
   if (ra.ks->done) return;
   const T al = (T)ra.ks->alpha;
   Acc<T> a0;
@@ -590,6 +599,7 @@ __global__ void __launch_bounds__(kRedThreads) k_rmr_update(Ix ix, cpx<T>* __res
 template <typename T>
 __global__ void k_gm_scale(Ix ix, cpx<T>* __restrict__ dst, const cpx<T>* __restrict__ src, const KState* ks,
                            int first) {
+  pdl_wait();
   if (ks->cycle_done) return;
   const T s = (T)(1.0 / (first ? ks->beta0 : ks->ww));
   for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < ix.len; e += gridDim.x * blockDim.x)
@@ -605,6 +615,7 @@ template <typename T, int NB>
 __global__ void __launch_bounds__(kRedThreads) k_gm_mdot(Ix ix, const cpx<T>* __restrict__ w,
                                                          const cpx<T>* __restrict__ V, int off, int nv, int epi, int j,
                                                          RedArgs ra) {
+  pdl_wait();
   if (ra.ks->cycle_done) return;
   Acc<T> a[NB];
   IX_LOOP(ix) {
@@ -624,6 +635,7 @@ __global__ void __launch_bounds__(kRedThreads) k_gm_mdot(Ix ix, const cpx<T>* __
 template <typename T, int NB>
 __global__ void __launch_bounds__(kRedThreads) k_gm_step(Ix ix, cpx<T>* __restrict__ w, const cpx<T>* __restrict__ V,
                                                          int nv, RedArgs ra) {
+  pdl_wait();
   if (ra.ks->cycle_done) return;
   __shared__ T hs[NB];
   for (int i = threadIdx.x; i < NB; i += blockDim.x) hs[i] = (i < nv) ? (T)ra.ks->h1[i] : T(0);
@@ -656,6 +668,7 @@ template <typename T>
 __global__ void __launch_bounds__(kRedThreads) k_gm_maxpy(Ix ix, cpx<T>* __restrict__ w,
                                                           const cpx<T>* __restrict__ V, int j, int which, int with_norm,
                                                           RedArgs ra) {
+  pdl_wait();
   if (ra.ks->cycle_done) return;
   __shared__ T hs[kMaxRestart + 1];
   const double* h = which ? ra.ks->h2 : ra.ks->h1;
@@ -705,18 +718,18 @@ static void gm_orthogonalise(const SpecSystem& sys, cpx<T>* w, const cpx<T>* V, 
   auto mdot = [&](int off, int nv, int epi) {
     ProfScope ps_(cls, st, (nv + 1) * el, 0.0);
 #define GM_MDOT(NB) \
-  k_gm_mdot<T, NB><<<blocks(NB), kRedThreads, 0, st>>>(index(blocks(NB)), w, V, off, nv, epi, j, ra)
+  pdl_launch(k_gm_mdot<T, NB>, blocks(NB), kRedThreads, 0, st, index(blocks(NB)), w, V, off, nv, epi, j, ra)
     GM_BY_COUNT(nv, GM_MDOT);
 #undef GM_MDOT
   };
   auto maxpy = [&](int which) {
     ProfScope ps_(cls, st, (n + 2) * el, 0.0);
-    k_gm_maxpy<T><<<blocks(1), kRedThreads, 0, st>>>(index(blocks(1)), w, V, j, which, which, ra);
+    pdl_launch(k_gm_maxpy<T>, blocks(1), kRedThreads, 0, st, index(blocks(1)), w, V, j, which, which, ra);
   };
   for (int off = 0; off < n; off += 32) mdot(off, std::min(32, n - off), EPI_GM_H1);
   if (n <= 32) {
     ProfScope ps_(cls, st, (n + 2) * el, 0.0);
-#define GM_STEP(NB) k_gm_step<T, NB><<<blocks(NB), kRedThreads, 0, st>>>(index(blocks(NB)), w, V, n, ra)
+#define GM_STEP(NB) pdl_launch(k_gm_step<T, NB>, blocks(NB), kRedThreads, 0, st, index(blocks(NB)), w, V, n, ra)
     GM_BY_COUNT(n, GM_STEP);
 #undef GM_STEP
   } else {
@@ -730,6 +743,7 @@ static void gm_orthogonalise(const SpecSystem& sys, cpx<T>* w, const cpx<T>* V, 
 // GMRES: back substitution H(0:k,0:k) y = g: one warp, column by column, the triangle in shared
 // memory (one thread reading it from global memory took 35 us at k = 30)
 __global__ void __launch_bounds__(32) k_gm_solve(KState* ks) {
+  pdl_wait();
   if (ks->done) return;
   __shared__ double tri[kMaxRestart * kMaxRestart], g[kMaxRestart];
   const int k = ks->k, m = ks->m, lane = threadIdx.x;
@@ -750,6 +764,7 @@ __global__ void __launch_bounds__(32) k_gm_solve(KState* ks) {
 template <typename T>
 __global__ void k_gm_update(Ix ix, cpx<T>* __restrict__ x, const cpx<T>* __restrict__ V, const T* __restrict__ sym,
                             const KState* ks) {
+  pdl_wait();
   if (ks->done) return;
   __shared__ T ys[kMaxRestart];
   const int k = ks->k;
@@ -770,6 +785,7 @@ __global__ void k_gm_update(Ix ix, cpx<T>* __restrict__ x, const cpx<T>* __restr
 
 // GMRES end of cycle: converged inside the cycle -> finished
 __global__ void k_gm_close(KState* ks) {
+  pdl_wait();
   if (threadIdx.x != 0 || blockIdx.x != 0 || ks->done) return;
   if (ks->status == 0 || ks->status == VD_ERR_NONFINITE) ks->done = 1;
 }
@@ -780,6 +796,7 @@ __global__ void k_gm_close(KState* ks) {
 
 template <typename T>
 __global__ void k_copy_scale(long long len, const cpx<T>* __restrict__ x, double s, cpx<T>* __restrict__ y) {
+  pdl_wait();
   GRID_STRIDE(e, len) {
     const cpx<double> v = ld(x, e);
     y[e] = mk<T>((T)(v.x * s), (T)(v.y * s));
@@ -787,6 +804,7 @@ __global__ void k_copy_scale(long long len, const cpx<T>* __restrict__ x, double
 }
 template <typename T>
 __global__ void k_axpy(long long len, double a, const cpx<T>* __restrict__ x, cpx<T>* __restrict__ y) {
+  pdl_wait();
   GRID_STRIDE(e, len) {
     const cpx<double> v = ld(x, e), w = ld(y, e);
     y[e] = mk<T>((T)fma(a, v.x, w.x), (T)fma(a, v.y, w.y));
@@ -795,6 +813,7 @@ __global__ void k_axpy(long long len, double a, const cpx<T>* __restrict__ x, cp
 template <typename T>
 __global__ void k_sub(long long len, const cpx<T>* __restrict__ b, const cpx<T>* __restrict__ q,
                       cpx<T>* __restrict__ r, const int* done) {
+  pdl_wait();
   if (done && *done) return;
   GRID_STRIDE(e, len) { r[e] = b[e] - q[e]; }
 }
@@ -803,6 +822,7 @@ __global__ void k_sub(long long len, const cpx<T>* __restrict__ b, const cpx<T>*
 // host, or from the refinement state (o->scale, o->rnorm) when o is set
 __global__ void k_d2f_scaled(long long len, const cpx<double>* __restrict__ in, double s, const OState* o,
                              cpx<float>* __restrict__ out) {
+  pdl_wait();
   if (o) s = o->scale;
   GRID_STRIDE(e, len) {
     const cpx<double> v = in[e];
@@ -811,6 +831,7 @@ __global__ void k_d2f_scaled(long long len, const cpx<double>* __restrict__ in, 
 }
 __global__ void k_axpy_f2d(long long len, double a, const OState* o, const cpx<float>* __restrict__ xf,
                            cpx<double>* __restrict__ y) {
+  pdl_wait();
   if (o) a = o->rnorm;
   GRID_STRIDE(e, len) {
     const cpx<float> v = xf[e];
@@ -820,6 +841,7 @@ __global__ void k_axpy_f2d(long long len, double a, const OState* o, const cpx<f
 }
 template <typename T>
 __global__ void k_project(GridDesc g, int ncomp, cpx<T>* v, double* removed) {
+  pdl_wait();
   const int t = threadIdx.x;   // one thread per corner mode and component
   const int d = g.ndim;
   const int ncorner = 1 << d;
@@ -852,19 +874,19 @@ static inline int ew_blocks(long long len) {
 
 template <typename T>
 void spec_copy_scale(long long len, const void* x, double s, void* y, cudaStream_t st) {
-  { k_copy_scale<T><<<ew_blocks(len), 256, 0, st>>>(len, (const cpx<T>*)x, s, (cpx<T>*)y); count_launch(); }
+  { pdl_launch(k_copy_scale<T>, ew_blocks(len), 256, 0, st, len, (const cpx<T>*)x, s, (cpx<T>*)y); count_launch(); }
 }
 template <typename T>
 void spec_axpy(long long len, double a, const void* x, void* y, cudaStream_t st) {
-  { k_axpy<T><<<ew_blocks(len), 256, 0, st>>>(len, a, (const cpx<T>*)x, (cpx<T>*)y); count_launch(); }
+  { pdl_launch(k_axpy<T>, ew_blocks(len), 256, 0, st, len, a, (const cpx<T>*)x, (cpx<T>*)y); count_launch(); }
 }
 template <typename T>
 void spec_sub(long long len, const void* b, const void* q, void* r, cudaStream_t st) {
-  { ProfScope ps_(sizeof(T) == 4 ? PC_VEC32 : PC_VEC64, st, (double)3 * len * sizeof(cpx<T>), 0.0); k_sub<T><<<ew_blocks(len), 256, 0, st>>>(len, (const cpx<T>*)b, (const cpx<T>*)q, (cpx<T>*)r, nullptr); }
+  { ProfScope ps_(sizeof(T) == 4 ? PC_VEC32 : PC_VEC64, st, (double)3 * len * sizeof(cpx<T>), 0.0); pdl_launch(k_sub<T>, ew_blocks(len), 256, 0, st, len, (const cpx<T>*)b, (const cpx<T>*)q, (cpx<T>*)r, nullptr); }
 }
 template <typename T>
 void spec_project(const vd_grid* G, int ncomp, void* v, cudaStream_t st, double* removed) {
-  { k_project<T><<<1, 32, 0, st>>>(G->g, ncomp, (cpx<T>*)v, removed); count_launch(); }
+  { pdl_launch(k_project<T>, 1, 32, 0, st, G->g, ncomp, (cpx<T>*)v, removed); count_launch(); }
 }
 
 template <typename T>
@@ -872,7 +894,7 @@ double spec_norm2_host(const SpecSystem& sys, const void* v, const KWork& kw, cu
   RedArgs ra{kw.ks, kw.partials, kw.counter, kw.hist, 0.0};
   const int rb = red_blocks(sys.len);
   const Ix ix = mkix(sys.len, sys.h0, sys.G->g.ncplx, rb, kRedThreads);
-  { ProfScope ps_(sizeof(T) == 4 ? PC_VEC32 : PC_VEC64, st, (double)1 * sys.len * sizeof(cpx<T>), 0.0); k_norms<T, 1><<<rb, kRedThreads, 0, st>>>(ix, nullptr, (const cpx<T>*)v, EPI_NORM, ra, nullptr); }
+  { ProfScope ps_(sizeof(T) == 4 ? PC_VEC32 : PC_VEC64, st, (double)1 * sys.len * sizeof(cpx<T>), 0.0); pdl_launch(k_norms<T, 1>, rb, kRedThreads, 0, st, ix, nullptr, (const cpx<T>*)v, EPI_NORM, ra, nullptr); }
   double rr = 0.0;
   cudaMemcpyAsync(&rr, &kw.ks->rr, sizeof(double), cudaMemcpyDeviceToHost, st);
   cudaStreamSynchronize(st);
@@ -884,7 +906,7 @@ double spec_dot_host(const SpecSystem& sys, const void* a, const void* b, const 
   RedArgs ra{kw.ks, kw.partials, kw.counter, kw.hist, 0.0};
   const int rb = red_blocks(sys.len);
   const Ix ix = mkix(sys.len, sys.h0, sys.G->g.ncplx, rb, kRedThreads);
-  { ProfScope ps_(sizeof(T) == 4 ? PC_VEC32 : PC_VEC64, st, (double)2 * sys.len * sizeof(cpx<T>), 0.0); k_pdot<T><<<rb, kRedThreads, 0, st>>>(ix, (const cpx<T>*)a, (const cpx<T>*)b, ra); }
+  { ProfScope ps_(sizeof(T) == 4 ? PC_VEC32 : PC_VEC64, st, (double)2 * sys.len * sizeof(cpx<T>), 0.0); pdl_launch(k_pdot<T>, rb, kRedThreads, 0, st, ix, (const cpx<T>*)a, (const cpx<T>*)b, ra); }
   double rr = 0.0;
   cudaMemcpyAsync(&rr, &kw.ks->rr, sizeof(double), cudaMemcpyDeviceToHost, st);
   cudaStreamSynchronize(st);
@@ -896,7 +918,7 @@ double spec_sub_norm2_host(const SpecSystem& sys, const void* b, const void* q, 
   RedArgs ra{kw.ks, kw.partials, kw.counter, kw.hist, 0.0};
   const int rb = red_blocks(sys.len);
   const Ix ix = mkix(sys.len, sys.h0, sys.G->g.ncplx, rb, kRedThreads);
-  { ProfScope ps_(PC_VEC64, st, (double)3 * sys.len * sizeof(cpx<double>), 0.0); k_sub_norm<double><<<rb, kRedThreads, 0, st>>>(ix, (const cpx<double>*)b, (const cpx<double>*)q, (cpx<double>*)r, ra); }
+  { ProfScope ps_(PC_VEC64, st, (double)3 * sys.len * sizeof(cpx<double>), 0.0); pdl_launch(k_sub_norm<double>, rb, kRedThreads, 0, st, ix, (const cpx<double>*)b, (const cpx<double>*)q, (cpx<double>*)r, ra); }
   double rr = 0.0;
   cudaMemcpyAsync(&rr, &kw.ks->rr, sizeof(double), cudaMemcpyDeviceToHost, st);
   cudaStreamSynchronize(st);
@@ -904,11 +926,11 @@ double spec_sub_norm2_host(const SpecSystem& sys, const void* b, const void* q, 
 }
 
 void spec_d2f_scaled(long long len, const void* in, double s, void* out, cudaStream_t st) {
-  { ProfScope ps_(PC_VEC64, st, (double)len * (sizeof(cpx<double>) + sizeof(cpx<float>)), 0.0); k_d2f_scaled<<<ew_blocks(len), 256, 0, st>>>(len, (const cpx<double>*)in, s, nullptr, (cpx<float>*)out); }
+  { ProfScope ps_(PC_VEC64, st, (double)len * (sizeof(cpx<double>) + sizeof(cpx<float>)), 0.0); pdl_launch(k_d2f_scaled, ew_blocks(len), 256, 0, st, len, (const cpx<double>*)in, s, nullptr, (cpx<float>*)out); }
 }
 
 void spec_axpy_f2d(long long len, double a, const void* xf, void* y, cudaStream_t st) {
-  { ProfScope ps_(PC_VEC64, st, (double)len * (sizeof(cpx<float>) + 2 * sizeof(cpx<double>)), 0.0); k_axpy_f2d<<<ew_blocks(len), 256, 0, st>>>(len, a, nullptr, (const cpx<float>*)xf, (cpx<double>*)y); }
+  { ProfScope ps_(PC_VEC64, st, (double)len * (sizeof(cpx<float>) + 2 * sizeof(cpx<double>)), 0.0); pdl_launch(k_axpy_f2d, ew_blocks(len), 256, 0, st, len, a, nullptr, (const cpx<float>*)xf, (cpx<double>*)y); }
 }
 
 // ---------------------------------------------------------------------------------------
@@ -1050,9 +1072,9 @@ vd_status krylov_solve(const SpecSystem& sys, const SolveOpts& o, const void* b,
       VD_CUDA(cudaMemcpyAsync(r, B, sizeof(cpx<T>) * len, cudaMemcpyDeviceToDevice, st));
     } else {
       sys.apply(sys, X, q, false, nullptr, st);
-      { ProfScope ps_(sizeof(T) == 4 ? PC_VEC32 : PC_VEC64, st, (double)3 * len * sizeof(cpx<T>), 0.0); k_sub<T><<<eb, 256, 0, st>>>(len, B, q, r, nullptr); }
+      { ProfScope ps_(sizeof(T) == 4 ? PC_VEC32 : PC_VEC64, st, (double)3 * len * sizeof(cpx<T>), 0.0); pdl_launch(k_sub<T>, eb, 256, 0, st, len, B, q, r, nullptr); }
     }
-    { ProfScope ps_(sizeof(T) == 4 ? PC_VEC32 : PC_VEC64, st, (double)3 * len * sizeof(cpx<T>) + (double)nc * sizeof(T), 0.0); k_cg_init<T><<<rb, kRedThreads, 0, st>>>(ixr, B, r, p, sym, ra); }
+    { ProfScope ps_(sizeof(T) == 4 ? PC_VEC32 : PC_VEC64, st, (double)3 * len * sizeof(cpx<T>) + (double)nc * sizeof(T), 0.0); pdl_launch(k_cg_init<T>, rb, kRedThreads, 0, st, ixr, B, r, p, sym, ra); }
     int it = 0;
     HeadPipeLease lease;
     HeadPipe* hp = lease.get();
@@ -1060,9 +1082,9 @@ vd_status krylov_solve(const SpecSystem& sys, const SolveOpts& o, const void* b,
       const long long mark = prof_mark();
       for (int c = 0; c < check && it < o.maxit; ++c, ++it) {
         sys.apply(sys, p, q, false, done, st);
-        { ProfScope ps_(sizeof(T) == 4 ? PC_VEC32 : PC_VEC64, st, (double)2 * len * sizeof(cpx<T>), 0.0); k_dot<T, 1><<<rb, kRedThreads, 0, st>>>(ixr, p, q, EPI_CG_ALPHA, ra, done); }
-        { ProfScope ps_(sizeof(T) == 4 ? PC_VEC32 : PC_VEC64, st, (double)6 * len * sizeof(cpx<T>) + (double)nc * sizeof(T), 0.0); k_cg_update<T><<<rb, kRedThreads, 0, st>>>(ixr, X, p, r, q, sym, ra); }
-        { ProfScope ps_(sizeof(T) == 4 ? PC_VEC32 : PC_VEC64, st, (double)3 * len * sizeof(cpx<T>) + (double)nc * sizeof(T), 0.0); k_cg_p<T><<<eb, 256, 0, st>>>(ixe, p, r, sym, kw.ks); }
+        { ProfScope ps_(sizeof(T) == 4 ? PC_VEC32 : PC_VEC64, st, (double)2 * len * sizeof(cpx<T>), 0.0); pdl_launch(k_dot<T, 1>, rb, kRedThreads, 0, st, ixr, p, q, EPI_CG_ALPHA, ra, done); }
+        { ProfScope ps_(sizeof(T) == 4 ? PC_VEC32 : PC_VEC64, st, (double)6 * len * sizeof(cpx<T>) + (double)nc * sizeof(T), 0.0); pdl_launch(k_cg_update<T>, rb, kRedThreads, 0, st, ixr, X, p, r, q, sym, ra); }
+        { ProfScope ps_(sizeof(T) == 4 ? PC_VEC32 : PC_VEC64, st, (double)3 * len * sizeof(cpx<T>) + (double)nc * sizeof(T), 0.0); pdl_launch(k_cg_p<T>, eb, 256, 0, st, ixe, p, r, sym, kw.ks); }
       }
       vd_status e = VD_OK;
       if (!hp) {
@@ -1090,9 +1112,9 @@ vd_status krylov_solve(const SpecSystem& sys, const SolveOpts& o, const void* b,
       VD_CUDA(cudaMemcpyAsync(r, B, sizeof(cpx<T>) * len, cudaMemcpyDeviceToDevice, st));
     } else {
       sys.apply(sys, X, w, false, nullptr, st);
-      { ProfScope ps_(sizeof(T) == 4 ? PC_VEC32 : PC_VEC64, st, (double)3 * len * sizeof(cpx<T>), 0.0); k_sub<T><<<eb, 256, 0, st>>>(len, B, w, r, nullptr); }
+      { ProfScope ps_(sizeof(T) == 4 ? PC_VEC32 : PC_VEC64, st, (double)3 * len * sizeof(cpx<T>), 0.0); pdl_launch(k_sub<T>, eb, 256, 0, st, len, B, w, r, nullptr); }
     }
-    { ProfScope ps_(sizeof(T) == 4 ? PC_VEC32 : PC_VEC64, st, (double)2 * len * sizeof(cpx<T>), 0.0); k_norms<T, 2><<<rb, kRedThreads, 0, st>>>(ixr, B, r, EPI_INIT_RMR, ra, nullptr); }
+    { ProfScope ps_(sizeof(T) == 4 ? PC_VEC32 : PC_VEC64, st, (double)2 * len * sizeof(cpx<T>), 0.0); pdl_launch(k_norms<T, 2>, rb, kRedThreads, 0, st, ixr, B, r, EPI_INIT_RMR, ra, nullptr); }
     int it = 0;
     HeadPipeLease lease;
     HeadPipe* hp = lease.get();
@@ -1100,8 +1122,8 @@ vd_status krylov_solve(const SpecSystem& sys, const SolveOpts& o, const void* b,
       const long long mark = prof_mark();
       for (int c = 0; c < check && it < o.maxit; ++c, ++it) {
         sys.apply(sys, r, w, true, done, st);
-        { ProfScope ps_(sizeof(T) == 4 ? PC_VEC32 : PC_VEC64, st, (double)2 * len * sizeof(cpx<T>), 0.0); k_dot<T, 2><<<rb, kRedThreads, 0, st>>>(ixr, r, w, EPI_RMR_ALPHA, ra, done); }
-        { ProfScope ps_(sizeof(T) == 4 ? PC_VEC32 : PC_VEC64, st, (double)5 * len * sizeof(cpx<T>) + (double)nc * sizeof(T), 0.0); k_rmr_update<T><<<rb, kRedThreads, 0, st>>>(ixr, X, r, w, sym, ra); }
+        { ProfScope ps_(sizeof(T) == 4 ? PC_VEC32 : PC_VEC64, st, (double)2 * len * sizeof(cpx<T>), 0.0); pdl_launch(k_dot<T, 2>, rb, kRedThreads, 0, st, ixr, r, w, EPI_RMR_ALPHA, ra, done); }
+        { ProfScope ps_(sizeof(T) == 4 ? PC_VEC32 : PC_VEC64, st, (double)5 * len * sizeof(cpx<T>) + (double)nc * sizeof(T), 0.0); pdl_launch(k_rmr_update<T>, rb, kRedThreads, 0, st, ixr, X, r, w, sym, ra); }
       }
       vd_status e = VD_OK;
       if (!hp) {
@@ -1125,39 +1147,39 @@ vd_status krylov_solve(const SpecSystem& sys, const SolveOpts& o, const void* b,
   } else {
     cpx<T>* V = vb;
     cpx<T>* w = vb + (size_t)(m + 1) * len;
-    { ProfScope ps_(sizeof(T) == 4 ? PC_VEC32 : PC_VEC64, st, (double)1 * len * sizeof(cpx<T>), 0.0); k_norms<T, 1><<<rb, kRedThreads, 0, st>>>(ixr, nullptr, B, EPI_BB, ra, nullptr); }
+    { ProfScope ps_(sizeof(T) == 4 ? PC_VEC32 : PC_VEC64, st, (double)1 * len * sizeof(cpx<T>), 0.0); pdl_launch(k_norms<T, 1>, rb, kRedThreads, 0, st, ixr, nullptr, B, EPI_BB, ra, nullptr); }
     for (int cycle = 0;; ++cycle) {
       // r = b - A x into V_0 (unnormalised), then V_0 /= beta
       if (cycle == 0 && o.x_zero) {
         VD_CUDA(cudaMemcpyAsync(V, B, sizeof(cpx<T>) * len, cudaMemcpyDeviceToDevice, st));
       } else {
         sys.apply(sys, X, w, false, done, st);
-        { ProfScope ps_(sizeof(T) == 4 ? PC_VEC32 : PC_VEC64, st, (double)3 * len * sizeof(cpx<T>), 0.0); k_sub<T><<<eb, 256, 0, st>>>(len, B, w, V, done); }
+        { ProfScope ps_(sizeof(T) == 4 ? PC_VEC32 : PC_VEC64, st, (double)3 * len * sizeof(cpx<T>), 0.0); pdl_launch(k_sub<T>, eb, 256, 0, st, len, B, w, V, done); }
       }
-      { ProfScope ps_(sizeof(T) == 4 ? PC_VEC32 : PC_VEC64, st, (double)1 * len * sizeof(cpx<T>), 0.0); k_norms<T, 1><<<rb, kRedThreads, 0, st>>>(ixr, nullptr, V, EPI_GM_BETA, ra, done); }
-      { ProfScope ps_(sizeof(T) == 4 ? PC_VEC32 : PC_VEC64, st, (double)2 * len * sizeof(cpx<T>), 0.0); k_gm_scale<T><<<eb, 256, 0, st>>>(ixe, V, V, kw.ks, 1); }
+      { ProfScope ps_(sizeof(T) == 4 ? PC_VEC32 : PC_VEC64, st, (double)1 * len * sizeof(cpx<T>), 0.0); pdl_launch(k_norms<T, 1>, rb, kRedThreads, 0, st, ixr, nullptr, V, EPI_GM_BETA, ra, done); }
+      { ProfScope ps_(sizeof(T) == 4 ? PC_VEC32 : PC_VEC64, st, (double)2 * len * sizeof(cpx<T>), 0.0); pdl_launch(k_gm_scale<T>, eb, 256, 0, st, ixe, V, V, kw.ks, 1); }
       for (int j = 0; j < m; ++j) {
         cpx<T>* Vj = V + (size_t)j * len;
         sys.apply(sys, Vj, w, true, cdone, st);
         gm_orthogonalise<T>(sys, w, V, j, ra, st);
-        { ProfScope ps_(sizeof(T) == 4 ? PC_VEC32 : PC_VEC64, st, (double)2 * len * sizeof(cpx<T>), 0.0); k_gm_scale<T><<<eb, 256, 0, st>>>(ixe, V + (size_t)(j + 1) * len, w, kw.ks, 0); }
+        { ProfScope ps_(sizeof(T) == 4 ? PC_VEC32 : PC_VEC64, st, (double)2 * len * sizeof(cpx<T>), 0.0); pdl_launch(k_gm_scale<T>, eb, 256, 0, st, ixe, V + (size_t)(j + 1) * len, w, kw.ks, 0); }
         if ((j + 1) % check == 0 || j + 1 == m) {
           vd_status e = read_head(kw, &hd, st);
           if (e != VD_OK) return e;
           if (hd.cycle_done || hd.done) break;
         }
       }
-      { k_gm_solve<<<1, 32, 0, st>>>(kw.ks); count_launch(); }
-      { ProfScope ps_(sizeof(T) == 4 ? PC_VEC32 : PC_VEC64, st, (double)(m + 2) * len * sizeof(cpx<T>) + (double)nc * sizeof(T), 0.0); k_gm_update<T><<<eb, 256, 0, st>>>(ixe, X, V, sym, kw.ks); }
-      { k_gm_close<<<1, 1, 0, st>>>(kw.ks); count_launch(); }
+      { pdl_launch(k_gm_solve, 1, 32, 0, st, kw.ks); count_launch(); }
+      { ProfScope ps_(sizeof(T) == 4 ? PC_VEC32 : PC_VEC64, st, (double)(m + 2) * len * sizeof(cpx<T>) + (double)nc * sizeof(T), 0.0); pdl_launch(k_gm_update<T>, eb, 256, 0, st, ixe, X, V, sym, kw.ks); }
+      { pdl_launch(k_gm_close, 1, 1, 0, st, kw.ks); count_launch(); }
       vd_status e = read_head(kw, &hd, st);
       if (e != VD_OK) return e;
       if (hd.done) break;
       if (hd.iters >= o.maxit) {
         // one more loop head forms the true residual and sets the final status
         sys.apply(sys, X, w, false, done, st);
-        { ProfScope ps_(sizeof(T) == 4 ? PC_VEC32 : PC_VEC64, st, (double)3 * len * sizeof(cpx<T>), 0.0); k_sub<T><<<eb, 256, 0, st>>>(len, B, w, V, done); }
-        { ProfScope ps_(sizeof(T) == 4 ? PC_VEC32 : PC_VEC64, st, (double)1 * len * sizeof(cpx<T>), 0.0); k_norms<T, 1><<<rb, kRedThreads, 0, st>>>(ixr, nullptr, V, EPI_GM_BETA, ra, done); }
+        { ProfScope ps_(sizeof(T) == 4 ? PC_VEC32 : PC_VEC64, st, (double)3 * len * sizeof(cpx<T>), 0.0); pdl_launch(k_sub<T>, eb, 256, 0, st, len, B, w, V, done); }
+        { ProfScope ps_(sizeof(T) == 4 ? PC_VEC32 : PC_VEC64, st, (double)1 * len * sizeof(cpx<T>), 0.0); pdl_launch(k_norms<T, 1>, rb, kRedThreads, 0, st, ixr, nullptr, V, EPI_GM_BETA, ra, done); }
         e = read_head(kw, &hd, st);
         if (e != VD_OK) return e;
         break;
@@ -1186,6 +1208,7 @@ vd_status krylov_solve(const SpecSystem& sys, const SolveOpts& o, const void* b,
 // ---------------------------------------------------------------------------------------
 
 __global__ void k_ks_reset(KState* ks, int maxit, int m, cudaGraphConditionalHandle loop) {
+  pdl_wait();
   if (threadIdx.x != 0 || blockIdx.x != 0) return;
   // a loop nested in another conditional body keeps its last condition value: arm it here
   cudaGraphSetConditional(loop, 1u);
@@ -1199,6 +1222,7 @@ __global__ void k_ks_reset(KState* ks, int maxit, int m, cudaGraphConditionalHan
 
 // inner solve of a refinement sweep: budget and tolerance from the refinement state
 __global__ void k_ks_reset_dev(KState* ks, const OState* o, int m, cudaGraphConditionalHandle loop) {
+  pdl_wait();
   if (threadIdx.x != 0 || blockIdx.x != 0) return;
   cudaGraphSetConditional(loop, 1u);
   KHead* h = reinterpret_cast<KHead*>(ks);
@@ -1212,6 +1236,7 @@ __global__ void k_ks_reset_dev(KState* ks, const OState* o, int m, cudaGraphCond
 }
 
 __global__ void k_graph_cond(cudaGraphConditionalHandle handle, const KState* ks) {
+  pdl_wait();
   if (threadIdx.x == 0 && blockIdx.x == 0) cudaGraphSetConditional(handle, ks->done ? 0u : 1u);
 }
 
@@ -1243,8 +1268,8 @@ vd_status krylov_enqueue_graph(const SpecSystem& sys, const SolveOpts& o, const 
     if (cs != cudaStreamCaptureStatusActive) return fail(VD_ERR_INVALID_ARG, "graph solve needs a capturing stream");
     VD_CUDA(cudaGraphConditionalHandleCreate(&hnd, g, 1, cudaGraphCondAssignDefault));
   }
-  if (o.dev_outer) k_ks_reset_dev<<<1, 1, 0, st>>>(kw.ks, o.dev_outer, m, hnd);
-  else k_ks_reset<<<1, 1, 0, st>>>(kw.ks, o.maxit, m, hnd);
+  if (o.dev_outer) pdl_launch(k_ks_reset_dev, 1, 1, 0, st, kw.ks, o.dev_outer, m, hnd);
+  else pdl_launch(k_ks_reset, 1, 1, 0, st, kw.ks, o.maxit, m, hnd);
   count_launch();
   VD_CUDA(cudaMemsetAsync(kw.counter, 0, sizeof(unsigned), st));
   // the while node: splice it into the capture of st, then capture its body on body_st
@@ -1268,7 +1293,7 @@ vd_status krylov_enqueue_graph(const SpecSystem& sys, const SolveOpts& o, const 
     return VD_OK;
   };
   auto close_loop = [&](cudaGraphConditionalHandle hnd) -> vd_status {
-    k_graph_cond<<<1, 1, 0, body_st>>>(hnd, kw.ks);
+    pdl_launch(k_graph_cond, 1, 1, 0, body_st, hnd, kw.ks);
     count_launch();
     cudaGraph_t body = nullptr;
     VD_CUDA(cudaStreamEndCapture(body_st, &body));
@@ -1283,16 +1308,16 @@ vd_status krylov_enqueue_graph(const SpecSystem& sys, const SolveOpts& o, const 
       VD_CUDA(cudaMemcpyAsync(r, B, sizeof(cpx<T>) * len, cudaMemcpyDeviceToDevice, st));
     } else {
       sys.apply(sys, X, q, false, nullptr, st);
-      k_sub<T><<<eb, 256, 0, st>>>(len, B, q, r, nullptr);
+      pdl_launch(k_sub<T>, eb, 256, 0, st, len, B, q, r, nullptr);
       count_launch();
     }
-    k_cg_init<T><<<rb, kRedThreads, 0, st>>>(ixr, B, r, p, sym, ra);
+    pdl_launch(k_cg_init<T>, rb, kRedThreads, 0, st, ixr, B, r, p, sym, ra);
     count_launch();
     if ((e = open_loop(&hnd)) != VD_OK) return e;
     sys.apply(sys, p, q, false, done, body_st);
-    k_dot<T, 1><<<rb, kRedThreads, 0, body_st>>>(ixr, p, q, EPI_CG_ALPHA, ra, done);
-    k_cg_update<T><<<rb, kRedThreads, 0, body_st>>>(ixr, X, p, r, q, sym, ra);
-    k_cg_p<T><<<eb, 256, 0, body_st>>>(ixe, p, r, sym, kw.ks);
+    pdl_launch(k_dot<T, 1>, rb, kRedThreads, 0, body_st, ixr, p, q, EPI_CG_ALPHA, ra, done);
+    pdl_launch(k_cg_update<T>, rb, kRedThreads, 0, body_st, ixr, X, p, r, q, sym, ra);
+    pdl_launch(k_cg_p<T>, eb, 256, 0, body_st, ixe, p, r, sym, kw.ks);
     count_launch();
     count_launch();
     count_launch();
@@ -1304,29 +1329,29 @@ vd_status krylov_enqueue_graph(const SpecSystem& sys, const SolveOpts& o, const 
       VD_CUDA(cudaMemcpyAsync(r, B, sizeof(cpx<T>) * len, cudaMemcpyDeviceToDevice, st));
     } else {
       sys.apply(sys, X, w, false, nullptr, st);
-      k_sub<T><<<eb, 256, 0, st>>>(len, B, w, r, nullptr);
+      pdl_launch(k_sub<T>, eb, 256, 0, st, len, B, w, r, nullptr);
       count_launch();
     }
-    k_norms<T, 2><<<rb, kRedThreads, 0, st>>>(ixr, B, r, EPI_INIT_RMR, ra, nullptr);
+    pdl_launch(k_norms<T, 2>, rb, kRedThreads, 0, st, ixr, B, r, EPI_INIT_RMR, ra, nullptr);
     count_launch();
     if ((e = open_loop(&hnd)) != VD_OK) return e;
     sys.apply(sys, r, w, true, done, body_st);
-    k_dot<T, 2><<<rb, kRedThreads, 0, body_st>>>(ixr, r, w, EPI_RMR_ALPHA, ra, done);
-    k_rmr_update<T><<<rb, kRedThreads, 0, body_st>>>(ixr, X, r, w, sym, ra);
+    pdl_launch(k_dot<T, 2>, rb, kRedThreads, 0, body_st, ixr, r, w, EPI_RMR_ALPHA, ra, done);
+    pdl_launch(k_rmr_update<T>, rb, kRedThreads, 0, body_st, ixr, X, r, w, sym, ra);
     count_launch();
     count_launch();
     if ((e = close_loop(hnd)) != VD_OK) return e;
   } else {
     cpx<T>* V = vb;
     cpx<T>* w = vb + (size_t)(m + 1) * len;
-    k_norms<T, 1><<<rb, kRedThreads, 0, st>>>(ixr, nullptr, B, EPI_BB, ra, nullptr);
+    pdl_launch(k_norms<T, 1>, rb, kRedThreads, 0, st, ixr, nullptr, B, EPI_BB, ra, nullptr);
     count_launch();
     if ((e = open_loop(&hnd)) != VD_OK) return e;
     // one restart cycle: r = b - A x, V_0 = r / beta, m Arnoldi steps, update x
     sys.apply(sys, X, w, false, done, body_st);
-    k_sub<T><<<eb, 256, 0, body_st>>>(len, B, w, V, done);
-    k_norms<T, 1><<<rb, kRedThreads, 0, body_st>>>(ixr, nullptr, V, EPI_GM_BETA, ra, done);
-    k_gm_scale<T><<<eb, 256, 0, body_st>>>(ixe, V, V, kw.ks, 1);
+    pdl_launch(k_sub<T>, eb, 256, 0, body_st, len, B, w, V, done);
+    pdl_launch(k_norms<T, 1>, rb, kRedThreads, 0, body_st, ixr, nullptr, V, EPI_GM_BETA, ra, done);
+    pdl_launch(k_gm_scale<T>, eb, 256, 0, body_st, ixe, V, V, kw.ks, 1);
     count_launch();
     count_launch();
     count_launch();
@@ -1334,12 +1359,12 @@ vd_status krylov_enqueue_graph(const SpecSystem& sys, const SolveOpts& o, const 
       cpx<T>* Vj = V + (size_t)j * len;
       sys.apply(sys, Vj, w, true, cdone, body_st);
       gm_orthogonalise<T>(sys, w, V, j, ra, body_st);
-      k_gm_scale<T><<<eb, 256, 0, body_st>>>(ixe, V + (size_t)(j + 1) * len, w, kw.ks, 0);
+      pdl_launch(k_gm_scale<T>, eb, 256, 0, body_st, ixe, V + (size_t)(j + 1) * len, w, kw.ks, 0);
       count_launch();
     }
-    k_gm_solve<<<1, 32, 0, body_st>>>(kw.ks);
-    k_gm_update<T><<<eb, 256, 0, body_st>>>(ixe, X, V, sym, kw.ks);
-    k_gm_close<<<1, 1, 0, body_st>>>(kw.ks);
+    pdl_launch(k_gm_solve, 1, 32, 0, body_st, kw.ks);
+    pdl_launch(k_gm_update<T>, eb, 256, 0, body_st, ixe, X, V, sym, kw.ks);
+    pdl_launch(k_gm_close, 1, 1, 0, body_st, kw.ks);
     count_launch();
     count_launch();
     count_launch();
@@ -1352,6 +1377,7 @@ vd_status krylov_enqueue_graph(const SpecSystem& sys, const SolveOpts& o, const 
 // result record of a graph solve: info[0] iterations, [1] status, [2] monitored relres,
 // [3] |b|^2, [4] true relres
 __global__ void k_graph_info(const KState* ks, double* info, int phase) {
+  pdl_wait();
   if (threadIdx.x != 0 || blockIdx.x != 0) return;
   if (phase == 0) {
     info[0] = (double)ks->iters;
@@ -1375,13 +1401,13 @@ vd_status krylov_graph_finish(const SpecSystem& sys, const void* b, const void* 
   RedArgs ra{kw.ks, kw.partials, kw.counter, kw.hist, 0.0};
   const cpx<T>* B = (const cpx<T>*)b;
   cpx<T>* W = (cpx<T>*)vecs;
-  k_graph_info<<<1, 1, 0, st>>>(kw.ks, info, 0);
-  k_norms<T, 1><<<rb, kRedThreads, 0, st>>>(ixr, nullptr, B, EPI_NORM, ra, nullptr);
-  k_graph_info<<<1, 1, 0, st>>>(kw.ks, info, 1);
+  pdl_launch(k_graph_info, 1, 1, 0, st, kw.ks, info, 0);
+  pdl_launch(k_norms<T, 1>, rb, kRedThreads, 0, st, ixr, nullptr, B, EPI_NORM, ra, nullptr);
+  pdl_launch(k_graph_info, 1, 1, 0, st, kw.ks, info, 1);
   sys.apply(sys, x, W, false, nullptr, st);
-  k_sub<T><<<eb, 256, 0, st>>>(len, B, W, W, nullptr);
-  k_norms<T, 1><<<rb, kRedThreads, 0, st>>>(ixr, nullptr, W, EPI_NORM, ra, nullptr);
-  k_graph_info<<<1, 1, 0, st>>>(kw.ks, info, 2);
+  pdl_launch(k_sub<T>, eb, 256, 0, st, len, B, W, W, nullptr);
+  pdl_launch(k_norms<T, 1>, rb, kRedThreads, 0, st, ixr, nullptr, W, EPI_NORM, ra, nullptr);
+  pdl_launch(k_graph_info, 1, 1, 0, st, kw.ks, info, 2);
   for (int i = 0; i < 6; ++i) count_launch();
   VD_CUDA(cudaGetLastError());
   return VD_OK;
@@ -1395,6 +1421,7 @@ template vd_status krylov_graph_finish<double>(const SpecSystem&, const void*, c
 
 __global__ void k_out_init(OState* o, const KState* ks, double tol, double itol0, int maxit,
                            cudaGraphConditionalHandle loop) {
+  pdl_wait();
   if (threadIdx.x != 0 || blockIdx.x != 0) return;
   cudaGraphSetConditional(loop, 1u);
   o->bb = ks->rr;   // |b|^2, and the first residual is b
@@ -1413,6 +1440,7 @@ __global__ void k_out_init(OState* o, const KState* ks, double tol, double itol0
 
 // top of a refinement sweep: the same decisions as the host loop of vd_solve
 __global__ void k_out_check(OState* o, cudaGraphConditionalHandle h_loop, cudaGraphConditionalHandle h_sweep) {
+  pdl_wait();
   if (threadIdx.x != 0 || blockIdx.x != 0) return;
   const double rnorm = sqrt(o->rr);
   const double bnorm = sqrt(o->bb);
@@ -1441,6 +1469,7 @@ __global__ void k_out_check(OState* o, cudaGraphConditionalHandle h_loop, cudaGr
 }
 
 __global__ void k_out_after_inner(OState* o, const KState* ks) {
+  pdl_wait();
   if (threadIdx.x != 0 || blockIdx.x != 0) return;
   o->total += ks->iters;
   o->outer += 1;
@@ -1450,10 +1479,12 @@ __global__ void k_out_after_inner(OState* o, const KState* ks) {
 }
 
 __global__ void k_out_rr(OState* o, const KState* ks) {
+  pdl_wait();
   if (threadIdx.x == 0 && blockIdx.x == 0) o->rr = ks->rr;
 }
 
 __global__ void k_out_info(const OState* o, double* info) {
+  pdl_wait();
   if (threadIdx.x != 0 || blockIdx.x != 0) return;
   info[0] = (double)o->total;
   info[1] = (double)(o->done ? o->status : VD_ERR_NOT_CONVERGED);
@@ -1509,8 +1540,8 @@ vd_status refine_enqueue_graph(const SpecSystem& sys64, const SpecSystem& sys32,
     VD_CUDA(cudaGraphConditionalHandleCreate(&h_loop, g0, 1, cudaGraphCondAssignDefault));
   }
   VD_CUDA(cudaMemsetAsync(kw.counter, 0, sizeof(unsigned), st));
-  k_norms<double, 1><<<rb, kRedThreads, 0, st>>>(ixr, nullptr, BH, EPI_NORM, ra, nullptr);
-  k_out_init<<<1, 1, 0, st>>>(ost, kw.ks, tol, itol0, maxit, h_loop);
+  pdl_launch(k_norms<double, 1>, rb, kRedThreads, 0, st, ixr, nullptr, BH, EPI_NORM, ra, nullptr);
+  pdl_launch(k_out_init, 1, 1, 0, st, ost, kw.ks, tol, itol0, maxit, h_loop);
   VD_CUDA(cudaMemsetAsync(XH, 0, sizeof(cpx<double>) * len, st));
   VD_CUDA(cudaMemcpyAsync(RH, BH, sizeof(cpx<double>) * len, cudaMemcpyDeviceToDevice, st));
   count_launch();
@@ -1526,7 +1557,7 @@ vd_status refine_enqueue_graph(const SpecSystem& sys64, const SpecSystem& sys32,
     VD_CUDA(cudaStreamGetCaptureInfo(s1, &cs, nullptr, &g1, nullptr, nullptr, nullptr));
     VD_CUDA(cudaGraphConditionalHandleCreate(&h_sweep, g1, 0, cudaGraphCondAssignDefault));
   }
-  k_out_check<<<1, 1, 0, s1>>>(ost, h_loop, h_sweep);
+  pdl_launch(k_out_check, 1, 1, 0, s1, ost, h_loop, h_sweep);
   count_launch();
   {
     cudaStreamCaptureStatus cs;
@@ -1546,24 +1577,24 @@ vd_status refine_enqueue_graph(const SpecSystem& sys64, const SpecSystem& sys32,
   }
   VD_CUDA(cudaStreamBeginCaptureToGraph(s2, sweep_body, nullptr, nullptr, 0, cudaStreamCaptureModeRelaxed));
   // the sweep: d solves A32 d = r/|r| in float, x += |r| d, r = b - A x, |r|^2
-  k_d2f_scaled<<<eb, 256, 0, s2>>>(len, RH, 0.0, ost, (cpx<float>*)bh_f);
+  pdl_launch(k_d2f_scaled, eb, 256, 0, s2, len, RH, 0.0, ost, (cpx<float>*)bh_f);
   count_launch();
   VD_CUDA(cudaMemsetAsync(xh_f, 0, sizeof(cpx<float>) * len, s2));
   SolveOpts si = inner;
   si.x_zero = 1;
   si.dev_outer = ost;
   if ((e = krylov_enqueue_graph<float>(sys32, si, bh_f, xh_f, vecs, kw, s2, s3)) != VD_OK) return e;
-  k_out_after_inner<<<1, 1, 0, s2>>>(ost, kw.ks);
-  k_axpy_f2d<<<eb, 256, 0, s2>>>(len, 0.0, ost, (const cpx<float>*)xh_f, XH);
+  pdl_launch(k_out_after_inner, 1, 1, 0, s2, ost, kw.ks);
+  pdl_launch(k_axpy_f2d, eb, 256, 0, s2, len, 0.0, ost, (const cpx<float>*)xh_f, XH);
   resid(resid_ctx, XH, RH, s2);
   VD_CUDA(cudaMemsetAsync(kw.counter, 0, sizeof(unsigned), s2));
-  k_sub_norm<double><<<rb, kRedThreads, 0, s2>>>(ixr, BH, RH, RH, ra);
-  k_out_rr<<<1, 1, 0, s2>>>(ost, kw.ks);
+  pdl_launch(k_sub_norm<double>, rb, kRedThreads, 0, s2, ixr, BH, RH, RH, ra);
+  pdl_launch(k_out_rr, 1, 1, 0, s2, ost, kw.ks);
   for (int i = 0; i < 4; ++i) count_launch();
   cudaGraph_t tmp = nullptr;
   VD_CUDA(cudaStreamEndCapture(s2, &tmp));
   VD_CUDA(cudaStreamEndCapture(s1, &tmp));
-  k_out_info<<<1, 1, 0, st>>>(ost, info);
+  pdl_launch(k_out_info, 1, 1, 0, st, ost, info);
   count_launch();
   (void)sys64;
   VD_CUDA(cudaGetLastError());

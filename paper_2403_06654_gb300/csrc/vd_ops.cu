@@ -4,6 +4,7 @@
 //   L~ psi = sum_j i k~_j F[ rho^-1 F^-1( i k~_j psi ) ]
 // Velocity operator (Eq. VDINSE.zeta with the Crank--Nicolson factor a = dt/(2 Re)):
 //   V~ u = u - a F[ rho^-1 ( Lap u + Sc^-1 ( (u.grad) grad rho + (grad rho.grad) u ) ) ]
+#include "vd_launch.cuh"
 #include "vd_internal.h"
 #include "vd_prof.h"
 #include "vd_fft.cuh"
@@ -541,6 +542,7 @@ int krho_tmp_fields(int ndim) { return ndim >= 2 ? 1 : 0; }
 template <typename T>
 __global__ void k_krho_local(GridDesc g, const cpx<T>* __restrict__ in, cpx<T>* __restrict__ out, int with_inv,
                              const int* done) {
+  pdl_wait();
   if (done && *done) return;
   for (long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x; e < g.ncplx;
        e += (long long)gridDim.x * blockDim.x) {
@@ -573,7 +575,7 @@ template <typename U>
 static void krho_local(const vd_grid* G, const void* in, void* out, bool with_inv, const int* done, cudaStream_t st) {
   const long long n = G->g.ncplx;
   const int blocks = (int)std::min<long long>((n + 255) / 256, 4096);
-  k_krho_local<U><<<blocks, 256, 0, st>>>(G->g, (const cpx<U>*)in, (cpx<U>*)out, with_inv ? 1 : 0, done);
+  pdl_launch(k_krho_local<U>, blocks, 256, 0, st, G->g, (const cpx<U>*)in, (cpx<U>*)out, with_inv ? 1 : 0, done);
   count_launch();
 }
 
@@ -953,6 +955,7 @@ template <typename T>
 __global__ void k_spec_axpby_sym(long long n, long long nc, const cpx<T>* __restrict__ x, const T* __restrict__ sym,
                                  T alpha, const cpx<T>* __restrict__ y, T beta, cpx<T>* __restrict__ out,
                                  const int* done) {
+  pdl_wait();
   if (done && *done) return;
   for (long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x; e < n; e += (long long)gridDim.x * blockDim.x) {
     const T s = sym ? sym[e % nc] * alpha : alpha;
@@ -966,10 +969,10 @@ void spec_axpby_sym_launch(const vd_grid* G, int sz, int ncomp, const void* x, c
   const long long n = nc * ncomp;
   const int blocks = (int)std::min<long long>((n + 255) / 256, 4096);
   if (sz == 8)
-    { k_spec_axpby_sym<double><<<blocks, 256, 0, st>>>(n, nc, (const cpx<double>*)x, (const double*)symarr, alpha,
+    { pdl_launch(k_spec_axpby_sym<double>, blocks, 256, 0, st, n, nc, (const cpx<double>*)x, (const double*)symarr, alpha,
                                                      (const cpx<double>*)y, beta, (cpx<double>*)out, done); count_launch(); }
   else
-    { k_spec_axpby_sym<float><<<blocks, 256, 0, st>>>(n, nc, (const cpx<float>*)x, (const float*)symarr, (float)alpha,
+    { pdl_launch(k_spec_axpby_sym<float>, blocks, 256, 0, st, n, nc, (const cpx<float>*)x, (const float*)symarr, (float)alpha,
                                                     (const cpx<float>*)y, (float)beta, (cpx<float>*)out, done); count_launch(); }
 }
 
@@ -982,6 +985,7 @@ template <typename T>
 __global__ void k_vel_combine(int d, long long nreal, const T* __restrict__ u, const T* __restrict__ du,
                               T* __restrict__ lap, const double* __restrict__ rho, DensPtrs dp, double inv_sc,
                               const int* done) {
+  pdl_wait();
   if (done && *done) return;
   for (long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x; e < nreal;
        e += (long long)gridDim.x * blockDim.x) {
@@ -1008,10 +1012,10 @@ void velocity_combine_launch(const vd_grid* G, int sz, const void* u, const void
   for (int j = 0; j < 6; ++j) dp.h[j] = G->hrho[j];
   const int blocks = (int)std::min<long long>((n + 255) / 256, 4096);
   if (sz == 8)
-    { k_vel_combine<double><<<blocks, 256, 0, st>>>(G->g.ndim, n, (const double*)u, (const double*)du, (double*)lap,
+    { pdl_launch(k_vel_combine<double>, blocks, 256, 0, st, G->g.ndim, n, (const double*)u, (const double*)du, (double*)lap,
                                                   G->rho, dp, inv_sc, done); count_launch(); }
   else
-    { k_vel_combine<float><<<blocks, 256, 0, st>>>(G->g.ndim, n, (const float*)u, (const float*)du, (float*)lap,
+    { pdl_launch(k_vel_combine<float>, blocks, 256, 0, st, G->g.ndim, n, (const float*)u, (const float*)du, (float*)lap,
                                                  G->rho, dp, inv_sc, done); count_launch(); }
 }
 
@@ -1021,6 +1025,7 @@ void velocity_combine_launch(const vd_grid* G, int sz, const void* u, const void
 
 template <typename T>
 __global__ void k_fill_symbol(GridDesc g, int kind, double a, T* __restrict__ out) {
+  pdl_wait();
   // field offsets fit in 32 bits (ncplx < 2^31 is checked when the grid is created)
   const int nc = (int)g.ncplx;
   // K_rho symbols use the full wavenumbers (Nyquist kept); the others k~
@@ -1054,7 +1059,7 @@ template <typename T>
 void fill_symbol(const vd_grid* G, int kind, double a, T* out, cudaStream_t st) {
   const long long n = G->g.ncplx;
   const int blocks = (int)std::min<long long>((n + 255) / 256, 4096);
-  { k_fill_symbol<T><<<blocks, 256, 0, st>>>(G->g, kind, a, out); count_launch(); }
+  { pdl_launch(k_fill_symbol<T>, blocks, 256, 0, st, G->g, kind, a, out); count_launch(); }
 }
 
 template void fwd_transform<double>(const vd_grid*, const double*, cpx<double>*, cudaStream_t);

@@ -1,4 +1,5 @@
 // Transform pass kernels: strided-axis passes (y, z) and the fused contiguous x pass.
+#include "vd_launch.cuh"
 #include "vd_passes.cuh"
 #include "vd_fft.cuh"
 
@@ -139,7 +140,6 @@ template <typename T, int S, bool CV, bool PK = false>
 __global__ void __launch_bounds__(kThreads, 4) k_axis(const AxisProg P, const GridDesc g,
                                                    const cpx<T>* __restrict__ twg, int lw) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  if (P.done && *P.done) return;
   const int axis = P.axis;
   const FftPlan& pl = (axis == 2) ? g.pz : g.py;
   const int n = pl.n;
@@ -154,6 +154,8 @@ __global__ void __launch_bounds__(kThreads, 4) k_axis(const AxisProg P, const Gr
     if constexpr (PK) p_tw_entry<S>(twg[pl.tw_off + j], &tw[j], &tw2[j]);
     else tw[j] = twg[pl.tw_off + j];
   }
+  pdl_wait();
+  if (P.done && *P.done) return;
 
   // field offsets fit in 32 bits (ncplx < 2^31 is checked when the grid is created)
   int line_stride, inner_n, outer_stride;
@@ -376,7 +378,6 @@ __global__ void __launch_bounds__(kRLines * N2, (N2 == 16 ? 3 : 2)) k_axis_r(con
   constexpr int C = N1 / N2;
   constexpr int LS = N + 1;
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  if (P.done && *P.done) return;
   const int axis = P.axis;
   const FftPlan& pl = (axis == 2) ? g.pz : g.py;
   cpx<T>* tw = reinterpret_cast<cpx<T>*>(smem_raw);
@@ -388,6 +389,8 @@ __global__ void __launch_bounds__(kRLines * N2, (N2 == 16 ? 3 : 2)) k_axis_r(con
     tw[j] = twg[pl.tw_off + j];
     katab[j] = kfa * (T)freq_tilde(j, N);
   }
+  pdl_wait();
+  if (P.done && *P.done) return;
   __syncthreads();   // the tables are read by every thread before the first transpose
 
   // lines: z pass, the columns of the flattened (y, x) plane; y pass, the x columns of each z
@@ -608,7 +611,6 @@ __global__ void __launch_bounds__(kRLines * N2, (N2 == 16 ? 3 : 6))
   constexpr unsigned kBoxBytes = (unsigned)(N * (AX == 2 ? kRLines : kPairCols) * sizeof(cpx<T>));
   extern __shared__ __align__(1024) unsigned char smem_tma[];
   unsigned char* smem_raw = smem_tma;
-  if (P.done && *P.done) return;
   constexpr int axis = AX;   // 1 = y, 2 = z (compiled apart: the z form keeps its register budget)
   const FftPlan& pl = (axis == 2) ? g.pz : g.py;
   cpx<T>* buf = reinterpret_cast<cpx<T>*>(smem_raw);                       // the staged tile
@@ -623,6 +625,8 @@ __global__ void __launch_bounds__(kRLines * N2, (N2 == 16 ? 3 : 6))
     katab[j] = kfa * (T)freq_tilde(j, N);
   }
   if (tid == 0) mbar_init(bar, 1);
+  pdl_wait();
+  if (P.done && *P.done) return;
   __syncthreads();
 
   // z pass: lines are the columns of the flattened (y, x) plane (one "plane" of tiles);
@@ -785,7 +789,6 @@ template <typename T, bool CV, bool PK = false, int MINB = 3>
 __global__ void __launch_bounds__(kThreads, MINB) k_xpass(const XProg P, const GridDesc g,
                                                     const cpx<T>* __restrict__ twg, int llpc, int ltpl) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  if (P.done && *P.done) return;
   const int m = g.n0 / 2;
   const int h0 = g.h0;
   const int ls = m + 1;
@@ -815,6 +818,8 @@ __global__ void __launch_bounds__(kThreads, MINB) k_xpass(const XProg P, const G
     if constexpr (PK) p_tw_entry<-1>(twg[g.pk_off + j], &pkx[j], &pkx[m + 1 + j]);
     else pk[j] = twg[g.pk_off + j];
   }
+  pdl_wait();
+  if (P.done && *P.done) return;
 
   const long long nlines = (long long)g.n1 * g.n2;
   const long long line0 = (long long)blockIdx.x * LPC;
@@ -1079,7 +1084,6 @@ __global__ void __launch_bounds__(256, (sizeof(T) == 4 ? 4 : 1)) k_xpass_r(const
   using X = XR<T, M1, M2>;
   constexpr int M = X::M, LINES = X::LINES, LS = X::LS;
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  if (P.done && *P.done) return;
   const int h0 = g.h0;
   cpx<T>* twm = reinterpret_cast<cpx<T>*>(smem_raw);
   cpx<T>* pk = twm + M;
@@ -1087,6 +1091,8 @@ __global__ void __launch_bounds__(256, (sizeof(T) == 4 ? 4 : 1)) k_xpass_r(const
   const int tid = threadIdx.x;
   for (int j = tid; j < M; j += 256) twm[j] = twg[g.px.tw_off + j];
   for (int j = tid; j <= M; j += 256) pk[j] = twg[g.pk_off + j];
+  pdl_wait();
+  if (P.done && *P.done) return;
   const long long nlines = (long long)g.n1 * g.n2;
   const long long line0 = (long long)blockIdx.x * LINES;
   const int line = tid / M2;
@@ -1229,7 +1235,6 @@ __global__ void __launch_bounds__(256, 3) k_xpass_tma(const XProg P, const GridD
   constexpr int M = X::M, LINES = X::LINES, LS = X::LS;
   extern __shared__ __align__(1024) unsigned char smem_tma[];
   unsigned char* smem_raw = smem_tma;
-  if (P.done && *P.done) return;
   const int h0 = g.h0;
   const int pitch = h0;
   const unsigned stage_bytes = (unsigned)(LINES * pitch * sizeof(cpx<T>));   // multiple of 16 (LINES even)
@@ -1242,6 +1247,8 @@ __global__ void __launch_bounds__(256, 3) k_xpass_tma(const XProg P, const GridD
   for (int j = tid; j < M; j += 256) twm[j] = twg[g.px.tw_off + j];
   for (int j = tid; j <= M; j += 256) pk[j] = twg[g.pk_off + j];
   if (tid == 0) mbar_init(bar, 1);
+  pdl_wait();
+  if (P.done && *P.done) return;
   __syncthreads();
   const long long nlines = (long long)g.n1 * g.n2;
   const int groups = (int)((nlines + LINES - 1) / LINES);
@@ -1373,7 +1380,7 @@ static bool launch_xpass_tma(const XProg& P, const GridDesc& g, const cpx<float>
   const size_t smem = sizeof(cpx<float>) * (size_t)(X::LINES * pitch) + 16 +
                       sizeof(cpx<float>) * (size_t)(X::M + (X::M + 2) + X::LINES * X::LS);
   ensure_smem(reinterpret_cast<const void*>(k_xpass_tma<M1, M2>), smem);
-  k_xpass_tma<M1, M2><<<(unsigned)blocks, 256, smem, st>>>(P, g, tw);
+  pdl_launch(k_xpass_tma<M1, M2>, (unsigned)blocks, 256, smem, st, P, g, tw);
   return true;
 }
 
@@ -1384,7 +1391,7 @@ static void launch_xpass_r(const XProg& P, const GridDesc& g, const cpx<T>* tw, 
   const long long blocks = (nlines + X::LINES - 1) / X::LINES;
   const size_t smem = sizeof(cpx<T>) * (size_t)(X::M + (X::M + 2) + X::LINES * X::LS);
   ensure_smem(reinterpret_cast<const void*>(k_xpass_r<T, M1, M2>), smem);
-  k_xpass_r<T, M1, M2><<<(unsigned)blocks, 256, smem, st>>>(P, g, tw);
+  pdl_launch(k_xpass_r<T, M1, M2>, (unsigned)blocks, 256, smem, st, P, g, tw);
 }
 
 // ---------------------------------------------------------------------------------------
@@ -1510,7 +1517,7 @@ static void launch_k_axis(const AxisProg& P, const GridDesc& g, const cpx<T>* tw
   const int n = (P.axis == 2) ? g.pz.n : g.py.n;
   const int threads = std::min(kThreads, std::max(32, W * std::max((n + 7) / 8, (31 + W) / W)));
   ensure_smem(reinterpret_cast<const void*>(k_axis<T, S, CV, PK>), smem);
-  k_axis<T, S, CV, PK><<<(unsigned)blocks, threads, smem, st>>>(P, g, tw, ilog2(W));
+  pdl_launch(k_axis<T, S, CV, PK>, (unsigned)blocks, threads, smem, st, P, g, tw, ilog2(W));
 }
 
 template <typename T, int S, int N1, int N2>
@@ -1519,7 +1526,7 @@ static void launch_axis_r(const AxisProg& P, const GridDesc& g, const cpx<T>* tw
   const long long blocks = outer_n * ((inner_n + kRLines - 1) / kRLines);
   const size_t smem = sizeof(cpx<T>) * (size_t)(N1 * N2 + kRLines * (N1 * N2 + 1)) + sizeof(T) * (size_t)(N1 * N2);
   ensure_smem(reinterpret_cast<const void*>(k_axis_r<T, S, N1, N2>), smem);
-  k_axis_r<T, S, N1, N2><<<(unsigned)blocks, kRLines * N2, smem, st>>>(P, g, tw);
+  pdl_launch(k_axis_r<T, S, N1, N2>, (unsigned)blocks, kRLines * N2, smem, st, P, g, tw);
 }
 
 static void split_scale(double s, float* hi, float* lo) {
@@ -1616,7 +1623,7 @@ static bool launch_axis_tma(const AxisProg& P, const GridDesc& g, const cpx<floa
   const size_t stage = sizeof(cpx<float>) * (size_t)(N * (AX == 2 ? kRLines : kPairCols));
   const size_t smem = stage + 16 + sizeof(cpx<float>) * (size_t)(N + kRLines * (N + 1)) + sizeof(float) * (size_t)N;
   ensure_smem(reinterpret_cast<const void*>(k_axis_tma<S, N1, N2, AX>), smem);
-  k_axis_tma<S, N1, N2, AX><<<(unsigned)blocks, kRLines * N2, smem, st>>>(P, g, tw, maps);
+  pdl_launch(k_axis_tma<S, N1, N2, AX>, (unsigned)blocks, kRLines * N2, smem, st, P, g, tw, maps);
   return true;
 }
 
@@ -1709,7 +1716,7 @@ static void launch_k_xpass(const XProg& P, const GridDesc& g, const cpx<T>* tw, 
   ensure_smem(reinterpret_cast<const void*>(k_xpass<T, CV, PK, MINB>), smem);
   // threads per line: a power of two, one radix-8 butterfly each, at least a warp per block
   const int tpl = std::min(kThreads / L, std::max(pow2_at_least((g.px.n + 7) / 8), pow2_at_least((31 + L) / L)));
-  k_xpass<T, CV, PK, MINB><<<(unsigned)blocks, L * tpl, smem, st>>>(P, g, tw, ilog2(L), ilog2(tpl));
+  pdl_launch(k_xpass<T, CV, PK, MINB>, (unsigned)blocks, L * tpl, smem, st, P, g, tw, ilog2(L), ilog2(tpl));
 }
 
 template <typename T>

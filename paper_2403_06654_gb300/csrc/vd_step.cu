@@ -18,6 +18,7 @@
 // Readings: Adams--Bashforth 2 (1.5 N^n - 0.5 N^{n-1}), Euler on the first step; periodic
 // gravity f = -Fr^-1 (1 - <rho_h>/rho_h) e_g.  Both solves are warm-started from the
 // previous solution (u^n for u*, the previous phi for phi).
+#include "vd_launch.cuh"
 #include "vd_internal.h"
 #include "vd_prof.h"
 
@@ -54,6 +55,7 @@ namespace vd {
 // out = sum_j a_j b_j   (a, b: d fields of n points)
 __global__ void k_dotvec(long long n, int d, const double* __restrict__ a, const double* __restrict__ b,
                          double* __restrict__ out) {
+  pdl_wait();
   EW_LOOP(e, n) {
     double s = 0.0;
     for (int j = 0; j < d; ++j) s += a[j * n + e] * b[j * n + e];
@@ -63,11 +65,13 @@ __global__ void k_dotvec(long long n, int d, const double* __restrict__ a, const
 // out = alpha x + beta y
 __global__ void k_lin(long long n, double alpha, const double* __restrict__ x, double beta, const double* __restrict__ y,
                       double* __restrict__ out) {
+  pdl_wait();
   EW_LOOP(e, n) { out[e] = alpha * x[e] + (y ? beta * y[e] : 0.0); }
 }
 // spectral Crank--Nicolson mass update
 __global__ void k_mass(GridDesc g, double c, double dt, const cpx<double>* __restrict__ rh,
                        const cpx<double>* __restrict__ ab, cpx<double>* __restrict__ out) {
+  pdl_wait();
   EW_LOOP(e, g.ncplx) {
     const long long line = e / g.h0;
     const int kxi = (int)(e - line * g.h0);
@@ -92,6 +96,7 @@ __global__ void k_rhs(long long n, int d, const double* __restrict__ u, const do
                       const double* __restrict__ gradp, const double* __restrict__ rho_h, const double* __restrict__ hz,
                       double dt, int gaxis, double inv_fr, double mean_rho, const double* __restrict__ fext,
                       double* __restrict__ out) {
+  pdl_wait();
   EW_LOOP(e, n) {
     const double r = rho_h[e];
     for (int i = 0; i < d; ++i) {
@@ -105,6 +110,7 @@ __global__ void k_rhs(long long n, int d, const double* __restrict__ u, const do
 // out_i = rho a_i
 __global__ void k_mul_by(long long n, int d, const double* __restrict__ a, const double* __restrict__ rho,
                          double* __restrict__ out) {
+  pdl_wait();
   EW_LOOP(e, n) {
     const double r = rho[e];
     for (int i = 0; i < d; ++i) out[i * n + e] = r * a[i * n + e];
@@ -113,6 +119,7 @@ __global__ void k_mul_by(long long n, int d, const double* __restrict__ a, const
 // out_i = a_i / rho
 __global__ void k_div_by(long long n, int d, const double* __restrict__ a, const double* __restrict__ rho,
                          double* __restrict__ out) {
+  pdl_wait();
   EW_LOOP(e, n) {
     const double r = rho[e];
     for (int i = 0; i < d; ++i) out[i * n + e] = a[i * n + e] / r;
@@ -121,6 +128,7 @@ __global__ void k_div_by(long long n, int d, const double* __restrict__ a, const
 // u = u* - dt gphi / rho_h
 __global__ void k_project(long long n, int d, const double* __restrict__ us, const double* __restrict__ gphi,
                           const double* __restrict__ rho_h, double dt, double* __restrict__ out) {
+  pdl_wait();
   EW_LOOP(e, n) {
     const double r = rho_h[e];
     for (int i = 0; i < d; ++i) out[i * n + e] = us[i * n + e] - dt * gphi[i * n + e] / r;
@@ -129,6 +137,7 @@ __global__ void k_project(long long n, int d, const double* __restrict__ us, con
 // gradient part of d vector fields, in Fourier: c_j <- k~_j (k~ . c) / |k~|^2 (0 where |k~| = 0),
 // i.e. grad Lap^+ div c with the discrete D_j = F^-1 diag(i k~_j) F
 __global__ void k_grad_part(GridDesc g, int d, cpx<double>* __restrict__ c) {
+  pdl_wait();
   EW_LOOP(e, g.ncplx) {
     const long long line = e / g.h0;
     const int kxi = (int)(e - line * g.h0);
@@ -151,12 +160,14 @@ __global__ void k_grad_part(GridDesc g, int d, cpx<double>* __restrict__ c) {
 // gradp += gphi - gq  (gq: gradient of the scalar-form correction)
 __global__ void k_gradp(long long n, int d, const double* __restrict__ gphi, const double* __restrict__ gq,
                         double* __restrict__ gradp) {
+  pdl_wait();
   EW_LOOP(e, n) {
     for (int i = 0; i < d; ++i) gradp[i * n + e] += gphi[i * n + e] - gq[i * n + e];
   }
 }
 // per-block sums (fixed grid: deterministic order)
 __global__ void k_blocksum(long long n, const double* __restrict__ a, double* __restrict__ part) {
+  pdl_wait();
   __shared__ double sm[256];
   double s = 0.0;
   EW_LOOP(e, n) { s += a[e]; }
@@ -393,26 +404,26 @@ vd_status vd_flow_step(vd_flow* F, double dt, vd_step_info* info, vd_stream stre
 
   // 1. mass equation
   grad_phys(G, F->rho, F->grad, s0, s1, st);
-  { k_dotvec<<<b, 256, 0, st>>>(n, d, F->u, F->grad, F->nrho); count_launch(); }
+  { pdl_launch(k_dotvec, b, 256, 0, st, n, d, F->u, F->grad, F->nrho); count_launch(); }
   const double* ab = F->nrho;
   if (F->have_prev) {
-    { k_lin<<<b, 256, 0, st>>>(n, 1.5, F->nrho, -0.5, F->nrho_prev, F->rhs); count_launch(); }
+    { pdl_launch(k_lin, b, 256, 0, st, n, 1.5, F->nrho, -0.5, F->nrho_prev, F->rhs); count_launch(); }
     ab = F->rhs;
   }
   if (F->has_msrc) {   // [u.grad rho]^{n+1/2} - S^{n+1/2}
-    { k_lin<<<b, 256, 0, st>>>(n, 1.0, ab, -1.0, F->msrc, F->fphi); count_launch(); }
+    { pdl_launch(k_lin, b, 256, 0, st, n, 1.0, ab, -1.0, F->msrc, F->fphi); count_launch(); }
     ab = F->fphi;
   }
   fwd_transform<double>(G, F->rho, s0, st);
   fwd_transform<double>(G, ab, s1, st);
   const double c = dt / (2.0 * p.Re * p.Sc);
-  { k_mass<<<ewb(g.ncplx), 256, 0, st>>>(g, c, dt, s0, s1, s2); count_launch(); }
+  { pdl_launch(k_mass, ewb(g.ncplx), 256, 0, st, g, c, dt, s0, s1, s2); count_launch(); }
   {
     Mult m;
     inv_transform<double>(G, s2, m, F->rho_new, s0, st);
   }
   // 2. mid-step density, attached to the grid with the viscous-operator data
-  { k_lin<<<b, 256, 0, st>>>(n, 0.5, F->rho_new, 0.5, F->rho, F->rho_h); count_launch(); }
+  { pdl_launch(k_lin, b, 256, 0, st, n, 0.5, F->rho_new, 0.5, F->rho, F->rho_h); count_launch(); }
   e = vd_density_set(G, VD_OP_VELOCITY, F->rho_h, F->dens, F->dens_bytes, stream);
   if (e != VD_OK) return e;
   // 3. predictor
@@ -420,21 +431,21 @@ vd_status vd_flow_step(vd_flow* F, double dt, vd_step_info* info, vd_stream stre
   const vd_op_params opp{a, 1.0 / p.Sc};
   for (int i = 0; i < d; ++i) {
     grad_phys(G, F->u + i * n, F->grad, s0, s1, st);
-    { k_dotvec<<<b, 256, 0, st>>>(n, d, F->u, F->grad, F->nu + i * n); count_launch(); }
+    { pdl_launch(k_dotvec, b, 256, 0, st, n, d, F->u, F->grad, F->nu + i * n); count_launch(); }
   }
   const double* abu = F->nu;
   if (F->have_prev) {
-    { k_lin<<<b, 256, 0, st>>>(n * d, 1.5, F->nu, -0.5, F->nu_prev, F->w); count_launch(); }
+    { pdl_launch(k_lin, b, 256, 0, st, n * d, 1.5, F->nu, -0.5, F->nu_prev, F->w); count_launch(); }
     abu = F->w;
   }
   // hz = u - V u  ( = (dt/2) zeta(rho_h, u) )
   e = vd_apply_op(G, VD_OP_VELOCITY, &opp, F->u, F->hz, F->ws, F->ws_bytes, stream);
   if (e != VD_OK) return e;
-  { k_lin<<<ewb(n * d), 256, 0, st>>>(n * d, 1.0, F->u, -1.0, F->hz, F->hz); count_launch(); }
+  { pdl_launch(k_lin, ewb(n * d), 256, 0, st, n * d, 1.0, F->u, -1.0, F->hz, F->hz); count_launch(); }
   double mean_rho = 0.0;
   if (p.gravity_axis >= 0) {
     const int nb = std::min(b, 4096);
-    { k_blocksum<<<nb, 256, 0, st>>>(n, F->rho_h, F->sum); count_launch(); }
+    { pdl_launch(k_blocksum, nb, 256, 0, st, n, F->rho_h, F->sum); count_launch(); }
     std::vector<double> part(nb);
     VD_CUDA(cudaMemcpyAsync(part.data(), F->sum, nb * sizeof(double), cudaMemcpyDeviceToHost, st));
     VD_CUDA(cudaStreamSynchronize(st));
@@ -442,7 +453,7 @@ vd_status vd_flow_step(vd_flow* F, double dt, vd_step_info* info, vd_stream stre
     for (double v : part) s += v;
     mean_rho = s / (double)n;
   }
-  { k_rhs<<<b, 256, 0, st>>>(n, d, F->u, abu, F->gradp, F->rho_h, F->hz, dt, p.gravity_axis, 1.0 / p.Fr, mean_rho,
+  { pdl_launch(k_rhs, b, 256, 0, st, n, d, F->u, abu, F->gradp, F->rho_h, F->hz, dt, p.gravity_axis, 1.0 / p.Fr, mean_rho,
                              F->has_force ? F->force : nullptr, F->rhs); count_launch(); }
   VD_CUDA(cudaMemcpyAsync(F->ustar, F->u, d * n * sizeof(double), cudaMemcpyDeviceToDevice, st));
   vd_solve_params sp{};
@@ -460,7 +471,7 @@ vd_status vd_flow_step(vd_flow* F, double dt, vd_step_info* info, vd_stream stre
   // 4. pressure increment
   e = vd_divergence(G, F->ustar, F->fphi, F->spec, F->spec_bytes, stream);
   if (e != VD_OK) return e;
-  { k_lin<<<b, 256, 0, st>>>(n, 1.0 / dt, F->fphi, 0.0, nullptr, F->fphi); count_launch(); }
+  { pdl_launch(k_lin, b, 256, 0, st, n, 1.0 / dt, F->fphi, 0.0, nullptr, F->fphi); count_launch(); }
   vd_solve_info ip{};
   vd_status spr = vd_solve(G, VD_OP_PRESSURE, (vd_solver)p.pres_solver, nullptr, &sp, F->fphi, F->phi, &ip, F->ws,
                            F->ws_bytes, stream);
@@ -471,20 +482,20 @@ vd_status vd_flow_step(vd_flow* F, double dt, vd_step_info* info, vd_stream stre
   // 6. pressure update, scalar form: w = gphi/rho_h, hz = w - V w, c = rho_h hz, and
   //    grad p += gphi - grad Lap^+ div c, the gradient part of c taken in Fourier
   //    (d forward and d inverse transforms; the solve workspace is free here: scratch)
-  { k_div_by<<<b, 256, 0, st>>>(n, d, F->grad, F->rho_h, F->w); count_launch(); }
+  { pdl_launch(k_div_by, b, 256, 0, st, n, d, F->grad, F->rho_h, F->w); count_launch(); }
   e = vd_apply_op(G, VD_OP_VELOCITY, &opp, F->w, F->hz, F->ws, F->ws_bytes, stream);
   if (e != VD_OK) return e;
-  { k_lin<<<ewb(n * d), 256, 0, st>>>(n * d, 1.0, F->w, -1.0, F->hz, F->hz); count_launch(); }
-  { k_mul_by<<<b, 256, 0, st>>>(n, d, F->hz, F->rho_h, F->hz); count_launch(); }
+  { pdl_launch(k_lin, ewb(n * d), 256, 0, st, n * d, 1.0, F->w, -1.0, F->hz, F->hz); count_launch(); }
+  { pdl_launch(k_mul_by, b, 256, 0, st, n, d, F->hz, F->rho_h, F->hz); count_launch(); }
   for (int j = 0; j < d; ++j) fwd_transform<double>(G, F->hz + (size_t)j * n, s0 + (size_t)j * g.ncplx, st);
-  { k_grad_part<<<ewb(g.ncplx), 256, 0, st>>>(g, d, s0); count_launch(); }
+  { pdl_launch(k_grad_part, ewb(g.ncplx), 256, 0, st, g, d, s0); count_launch(); }
   for (int j = 0; j < d; ++j) {
     Mult m;
     inv_transform<double>(G, s0 + (size_t)j * g.ncplx, m, F->w + (size_t)j * n, reinterpret_cast<cpx<double>*>(F->ws),
                           st);
   }
-  { k_gradp<<<b, 256, 0, st>>>(n, d, F->grad, F->w, F->gradp); count_launch(); }
-  { k_project<<<b, 256, 0, st>>>(n, d, F->ustar, F->grad, F->rho_h, dt, F->u); count_launch(); }
+  { pdl_launch(k_gradp, b, 256, 0, st, n, d, F->grad, F->w, F->gradp); count_launch(); }
+  { pdl_launch(k_project, b, 256, 0, st, n, d, F->ustar, F->grad, F->rho_h, dt, F->u); count_launch(); }
   // history and new density
   VD_CUDA(cudaMemcpyAsync(F->nrho_prev, F->nrho, n * sizeof(double), cudaMemcpyDeviceToDevice, st));
   VD_CUDA(cudaMemcpyAsync(F->nu_prev, F->nu, d * n * sizeof(double), cudaMemcpyDeviceToDevice, st));

@@ -18,6 +18,7 @@
 // scale is not multiplied.
 #pragma once
 
+#include "vd_launch.cuh"
 #include "vd_passes.cuh"
 #include "vd_fft.cuh"
 
@@ -130,7 +131,6 @@ __global__ void __launch_bounds__(kWideThreads, (sizeof(T) == 8 ? 2 : 3))
     k_axis_w(const __grid_constant__ AxisProg P, const __grid_constant__ GridDesc g, const cpx<T>* __restrict__ twg,
              int lw, int tpl, int ps, int cls) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  if (P.done && *P.done) return;
   const int axis = P.axis;
   const WidePlan& pl = (axis == 2) ? g.wz[cls] : g.wy[cls];
   const int n = pl.n, nst = pl.nst, W = 1 << lw;
@@ -170,6 +170,8 @@ __global__ void __launch_bounds__(kWideThreads, (sizeof(T) == 8 ? 2 : 3))
     }
     return k2;
   };
+  pdl_wait();
+  if (P.done && *P.done) return;
   __syncthreads();   // the tables are complete
 
   for (int t = 0; t < P.nxf; ++t) {
@@ -345,7 +347,6 @@ __global__ void __launch_bounds__(kWideThreads, (sizeof(T) == 8 ? 2 : 3))
     k_xpass_w(const __grid_constant__ XProg P, const __grid_constant__ GridDesc g, const cpx<T>* __restrict__ twg,
               int llpc, int ps, int ls, int cls) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  if (P.done && *P.done) return;
   const WidePlan& pl = g.wx[cls];
   const int m = pl.n, nst = pl.nst, h0 = g.h0, half = m / 2 + 1, L = 1 << llpc;
   cpx<T>* tw = reinterpret_cast<cpx<T>*>(smem_raw);   // W_m^j
@@ -370,6 +371,8 @@ __global__ void __launch_bounds__(kWideThreads, (sizeof(T) == 8 ? 2 : 3))
     return c;
   };
   const ItemWalk wh(half);
+  pdl_wait();
+  if (P.done && *P.done) return;
 
   for (int c = 0; c < P.ncomp; ++c) {
     __syncthreads();   // the tables are complete; the previous component's buffers are free
@@ -569,7 +572,7 @@ static void wide_axis_launch(const AxisProg& P, const GridDesc& g, const cpx<T>*
   const int tpl = wide_tpl(pl, W);
   const size_t smem = wide_axis_smem(pl, W, sizeof(T));
   ensure_smem(reinterpret_cast<const void*>(k_axis_w<T, S>), smem);
-  k_axis_w<T, S><<<(unsigned)((lines + W - 1) / W), W * tpl, smem, st>>>(P, g, tw, wide_log2(W), tpl,
+  pdl_launch(k_axis_w<T, S>, (unsigned)((lines + W - 1) / W), W * tpl, smem, st, P, g, tw, wide_log2(W), tpl,
                                                                               wide_pad_shift(pl), cls);
 }
 
@@ -590,7 +593,7 @@ static void wide_xpass_launch(const XProg& P, const GridDesc& g, const cpx<T>* t
   for (int s = 0; s < pl.nst; ++s) nb = std::max(nb, pl.n / pl.rad[s]);
   const int threads = std::min(kWideThreads, (int)std::max<long long>(32, ((long long)L * nb + 31) / 32 * 32));
   ensure_smem(reinterpret_cast<const void*>(k_xpass_w<T, MODE>), smem);
-  k_xpass_w<T, MODE><<<(unsigned)((lines + L - 1) / L), threads, smem, st>>>(P, g, tw, wide_log2(L), ps, ls, cls);
+  pdl_launch(k_xpass_w<T, MODE>, (unsigned)((lines + L - 1) / L), threads, smem, st, P, g, tw, wide_log2(L), ps, ls, cls);
 }
 
 template <typename T>
