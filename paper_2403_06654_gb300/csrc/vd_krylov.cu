@@ -50,17 +50,26 @@ __host__ __device__ constexpr int log2_ceil(int n) { return n <= 1 ? 0 : 1 + log
 // Sums of v[0..NV) (NV <= 32) over the block, one value per group of 8 threads: on return
 // thread 8 i holds the total of value i (other threads nothing).  Within a warp the values are
 // exchanged and halved (lanes whose bit is set keep the upper half of the values, the others the
-// lower half), so NV values cost about NV + 5 - log2 NV additions per lane instead of 5 NV: the
-// tail of a reduction kernel is its FP64 additions (8 values with one butterfly each, 608 blocks:
-// k_gm_mdot 31 us on 87k points, 6 us this way).
-template <int NV>
-__device__ __forceinline__ double block_sums(const double (&v)[NV], double (*sm)[kRedThreads / 32]) {
+// lower half), so NV values cost about NV + 5 - log2 NV additions per lane instead of 5 NV.  V =
+// double, or dd: float-pair totals (of compensated float sums) are added as pairs on the FP32 pipes
+// and widened once per warp, since a block's double additions queue for the FP64 pipe (a lone warp
+// issues one per 64 cycles, eight warps one per 153 each).  87k points, 8 dots, caches flushed: 31.5 us
+// with one double butterfly per value, 17.3 with the exchange in double; 32 dots, caches warm: 22.5 us
+// in double, 14.9 in pairs.
+__device__ __forceinline__ double shfl_xor(double v, int o) { return __shfl_xor_sync(0xffffffffu, v, o); }
+__device__ __forceinline__ dd shfl_xor(dd v, int o) {
+  return dd(__shfl_xor_sync(0xffffffffu, v.hi, o), __shfl_xor_sync(0xffffffffu, v.lo, o));
+}
+__device__ __forceinline__ double to_double(double v) { return v; }
+__device__ __forceinline__ double to_double(dd v) { return widen(v.hi) + widen(v.lo); }
+template <int NV, typename V>
+__device__ __forceinline__ double block_sums(const V (&v)[NV], double (*sm)[kRedThreads / 32]) {
   constexpr int L = log2_ceil(NV), P = 1 << L;
   static_assert(NV >= 1 && P <= 32 && kRedThreads == 256, "one exchange step per lane bit");
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  double a[P];
+  V a[P];
 #pragma unroll
-  for (int i = 0; i < P; ++i) a[i] = i < NV ? v[i < NV ? i : 0] : 0.0;
+  for (int i = 0; i < P; ++i) a[i] = i < NV ? v[i < NV ? i : 0] : V(0.0);
 #pragma unroll
   for (int s = 0; s < 5; ++s) {
     const int o = 16 >> s, cnt = P >> (s + 1);   // values kept after this step
@@ -68,15 +77,15 @@ __device__ __forceinline__ double block_sums(const double (&v)[NV], double (*sm)
       const bool up = (lane & o) != 0;
 #pragma unroll
       for (int i = 0; i < cnt; ++i) {
-        const double give = up ? a[i] : a[i + cnt], keep = up ? a[i + cnt] : a[i];
-        a[i] = keep + __shfl_xor_sync(0xffffffffu, give, o);
+        const V give = up ? a[i] : a[i + cnt], keep = up ? a[i + cnt] : a[i];
+        a[i] = keep + shfl_xor(give, o);
       }
     } else {
-      a[0] += __shfl_xor_sync(0xffffffffu, a[0], o);
+      a[0] = a[0] + shfl_xor(a[0], o);
     }
   }
   const int mine = lane >> (5 - L);   // the value this lane ended with
-  if ((lane & ((32 >> L) - 1)) == 0 && mine < NV) sm[mine][warp] = a[0];
+  if ((lane & ((32 >> L) - 1)) == 0 && mine < NV) sm[mine][warp] = to_double(a[0]);
   __syncthreads();
   double s = 0.0;
   if (warp * 4 < NV) {   // warps holding a thread t with t / 8 < NV
@@ -92,13 +101,13 @@ __device__ __forceinline__ double block_sums(const double (&v)[NV], double (*sm)
 // Block-sum v[0..NV) into per-block partials (partials[i * blocks + block]); the last block gets
 // the totals in tot (every thread).  Returns true (in every thread of the last block) when the
 // caller must run the epilogue.  Fixed order: deterministic.
-template <int NV>
-__device__ bool reduce_last(const double (&v)[NV], double* partials, unsigned* counter, double (&tot)[NV]) {
+template <int NV, typename V>
+__device__ bool reduce_last(const V (&v)[NV], double* partials, unsigned* counter, double (&tot)[NV]) {
   __shared__ double sm[NV][kRedThreads / 32];
   __shared__ int am_last;
   const int nb = (int)gridDim.x;
   const int vi = threadIdx.x >> 3;
-  const double s = block_sums<NV>(v, sm);
+  const double s = block_sums<NV, V>(v, sm);
   if (nb > 1) {
     if ((threadIdx.x & 7) == 0 && vi < NV) {
       partials[vi * nb + blockIdx.x] = s;
@@ -117,17 +126,25 @@ __device__ bool reduce_last(const double (&v)[NV], double* partials, unsigned* c
 #pragma unroll
         for (int i = 0; i < NV; ++i) a[i] += __ldcg(partials + i * nb + b);
       }
-      const double f = block_sums<NV>(a, sm);
+      const double f = block_sums<NV, double>(a, sm);
       if ((threadIdx.x & 7) == 0 && vi < NV) sm[vi][0] = f;
     } else {
-      // warp w sums the values w, w + 8, ...
-      const int lane = threadIdx.x & 31;
-      for (int i = threadIdx.x >> 5; i < NV; i += kRedThreads / 32) {
-        double f = 0.0;
-        for (int b = lane; b < nb; b += 32) f += __ldcg(partials + i * nb + b);
+      // warp w sums the values w, w + 8, ...: their loads together, then the lanes' exchange
+      constexpr int K = (NV + 7) / 8;
+      const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+      double f[K];
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) f += __shfl_xor_sync(0xffffffffu, f, o);
-        if (lane == 0) sm[i][0] = f;
+      for (int k = 0; k < K; ++k) f[k] = 0.0;
+      for (int b = lane; b < nb; b += 32) {
+#pragma unroll
+        for (int k = 0; k < K; ++k)
+          if (w + 8 * k < NV) f[k] += __ldcg(partials + (w + 8 * k) * nb + b);
+      }
+#pragma unroll
+      for (int k = 0; k < K; ++k) {
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) f[k] += __shfl_xor_sync(0xffffffffu, f[k], o);
+        if (lane == 0 && w + 8 * k < NV) sm[w + 8 * k][0] = f[k];
       }
     }
     if (threadIdx.x == 0) *counter = 0u;
@@ -412,6 +429,7 @@ struct Acc {
   __device__ __forceinline__ void add(T v) { a += (double)v; }
   __device__ __forceinline__ void dot(cpx<T> u, cpx<T> v) { a = fma(u.x, v.x, fma(u.y, v.y, a)); }   // += Re(u conj v)
   __device__ __forceinline__ double total() const { return a; }
+  using Sum = double;
 };
 template <>
 struct Acc<float> {
@@ -423,7 +441,8 @@ struct Acc<float> {
     s = t;
   }
   __device__ __forceinline__ void dot(cpx<float> u, cpx<float> v) { add(u.x * v.x + u.y * v.y); }
-  __device__ __forceinline__ double total() const { return widen(s) + widen(c); }
+  __device__ __forceinline__ dd total() const { return dd_fast_two_sum(s, c); }
+  using Sum = dd;
 };
 
 // CG start: p = S r, reduce [bb, rr, rz]
@@ -443,9 +462,9 @@ __global__ void __launch_bounds__(kRedThreads) k_cg_init(Ix ix, const cpx<T>* __
     a1.add(w * r2);
     a2.add(w * sv * r2);
   }
-  double v[3] = {a0.total(), a1.total(), a2.total()};
+  const typename Acc<T>::Sum v[3] = {a0.total(), a1.total(), a2.total()};
   double t[3];
-  if (reduce_last<3>(v, ra.partials, ra.counter, t) && threadIdx.x == 0)
+  if (reduce_last(v, ra.partials, ra.counter, t) && threadIdx.x == 0)
     epilogue<3>(EPI_INIT_CG, t, ra.ks, ra.hist, ra.tol, 0, 0);
 }
 
@@ -462,11 +481,11 @@ __global__ void __launch_bounds__(kRedThreads) k_dot(Ix ix, const cpx<T>* __rest
     a0.dot(wv, u[e]);
     if (NV > 1) a1.dot(wv, vv);
   }
-  double a[NV];
+  typename Acc<T>::Sum a[NV];
   a[0] = a0.total();
   if (NV > 1) a[NV - 1] = a1.total();
   double t[NV];
-  if (reduce_last<NV>(a, ra.partials, ra.counter, t) && threadIdx.x == 0)
+  if (reduce_last(a, ra.partials, ra.counter, t) && threadIdx.x == 0)
     epilogue<NV>(epi, t, ra.ks, ra.hist, ra.tol, 0, 0);
 }
 
@@ -492,9 +511,9 @@ __global__ void __launch_bounds__(kRedThreads) k_cg_update(Ix ix, cpx<T>* __rest
     a0.add(w * r2);
     a1.add(w * sym[si] * r2);
   }
-  double v[2] = {a0.total(), a1.total()};
+  const typename Acc<T>::Sum v[2] = {a0.total(), a1.total()};
   double t[2];
-  if (reduce_last<2>(v, ra.partials, ra.counter, t) && threadIdx.x == 0)
+  if (reduce_last(v, ra.partials, ra.counter, t) && threadIdx.x == 0)
     epilogue<2>(EPI_CG_UPDATE, t, ra.ks, ra.hist, ra.tol, 0, 0);
 }
 
@@ -529,11 +548,11 @@ __global__ void __launch_bounds__(kRedThreads) k_norms(Ix ix, const cpx<T>* __re
     }
     a1.add(w * (rv.x * rv.x + rv.y * rv.y));
   }
-  double v[NV];
+  typename Acc<T>::Sum v[NV];
   if (NV == 2) v[0] = a0.total();
   v[NV - 1] = a1.total();
   double t[NV];
-  if (reduce_last<NV>(v, ra.partials, ra.counter, t) && threadIdx.x == 0)
+  if (reduce_last(v, ra.partials, ra.counter, t) && threadIdx.x == 0)
     epilogue<NV>(epi, t, ra.ks, ra.hist, ra.tol, 0, 0);
 }
 
@@ -547,9 +566,9 @@ __global__ void __launch_bounds__(kRedThreads) k_pdot(Ix ix, const cpx<T>* __res
     const cpx<T> u = a[e], v = b[e];
     a0.add(pweight<T>(kx, ix.h0) * (u.x * v.x + u.y * v.y));
   }
-  double v[1] = {a0.total()};
+  const typename Acc<T>::Sum v[1] = {a0.total()};
   double t[1];
-  if (reduce_last<1>(v, ra.partials, ra.counter, t) && threadIdx.x == 0) epilogue<1>(EPI_NORM, t, ra.ks, ra.hist, ra.tol, 0, 0);
+  if (reduce_last(v, ra.partials, ra.counter, t) && threadIdx.x == 0) epilogue<1>(EPI_NORM, t, ra.ks, ra.hist, ra.tol, 0, 0);
 }
 
 // r = b - q and |r|^2 (weighted) -> ks->rr, accumulated like k_norms
@@ -564,9 +583,9 @@ __global__ void __launch_bounds__(kRedThreads) k_sub_norm(Ix ix, const cpx<T>* _
     r[e] = rv;
     a1.add(pweight<T>(kx, ix.h0) * (rv.x * rv.x + rv.y * rv.y));
   }
-  double v[1] = {a1.total()};
+  const typename Acc<T>::Sum v[1] = {a1.total()};
   double t[1];
-  if (reduce_last<1>(v, ra.partials, ra.counter, t) && threadIdx.x == 0) epilogue<1>(EPI_NORM, t, ra.ks, ra.hist, ra.tol, 0, 0);
+  if (reduce_last(v, ra.partials, ra.counter, t) && threadIdx.x == 0) epilogue<1>(EPI_NORM, t, ra.ks, ra.hist, ra.tol, 0, 0);
 }
 
 // RMR: x += alpha S r, r -= alpha w; reduce [rr]
@@ -589,9 +608,9 @@ __global__ void __launch_bounds__(kRedThreads) k_rmr_update(Ix ix, cpx<T>* __res
     r[e] = rv;
     a0.add(w * (rv.x * rv.x + rv.y * rv.y));
   }
-  double v[1] = {a0.total()};
+  const typename Acc<T>::Sum v[1] = {a0.total()};
   double t[1];
-  if (reduce_last<1>(v, ra.partials, ra.counter, t) && threadIdx.x == 0)
+  if (reduce_last(v, ra.partials, ra.counter, t) && threadIdx.x == 0)
     epilogue<1>(EPI_RMR_UPDATE, t, ra.ks, ra.hist, ra.tol, 0, 0);
 }
 
@@ -624,11 +643,11 @@ __global__ void __launch_bounds__(kRedThreads) k_gm_mdot(Ix ix, const cpx<T>* __
     for (int i = 0; i < NB; ++i)
       if (i < nv) a[i].dot(wv, V[(size_t)(off + i) * ix.len + e]);
   }
-  double v[NB];
+  typename Acc<T>::Sum v[NB];
 #pragma unroll
   for (int i = 0; i < NB; ++i) v[i] = a[i].total();
   double t[NB];
-  if (reduce_last<NB>(v, ra.partials, ra.counter, t) && threadIdx.x == 0)
+  if (reduce_last(v, ra.partials, ra.counter, t) && threadIdx.x == 0)
     epilogue<NB>(epi, t, ra.ks, ra.hist, ra.tol, off, j);
 }
 
@@ -655,11 +674,11 @@ __global__ void __launch_bounds__(kRedThreads) k_gm_step(Ix ix, cpx<T>* __restri
     for (int i = 0; i < NB; ++i)
       if (i < nv) a[i].dot(wv, vv[i]);
   }
-  double v[NB];
+  typename Acc<T>::Sum v[NB];
 #pragma unroll
   for (int i = 0; i < NB; ++i) v[i] = a[i].total();
   double t[NB];
-  if (reduce_last<NB>(v, ra.partials, ra.counter, t) && threadIdx.x == 0)
+  if (reduce_last(v, ra.partials, ra.counter, t) && threadIdx.x == 0)
     epilogue<NB>(EPI_GM_H2, t, ra.ks, ra.hist, ra.tol, 0, nv - 1);
 }
 
@@ -687,9 +706,9 @@ __global__ void __launch_bounds__(kRedThreads) k_gm_maxpy(Ix ix, cpx<T>* __restr
     a0.dot(scal(wv, pweight<T>(kx, ix.h0)), wv);
   }
   if (!with_norm) return;
-  double v[1] = {a0.total()};
+  const typename Acc<T>::Sum v[1] = {a0.total()};
   double t[1];
-  if (reduce_last<1>(v, ra.partials, ra.counter, t) && threadIdx.x == 0)
+  if (reduce_last(v, ra.partials, ra.counter, t) && threadIdx.x == 0)
     epilogue<1>(EPI_GM_NORM, t, ra.ks, ra.hist, ra.tol, 0, j);
 }
 
@@ -745,14 +764,20 @@ static void gm_orthogonalise(const SpecSystem& sys, cpx<T>* w, const cpx<T>* V, 
 __global__ void __launch_bounds__(32) k_gm_solve(KState* ks) {
   pdl_wait();
   if (ks->done) return;
-  __shared__ double tri[kMaxRestart * kMaxRestart], g[kMaxRestart];
+  __shared__ double tri[kMaxRestart * kMaxRestart], g[kMaxRestart], inv[kMaxRestart];
   const int k = ks->k, m = ks->m, lane = threadIdx.x;
   for (int l = 0; l < k; ++l)
     for (int i = lane; i <= l; i += 32) tri[i + l * kMaxRestart] = ks->H[i + (size_t)l * (m + 1)];
-  for (int i = lane; i < k; i += 32) g[i] = ks->gv[i];
+  __syncwarp();
+  for (int i = lane; i < k; i += 32) {
+    g[i] = ks->gv[i];
+    inv[i] = 1.0 / tri[i + i * kMaxRestart];
+  }
   __syncwarp();
   for (int l = k - 1; l >= 0; --l) {
-    const double y = g[l] / tri[l + l * kMaxRestart];
+    // g / H by the reciprocal and one correction (a division takes ~600 cycles, the three products 200)
+    const double h = tri[l + l * kMaxRestart], y0 = g[l] * inv[l];
+    const double y = isfinite(y0) ? fma(fma(-h, y0, g[l]), inv[l], y0) : g[l] / h;
     __syncwarp();
     for (int i = lane; i < l; i += 32) g[i] -= tri[i + l * kMaxRestart] * y;
     if (lane == 0) ks->y[l] = y;
