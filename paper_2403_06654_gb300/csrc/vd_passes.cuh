@@ -110,11 +110,12 @@ void tune_save();                    // write the table to $VD_TUNE_FILE (if set
 void ensure_smem(const void* func, size_t smem);
 int sm_count();
 
-// the float and double passes of any length (vd_wide.cuh): W / L lines per block, powers of two
+// the float and double passes of any length (vd_wide.cuh): W / L lines per block, powers of two; the
+// transforms / components shared out over `groups` blocks per tile
 template <typename T>
-void wide_axis(const AxisProg& P, int dir, const GridDesc& g, const void* tw, int W, cudaStream_t st);
+void wide_axis(const AxisProg& P, int dir, const GridDesc& g, const void* tw, int W, int groups, cudaStream_t st);
 template <typename T>
-void wide_xpass(const XProg& P, const GridDesc& g, const void* tw, int L, cudaStream_t st);
+void wide_xpass(const XProg& P, const GridDesc& g, const void* tw, int L, int groups, cudaStream_t st);
 // the plans of length n in every radix class, their tables at tw_off
 bool make_wide_plans(int n, int tw_off, WidePlan p[kWideClasses]);
 // The radix class of a pass over a field of ncplx points.  Wide radices make fewer trips through

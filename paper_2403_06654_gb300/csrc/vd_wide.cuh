@@ -174,7 +174,8 @@ __global__ void __launch_bounds__(kWideThreads, (sizeof(T) == 8 ? 2 : 3))
   if (P.done && *P.done) return;
   __syncthreads();   // the tables are complete
 
-  for (int t = 0; t < P.nxf; ++t) {
+  // (blocks of one y index take every gridDim.y-th transform: independent ones only, see split_axis)
+  for (int t = blockIdx.y; t < P.nxf; t += gridDim.y) {
     const Xf xf = P.xf[t];
     const cpx<T>* src = reinterpret_cast<const cpx<T>*>(P.in[xf.src]);
     cpx<T>* dst = reinterpret_cast<cpx<T>*>(P.out[xf.dst]);
@@ -212,7 +213,7 @@ __global__ void __launch_bounds__(kWideThreads, (sizeof(T) == 8 ? 2 : 3))
       continue;
     }
     // an even number of stages ends reading A, which the next transform's first stage writes
-    if (t > 0 && !(nst & 1)) __syncthreads();
+    if (t >= (int)gridDim.y && !(nst & 1)) __syncthreads();
     auto first_stage = [&](auto rc) {
       constexpr int R = decltype(rc)::value;
       const int nb = n / R;
@@ -374,7 +375,7 @@ __global__ void __launch_bounds__(kWideThreads, (sizeof(T) == 8 ? 2 : 3))
   pdl_wait();
   if (P.done && *P.done) return;
 
-  for (int c = 0; c < P.ncomp; ++c) {
+  for (int c = blockIdx.y; c < P.ncomp; c += gridDim.y) {
     __syncthreads();   // the tables are complete; the previous component's buffers are free
     cpx<T>*cur = A, *oth = B;
     if constexpr (MODE != 1) {
@@ -565,25 +566,27 @@ inline int wide_tpl(const WidePlan& pl, int W) {
 }
 
 template <typename T, int S>
-static void wide_axis_launch(const AxisProg& P, const GridDesc& g, const cpx<T>* tw, int W, cudaStream_t st) {
+static void wide_axis_launch(const AxisProg& P, const GridDesc& g, const cpx<T>* tw, int W, int groups,
+                             cudaStream_t st) {
   const int cls = wide_class(sizeof(T), (long long)g.ncplx);
   const WidePlan& pl = (P.axis == 2 ? g.wz : g.wy)[cls];
   const long long lines = (long long)g.h0 * (P.axis == 2 ? g.n1 : g.n2);
   const int tpl = wide_tpl(pl, W);
   const size_t smem = wide_axis_smem(pl, W, sizeof(T));
   ensure_smem(reinterpret_cast<const void*>(k_axis_w<T, S>), smem);
-  pdl_launch(k_axis_w<T, S>, (unsigned)((lines + W - 1) / W), W * tpl, smem, st, P, g, tw, wide_log2(W), tpl,
+  pdl_launch(k_axis_w<T, S>, dim3((unsigned)((lines + W - 1) / W), groups), W * tpl, smem, st, P, g, tw, wide_log2(W), tpl,
                                                                               wide_pad_shift(pl), cls);
 }
 
 template <typename T>
-void wide_axis(const AxisProg& P, int dir, const GridDesc& g, const void* tw, int W, cudaStream_t st) {
-  if (dir < 0) wide_axis_launch<T, -1>(P, g, reinterpret_cast<const cpx<T>*>(tw), W, st);
-  else wide_axis_launch<T, 1>(P, g, reinterpret_cast<const cpx<T>*>(tw), W, st);
+void wide_axis(const AxisProg& P, int dir, const GridDesc& g, const void* tw, int W, int groups, cudaStream_t st) {
+  if (dir < 0) wide_axis_launch<T, -1>(P, g, reinterpret_cast<const cpx<T>*>(tw), W, groups, st);
+  else wide_axis_launch<T, 1>(P, g, reinterpret_cast<const cpx<T>*>(tw), W, groups, st);
 }
 
 template <typename T, int MODE>
-static void wide_xpass_launch(const XProg& P, const GridDesc& g, const cpx<T>* tw, int L, cudaStream_t st) {
+static void wide_xpass_launch(const XProg& P, const GridDesc& g, const cpx<T>* tw, int L, int groups,
+                              cudaStream_t st) {
   const int cls = wide_class(sizeof(T), (long long)g.ncplx);
   const WidePlan& pl = g.wx[cls];
   const int ps = wide_pad_shift(pl), ls = wide_line_stride(pl);
@@ -593,15 +596,15 @@ static void wide_xpass_launch(const XProg& P, const GridDesc& g, const cpx<T>* t
   for (int s = 0; s < pl.nst; ++s) nb = std::max(nb, pl.n / pl.rad[s]);
   const int threads = std::min(kWideThreads, (int)std::max<long long>(32, ((long long)L * nb + 31) / 32 * 32));
   ensure_smem(reinterpret_cast<const void*>(k_xpass_w<T, MODE>), smem);
-  pdl_launch(k_xpass_w<T, MODE>, (unsigned)((lines + L - 1) / L), threads, smem, st, P, g, tw, wide_log2(L), ps, ls, cls);
+  pdl_launch(k_xpass_w<T, MODE>, dim3((unsigned)((lines + L - 1) / L), groups), threads, smem, st, P, g, tw, wide_log2(L), ps, ls, cls);
 }
 
 template <typename T>
-void wide_xpass(const XProg& P, const GridDesc& g, const void* tw, int L, cudaStream_t st) {
+void wide_xpass(const XProg& P, const GridDesc& g, const void* tw, int L, int groups, cudaStream_t st) {
   const cpx<T>* twp = reinterpret_cast<const cpx<T>*>(tw);
-  if (P.mode == 0) wide_xpass_launch<T, 0>(P, g, twp, L, st);
-  else if (P.mode == 1) wide_xpass_launch<T, 1>(P, g, twp, L, st);
-  else wide_xpass_launch<T, 2>(P, g, twp, L, st);
+  if (P.mode == 0) wide_xpass_launch<T, 0>(P, g, twp, L, groups, st);
+  else if (P.mode == 1) wide_xpass_launch<T, 1>(P, g, twp, L, groups, st);
+  else wide_xpass_launch<T, 2>(P, g, twp, L, groups, st);
 }
 
 }  // namespace vd

@@ -2,6 +2,6 @@
 #include "vd_wide.cuh"
 
 namespace vd {
-template void wide_axis<float>(const AxisProg&, int, const GridDesc&, const void*, int, cudaStream_t);
-template void wide_xpass<float>(const XProg&, const GridDesc&, const void*, int, cudaStream_t);
+template void wide_axis<float>(const AxisProg&, int, const GridDesc&, const void*, int, int, cudaStream_t);
+template void wide_xpass<float>(const XProg&, const GridDesc&, const void*, int, int, cudaStream_t);
 }  // namespace vd
