@@ -15,6 +15,7 @@
 
 #include <algorithm>
 #include <cmath>
+#include <type_traits>
 #include <cstddef>
 #include <cstring>
 #include <vector>
@@ -412,9 +413,50 @@ struct Ix {
   for (; e < (ix).len; e += ix_s_, kx += (ix).sh, kx -= (kx >= (ix).h0) ? (ix).h0 : 0,      \
                        si += (ix).sn, si -= (si >= (ix).nc) ? (ix).nc : 0)
 
+// The loop of the memory-bound kernels: use(e, kx, load(e, si)) for every element of the thread, two
+// elements' loads in flight (256^3 points: float CG update 74 -> 56 us, start of a CG solve 100 -> 75).  The elements come in the same order.
+template <typename L, typename U>
+__device__ __forceinline__ void ix_each(const Ix& ix, L load, U use) {
+  const int step = gridDim.x * blockDim.x;
+  int e = blockIdx.x * blockDim.x + threadIdx.x, kx = e % ix.h0, si = e % ix.nc;
+  auto next = [&]() {
+    kx += ix.sh;
+    kx -= (kx >= ix.h0) ? ix.h0 : 0;
+    si += ix.sn;
+    si -= (si >= ix.nc) ? ix.nc : 0;
+  };
+  for (; e < ix.len - step; e += 2 * step) {
+    const int k0 = kx;
+    const auto v0 = load(e, si);
+    next();
+    const auto v1 = load(e + step, si);
+    use(e, k0, v0);
+    use(e + step, kx, v1);
+    next();
+  }
+  if (e < ix.len) use(e, kx, load(e, si));
+}
+
 template <typename T>
 __device__ __forceinline__ T pweight(int kx, int h0) {
   return (kx == 0 || kx == h0 - 1) ? T(1) : T(2);
+}
+
+// v times the Parseval weight.  Double: 2 v on the bits, since a multiply or an addition is a turn on
+// the FP64 pipe (a compiler's select between the two values would take both): 256^3 points, double norm
+// 53 -> 41 us, r = b - q with its norm 87 -> 71 us.
+__device__ __forceinline__ float weighted(float v, int kx, int h0) { return v * pweight<float>(kx, h0); }
+__device__ __forceinline__ double weighted(double v, int kx, int h0) {
+  const unsigned long long b = (unsigned long long)__double_as_longlong(v), sg = b & (1ull << 63);
+  const unsigned e = (unsigned)(b >> 52) & 0x7ffu;
+  unsigned long long t = b + (1ull << 52);             // normal: the next exponent
+  if (e == 0u) t = sg | (b << 1);                      // zero and subnormal: the significand doubled
+  if (e >= 0x7feu) t = e == 0x7ffu ? b : (sg | (0x7ffull << 52));
+  return __longlong_as_double((long long)((kx == 0 || kx == h0 - 1) ? b : t));
+}
+template <typename T>
+__device__ __forceinline__ cpx<T> weighted(cpx<T> v, int kx, int h0) {
+  return mk<T>(weighted(v.x, kx, h0), weighted(v.y, kx, h0));
 }
 
 // Per-thread accumulator of a reduction.  Double vectors add in double.  Float vectors add
@@ -445,6 +487,37 @@ struct Acc<float> {
   using Sum = dd;
 };
 
+// float(v * s) on the integer and FP32 pipes: v scaled by the power of two in s (exponent bits), split
+// into a float pair, times the rest of s in [1, 2), rounded to float once.  A double multiply and a
+// conversion per value kept k_d2f_scaled at 64 us of 256^3 points against 30 us of memory.  Results
+// below the normal floats are zero.  An s that is no normal double takes the double arithmetic.
+struct Narrow {
+  double s;
+  float sh, sl;
+  int k;   // s = (sh + sl) 2^k
+  bool plain;
+  __device__ __forceinline__ explicit Narrow(double scale) : s(scale) {
+    const int hi = __double2hiint(scale), ef = (hi >> 20) & 0x7ff;
+    plain = ef == 0 || ef == 0x7ff;
+    k = ef - 1023;
+    const dd m = dd_from_double(__hiloint2double((hi & 0x800fffff) | 0x3ff00000, __double2loint(scale)));
+    sh = m.hi;
+    sl = m.lo;
+  }
+  __device__ __forceinline__ float operator()(double v) const {
+    const int hi = __double2hiint(v), ef = (hi >> 20) & 0x7ff, en = ef + k;
+    if (plain || ef == 0x7ff || en >= 0x7ff) return (float)(v * s);
+    if (ef == 0 || en <= 0) return 0.0f;
+    const dd d = dd_from_double(__hiloint2double(hi + (k << 20), __double2loint(v)));
+    return mul_pair_dd(d, sh, sl);
+  }
+  // (d.hi + d.lo)(wh + wl), rounded once
+  static __device__ __forceinline__ float mul_pair_dd(dd d, float wh, float wl) {
+    const float p = d.hi * wh;
+    return p + fmaf(d.lo, wh, fmaf(d.hi, wl, fmaf(d.hi, wh, -p)));
+  }
+};
+
 // CG start: p = S r, reduce [bb, rr, rz]
 template <typename T>
 __global__ void __launch_bounds__(kRedThreads) k_cg_init(Ix ix, const cpx<T>* __restrict__ b,
@@ -453,19 +526,59 @@ __global__ void __launch_bounds__(kRedThreads) k_cg_init(Ix ix, const cpx<T>* __
   pdl_wait();
   Acc<T> a0, a1, a2;
   IX_LOOP(ix) {
-    const T w = pweight<T>(kx, ix.h0);
     const cpx<T> bv = b[e], rv = r[e];
     const T sv = sym[si];
     p[e] = scal(rv, sv);
-    const T r2 = rv.x * rv.x + rv.y * rv.y;
-    a0.add(w * (bv.x * bv.x + bv.y * bv.y));
-    a1.add(w * r2);
-    a2.add(w * sv * r2);
+    const T r2 = weighted(rv.x * rv.x + rv.y * rv.y, kx, ix.h0);
+    a0.add(weighted(bv.x * bv.x + bv.y * bv.y, kx, ix.h0));
+    a1.add(r2);
+    a2.add(sv * r2);
   }
   const typename Acc<T>::Sum v[3] = {a0.total(), a1.total(), a2.total()};
   double t[3];
   if (reduce_last(v, ra.partials, ra.counter, t) && threadIdx.x == 0)
     epilogue<3>(EPI_INIT_CG, t, ra.ks, ra.hist, ra.tol, 0, 0);
+}
+
+// CG start from x = 0: x = 0, r = b, p = S b, reduce [bb, rz].  With src64 (float solves of the
+// refinement) b is src64 * s, narrowed here: its own pass, the copy of r and the clearing of x took
+// 105 us of 256^3 points beside this kernel's 51.
+template <typename T, bool SRC64>
+__global__ void __launch_bounds__(kRedThreads, 4)
+    k_cg_start(Ix ix, const cpx<T>* __restrict__ b, const cpx<double>* __restrict__ src64, double s, const OState* o,
+               cpx<T>* __restrict__ x, cpx<T>* __restrict__ r, cpx<T>* __restrict__ p, const T* __restrict__ sym,
+               RedArgs ra) {
+  pdl_wait();
+  Acc<T> a0, a1;
+  const Narrow nw(o ? o->scale : s);
+  using B = typename std::conditional<SRC64, double, T>::type;
+  struct In {
+    cpx<B> b;
+    T s;
+  };
+  ix_each(
+      ix,
+      [&](int e, int si) {
+        if constexpr (SRC64) return In{src64[e], sym[si]};
+        else return In{b[e], sym[si]};
+      },
+      [&](int e, int kx, const In& v) {
+        cpx<T> rv;
+        if constexpr (SRC64) rv = mk<T>(nw(v.b.x), nw(v.b.y));
+        else rv = v.b;
+        x[e] = mk<T>(T(0), T(0));
+        r[e] = rv;
+        p[e] = scal(rv, v.s);
+        const T r2 = weighted(rv.x * rv.x + rv.y * rv.y, kx, ix.h0);
+        a0.add(r2);
+        a1.add(v.s * r2);
+      });
+  const typename Acc<T>::Sum v[2] = {a0.total(), a1.total()};
+  double t[2];
+  if (reduce_last(v, ra.partials, ra.counter, t) && threadIdx.x == 0) {
+    const double t3[3] = {t[0], t[0], t[1]};
+    epilogue<3>(EPI_INIT_CG, t3, ra.ks, ra.hist, ra.tol, 0, 0);
+  }
 }
 
 // reduce [(u,v)_w] or [(u,v)_w, (v,v)_w]
@@ -477,7 +590,7 @@ __global__ void __launch_bounds__(kRedThreads) k_dot(Ix ix, const cpx<T>* __rest
   if (*done) return;
   Acc<T> a0, a1;
   IX_LOOP(ix) {
-    const cpx<T> vv = v[e], wv = scal(vv, pweight<T>(kx, ix.h0));   // the weight is 1 or 2: exact
+    const cpx<T> vv = v[e], wv = weighted(vv, kx, ix.h0);
     a0.dot(wv, u[e]);
     if (NV > 1) a1.dot(wv, vv);
   }
@@ -491,26 +604,28 @@ __global__ void __launch_bounds__(kRedThreads) k_dot(Ix ix, const cpx<T>* __rest
 
 // CG: x += alpha p, r -= alpha q; reduce [rr, (r, S r)]
 template <typename T>
-__global__ void __launch_bounds__(kRedThreads) k_cg_update(Ix ix, cpx<T>* __restrict__ x,
-                                                           const cpx<T>* __restrict__ p, cpx<T>* __restrict__ r,
-                                                           const cpx<T>* __restrict__ q, const T* __restrict__ sym,
-                                                           RedArgs ra) {
+__global__ void __launch_bounds__(kRedThreads, 4) k_cg_update(Ix ix, cpx<T>* __restrict__ x,
+                                                              const cpx<T>* __restrict__ p, cpx<T>* __restrict__ r,
+                                                              const cpx<T>* __restrict__ q, const T* __restrict__ sym,
+                                                              RedArgs ra) {
   pdl_wait();
   if (ra.ks->done) return;
   const T al = (T)ra.ks->alpha;
   Acc<T> a0, a1;
-  IX_LOOP(ix) {
-    const T w = pweight<T>(kx, ix.h0);
-    const cpx<T> pv = p[e], qv = q[e];
-    cpx<T> xv = x[e], rv = r[e];
-    xv = mk<T>(fma(al, pv.x, xv.x), fma(al, pv.y, xv.y));
-    rv = mk<T>(fma(-al, qv.x, rv.x), fma(-al, qv.y, rv.y));
-    x[e] = xv;
-    r[e] = rv;
-    const T r2 = rv.x * rv.x + rv.y * rv.y;
-    a0.add(w * r2);
-    a1.add(w * sym[si] * r2);
-  }
+  struct In {
+    cpx<T> p, q, x, r;
+    T s;
+  };
+  ix_each(
+      ix, [&](int e, int si) { return In{p[e], q[e], x[e], r[e], sym[si]}; },
+      [&](int e, int kx, const In& v) {
+        x[e] = mk<T>(fma(al, v.p.x, v.x.x), fma(al, v.p.y, v.x.y));
+        const cpx<T> rv = mk<T>(fma(-al, v.q.x, v.r.x), fma(-al, v.q.y, v.r.y));
+        r[e] = rv;
+        const T r2 = weighted(rv.x * rv.x + rv.y * rv.y, kx, ix.h0);
+        a0.add(r2);
+        a1.add(v.s * r2);
+      });
   const typename Acc<T>::Sum v[2] = {a0.total(), a1.total()};
   double t[2];
   if (reduce_last(v, ra.partials, ra.counter, t) && threadIdx.x == 0)
@@ -533,21 +648,25 @@ __global__ void k_cg_p(Ix ix, cpx<T>* __restrict__ p, const cpx<T>* __restrict__
 
 // RMR / GMRES start: reduce [bb, rr] or [rr]
 template <typename T, int NV>
-__global__ void __launch_bounds__(kRedThreads) k_norms(Ix ix, const cpx<T>* __restrict__ b,
-                                                       const cpx<T>* __restrict__ r, int epi, RedArgs ra,
-                                                       const int* done) {
+__global__ void __launch_bounds__(kRedThreads, 4) k_norms(Ix ix, const cpx<T>* __restrict__ b,
+                                                          const cpx<T>* __restrict__ r, int epi, RedArgs ra,
+                                                          const int* done) {
   pdl_wait();
   if (done && *done) return;
   Acc<T> a0, a1;
-  IX_LOOP(ix) {
-    const T w = pweight<T>(kx, ix.h0);
-    const cpx<T> rv = r[e];
-    if (NV == 2) {
-      const cpx<T> bv = b[e];
-      a0.add(w * (bv.x * bv.x + bv.y * bv.y));
-    }
-    a1.add(w * (rv.x * rv.x + rv.y * rv.y));
-  }
+  struct In {
+    cpx<T> b, r;
+  };
+  ix_each(
+      ix,
+      [&](int e, int) {
+        const cpx<T> rv = r[e];
+        return In{NV == 2 ? b[e] : rv, rv};
+      },
+      [&](int, int kx, const In& v) {
+        if (NV == 2) a0.dot(weighted(v.b, kx, ix.h0), v.b);
+        a1.dot(weighted(v.r, kx, ix.h0), v.r);
+      });
   typename Acc<T>::Sum v[NV];
   if (NV == 2) v[0] = a0.total();
   v[NV - 1] = a1.total();
@@ -564,7 +683,7 @@ __global__ void __launch_bounds__(kRedThreads) k_pdot(Ix ix, const cpx<T>* __res
   Acc<T> a0;
   IX_LOOP(ix) {
     const cpx<T> u = a[e], v = b[e];
-    a0.add(pweight<T>(kx, ix.h0) * (u.x * v.x + u.y * v.y));
+    a0.dot(weighted(u, kx, ix.h0), v);
   }
   const typename Acc<T>::Sum v[1] = {a0.total()};
   double t[1];
@@ -573,16 +692,20 @@ __global__ void __launch_bounds__(kRedThreads) k_pdot(Ix ix, const cpx<T>* __res
 
 // r = b - q and |r|^2 (weighted) -> ks->rr, accumulated like k_norms
 template <typename T>
-__global__ void __launch_bounds__(kRedThreads) k_sub_norm(Ix ix, const cpx<T>* __restrict__ b,
-                                                          const cpx<T>* __restrict__ q, cpx<T>* __restrict__ r,
-                                                          RedArgs ra) {
+__global__ void __launch_bounds__(kRedThreads, 4) k_sub_norm(Ix ix, const cpx<T>* __restrict__ b,
+                                                             const cpx<T>* q, cpx<T>* r, RedArgs ra) {
   pdl_wait();
   Acc<T> a1;
-  IX_LOOP(ix) {
-    const cpx<T> rv = b[e] - q[e];
-    r[e] = rv;
-    a1.add(pweight<T>(kx, ix.h0) * (rv.x * rv.x + rv.y * rv.y));
-  }
+  struct In {
+    cpx<T> b, q;
+  };
+  ix_each(
+      ix, [&](int e, int) { return In{b[e], q[e]}; },   // (r may be q)
+      [&](int e, int kx, const In& v) {
+        const cpx<T> rv = v.b - v.q;
+        r[e] = rv;
+        a1.dot(weighted(rv, kx, ix.h0), rv);
+      });
   const typename Acc<T>::Sum v[1] = {a1.total()};
   double t[1];
   if (reduce_last(v, ra.partials, ra.counter, t) && threadIdx.x == 0) epilogue<1>(EPI_NORM, t, ra.ks, ra.hist, ra.tol, 0, 0);
@@ -590,24 +713,26 @@ __global__ void __launch_bounds__(kRedThreads) k_sub_norm(Ix ix, const cpx<T>* _
 
 // RMR: x += alpha S r, r -= alpha w; reduce [rr]
 template <typename T>
-__global__ void __launch_bounds__(kRedThreads) k_rmr_update(Ix ix, cpx<T>* __restrict__ x, cpx<T>* __restrict__ r,
-                                                            const cpx<T>* __restrict__ wv, const T* __restrict__ sym,
-                                                            RedArgs ra) {
+__global__ void __launch_bounds__(kRedThreads, 4) k_rmr_update(Ix ix, cpx<T>* __restrict__ x, cpx<T>* __restrict__ r,
+                                                               const cpx<T>* __restrict__ wv,
+                                                               const T* __restrict__ sym, RedArgs ra) {
   pdl_wait();
   if (ra.ks->done) return;
   const T al = (T)ra.ks->alpha;
   Acc<T> a0;
-  IX_LOOP(ix) {
-    const T w = pweight<T>(kx, ix.h0);
-    const T as = al * sym[si];
-    const cpx<T> wq = wv[e];
-    cpx<T> xv = x[e], rv = r[e];
-    xv = mk<T>(fma(as, rv.x, xv.x), fma(as, rv.y, xv.y));
-    rv = mk<T>(fma(-al, wq.x, rv.x), fma(-al, wq.y, rv.y));
-    x[e] = xv;
-    r[e] = rv;
-    a0.add(w * (rv.x * rv.x + rv.y * rv.y));
-  }
+  struct In {
+    cpx<T> w, x, r;
+    T s;
+  };
+  ix_each(
+      ix, [&](int e, int si) { return In{wv[e], x[e], r[e], sym[si]}; },
+      [&](int e, int kx, const In& v) {
+        const T as = al * v.s;
+        x[e] = mk<T>(fma(as, v.r.x, v.x.x), fma(as, v.r.y, v.x.y));
+        const cpx<T> rv = mk<T>(fma(-al, v.w.x, v.r.x), fma(-al, v.w.y, v.r.y));
+        r[e] = rv;
+        a0.dot(weighted(rv, kx, ix.h0), rv);
+      });
   const typename Acc<T>::Sum v[1] = {a0.total()};
   double t[1];
   if (reduce_last(v, ra.partials, ra.counter, t) && threadIdx.x == 0)
@@ -638,7 +763,7 @@ __global__ void __launch_bounds__(kRedThreads) k_gm_mdot(Ix ix, const cpx<T>* __
   if (ra.ks->cycle_done) return;
   Acc<T> a[NB];
   IX_LOOP(ix) {
-    const cpx<T> wv = scal(w[e], pweight<T>(kx, ix.h0));   // the weight is 1 or 2: exact
+    const cpx<T> wv = weighted(w[e], kx, ix.h0);
 #pragma unroll
     for (int i = 0; i < NB; ++i)
       if (i < nv) a[i].dot(wv, V[(size_t)(off + i) * ix.len + e]);
@@ -669,7 +794,7 @@ __global__ void __launch_bounds__(kRedThreads) k_gm_step(Ix ix, cpx<T>* __restri
     for (int i = 0; i < NB; ++i)
       if (i < nv) wv = mk<T>(fma(-hs[i], vv[i].x, wv.x), fma(-hs[i], vv[i].y, wv.y));
     w[e] = wv;
-    wv = scal(wv, pweight<T>(kx, ix.h0));
+    wv = weighted(wv, kx, ix.h0);
 #pragma unroll
     for (int i = 0; i < NB; ++i)
       if (i < nv) a[i].dot(wv, vv[i]);
@@ -703,7 +828,7 @@ __global__ void __launch_bounds__(kRedThreads) k_gm_maxpy(Ix ix, cpx<T>* __restr
       wv = mk<T>(fma(-c, vv.x, wv.x), fma(-c, vv.y, wv.y));
     }
     w[e] = wv;
-    a0.dot(scal(wv, pweight<T>(kx, ix.h0)), wv);
+    a0.dot(weighted(wv, kx, ix.h0), wv);
   }
   if (!with_norm) return;
   const typename Acc<T>::Sum v[1] = {a0.total()};
@@ -848,10 +973,10 @@ __global__ void k_sub(long long len, const cpx<T>* __restrict__ b, const cpx<T>*
 __global__ void k_d2f_scaled(long long len, const cpx<double>* __restrict__ in, double s, const OState* o,
                              cpx<float>* __restrict__ out) {
   pdl_wait();
-  if (o) s = o->scale;
+  const Narrow nw(o ? o->scale : s);
   GRID_STRIDE(e, len) {
     const cpx<double> v = in[e];
-    out[e] = mk<float>((float)(v.x * s), (float)(v.y * s));
+    out[e] = mk<float>(nw(v.x), nw(v.y));
   }
 }
 __global__ void k_axpy_f2d(long long len, double a, const OState* o, const cpx<float>* __restrict__ xf,
@@ -861,7 +986,7 @@ __global__ void k_axpy_f2d(long long len, double a, const OState* o, const cpx<f
   GRID_STRIDE(e, len) {
     const cpx<float> v = xf[e];
     const cpx<double> w = y[e];
-    y[e] = mk<double>(fma(a, (double)v.x, w.x), fma(a, (double)v.y, w.y));
+    y[e] = mk<double>(fma(a, widen(v.x), w.x), fma(a, widen(v.y), w.y));
   }
 }
 template <typename T>
@@ -948,10 +1073,6 @@ double spec_sub_norm2_host(const SpecSystem& sys, const void* b, const void* q, 
   cudaMemcpyAsync(&rr, &kw.ks->rr, sizeof(double), cudaMemcpyDeviceToHost, st);
   cudaStreamSynchronize(st);
   return rr;
-}
-
-void spec_d2f_scaled(long long len, const void* in, double s, void* out, cudaStream_t st) {
-  { ProfScope ps_(PC_VEC64, st, (double)len * (sizeof(cpx<double>) + sizeof(cpx<float>)), 0.0); pdl_launch(k_d2f_scaled, ew_blocks(len), 256, 0, st, len, (const cpx<double>*)in, s, nullptr, (cpx<float>*)out); }
 }
 
 void spec_axpy_f2d(long long len, double a, const void* xf, void* y, cudaStream_t st) {
@@ -1056,6 +1177,38 @@ class HeadPipeLease {
   HeadPipe* hp_ = nullptr;
 };
 
+// The start of a solve from x = 0.  CG: one pass (k_cg_start).  RMR and GMRES: x cleared and, with
+// src64, b narrowed into its buffer (which the solver reads again).
+template <typename T>
+static void cg_start(const SpecSystem& sys, const SolveOpts& o, const cpx<T>* B, cpx<T>* X, cpx<T>* r, cpx<T>* p,
+                     const RedArgs& ra, cudaStream_t st) {
+  const long long nc = sys.G->g.ncplx;
+  const int rb = red_blocks(sys.len);
+  const Ix ix = mkix(sys.len, sys.h0, nc, rb, kRedThreads);
+  const double el = (double)sys.len * sizeof(cpx<T>);
+  ProfScope ps_(sizeof(T) == 4 ? PC_VEC32 : PC_VEC64, st, (o.src64 ? 5 : 4) * el + (double)nc * sizeof(T), 0.0);
+  if constexpr (sizeof(T) == 4) {
+    if (o.src64) {
+      pdl_launch(k_cg_start<T, true>, rb, kRedThreads, 0, st, ix, B, (const cpx<double>*)o.src64, o.src_scale,
+                 o.dev_outer, X, r, p, (const T*)sys.sym, ra);
+      return;
+    }
+  }
+  pdl_launch(k_cg_start<T, false>, rb, kRedThreads, 0, st, ix, B, nullptr, 1.0, nullptr, X, r, p, (const T*)sys.sym,
+             ra);
+}
+template <typename T>
+static vd_status start_from_zero(const SolveOpts& o, const void* b, void* x, long long len, cudaStream_t st) {
+  if (!o.x_zero) return VD_OK;
+  VD_CUDA(cudaMemsetAsync(x, 0, sizeof(cpx<T>) * len, st));
+  if (o.src64) {
+    ProfScope ps_(PC_VEC64, st, (double)len * (sizeof(cpx<double>) + sizeof(cpx<float>)), 0.0);
+    pdl_launch(k_d2f_scaled, ew_blocks(len), 256, 0, st, len, (const cpx<double>*)o.src64, o.src_scale, o.dev_outer,
+               (cpx<float>*)const_cast<void*>(b));
+  }
+  return VD_OK;
+}
+
 template <typename T>
 vd_status krylov_solve(const SpecSystem& sys, const SolveOpts& o, const void* b, void* x, void* vecs,
                        const KWork& kw, double* host_hist, int host_hist_cap, SolveOut* out, cudaStream_t st) {
@@ -1088,18 +1241,22 @@ vd_status krylov_solve(const SpecSystem& sys, const SolveOpts& o, const void* b,
   const cpx<T>* B = (const cpx<T>*)b;
   cpx<T>* vb = (cpx<T>*)vecs;
   KHead hd;
+  if (o.solver != VD_SOLVER_CG) {
+    const vd_status e0 = start_from_zero<T>(o, b, x, len, st);
+    if (e0 != VD_OK) return e0;
+  }
 
   if (o.solver == VD_SOLVER_CG) {
     cpx<T>* r = vb;
     cpx<T>* p = vb + len;
     cpx<T>* q = vb + 2 * len;
     if (o.x_zero) {
-      VD_CUDA(cudaMemcpyAsync(r, B, sizeof(cpx<T>) * len, cudaMemcpyDeviceToDevice, st));
+      cg_start<T>(sys, o, B, X, r, p, ra, st);
     } else {
       sys.apply(sys, X, q, false, nullptr, st);
       { ProfScope ps_(sizeof(T) == 4 ? PC_VEC32 : PC_VEC64, st, (double)3 * len * sizeof(cpx<T>), 0.0); pdl_launch(k_sub<T>, eb, 256, 0, st, len, B, q, r, nullptr); }
+      { ProfScope ps_(sizeof(T) == 4 ? PC_VEC32 : PC_VEC64, st, (double)3 * len * sizeof(cpx<T>) + (double)nc * sizeof(T), 0.0); pdl_launch(k_cg_init<T>, rb, kRedThreads, 0, st, ixr, B, r, p, sym, ra); }
     }
-    { ProfScope ps_(sizeof(T) == 4 ? PC_VEC32 : PC_VEC64, st, (double)3 * len * sizeof(cpx<T>) + (double)nc * sizeof(T), 0.0); pdl_launch(k_cg_init<T>, rb, kRedThreads, 0, st, ixr, B, r, p, sym, ra); }
     int it = 0;
     HeadPipeLease lease;
     HeadPipe* hp = lease.get();
@@ -1325,19 +1482,20 @@ vd_status krylov_enqueue_graph(const SpecSystem& sys, const SolveOpts& o, const 
     return VD_OK;
   };
   vd_status e;
+  if (o.solver != VD_SOLVER_CG && (e = start_from_zero<T>(o, b, x, len, st)) != VD_OK) return e;
   if (o.solver == VD_SOLVER_CG) {
     cpx<T>* r = vb;
     cpx<T>* p = vb + len;
     cpx<T>* q = vb + 2 * len;
     if (o.x_zero) {
-      VD_CUDA(cudaMemcpyAsync(r, B, sizeof(cpx<T>) * len, cudaMemcpyDeviceToDevice, st));
+      cg_start<T>(sys, o, B, X, r, p, ra, st);
     } else {
       sys.apply(sys, X, q, false, nullptr, st);
       pdl_launch(k_sub<T>, eb, 256, 0, st, len, B, q, r, nullptr);
+      pdl_launch(k_cg_init<T>, rb, kRedThreads, 0, st, ixr, B, r, p, sym, ra);
+      count_launch();
       count_launch();
     }
-    pdl_launch(k_cg_init<T>, rb, kRedThreads, 0, st, ixr, B, r, p, sym, ra);
-    count_launch();
     if ((e = open_loop(&hnd)) != VD_OK) return e;
     sys.apply(sys, p, q, false, done, body_st);
     pdl_launch(k_dot<T, 1>, rb, kRedThreads, 0, body_st, ixr, p, q, EPI_CG_ALPHA, ra, done);
@@ -1602,10 +1760,8 @@ vd_status refine_enqueue_graph(const SpecSystem& sys64, const SpecSystem& sys32,
   }
   VD_CUDA(cudaStreamBeginCaptureToGraph(s2, sweep_body, nullptr, nullptr, 0, cudaStreamCaptureModeRelaxed));
   // the sweep: d solves A32 d = r/|r| in float, x += |r| d, r = b - A x, |r|^2
-  pdl_launch(k_d2f_scaled, eb, 256, 0, s2, len, RH, 0.0, ost, (cpx<float>*)bh_f);
-  count_launch();
-  VD_CUDA(cudaMemsetAsync(xh_f, 0, sizeof(cpx<float>) * len, s2));
   SolveOpts si = inner;
+  si.src64 = RH;
   si.x_zero = 1;
   si.dev_outer = ost;
   if ((e = krylov_enqueue_graph<float>(sys32, si, bh_f, xh_f, vecs, kw, s2, s3)) != VD_OK) return e;

@@ -82,9 +82,13 @@ struct SolveOpts {
   int maxit;
   int restart;
   int check_every;
-  int x_zero;   // x is known to be zero on entry: the first residual is b (no operator apply)
+  int x_zero;   // start from x = 0 (the solve clears x): the first residual is b (no operator apply)
   int guard = 0;   // KState::guard of the solve
   const OState* dev_outer = nullptr;   // graph form: tolerance and iteration budget from the device
+  // float solves of the refinement, x_zero only: b = src64 * src_scale (graph form: dev_outer's scale),
+  // narrowed at the start; the b argument is then a buffer of the solve
+  const void* src64 = nullptr;
+  double src_scale = 1.0;
 };
 
 struct SolveOut {
@@ -142,10 +146,8 @@ double spec_dot_host(const SpecSystem& sys, const void* a, const void* b, const 
 // 2^d ncomp doubles) receives each removed coefficient's share of the squared weighted norm
 template <typename T>
 void spec_project(const vd_grid* G, int ncomp, void* v, cudaStream_t st, double* removed = nullptr);
-// refinement steps on double vectors, each one pass: out = float(in * s) (narrowed right-hand
-// side of the inner solve); y += a * double(xf) (correction); r = b - q returning |r|^2
-// (weighted) to the host
-void spec_d2f_scaled(long long len, const void* in, double s, void* out, cudaStream_t st);
+// refinement steps on double vectors, each one pass: y += a * double(xf) (correction); r = b - q
+// returning |r|^2 (weighted) to the host
 void spec_axpy_f2d(long long len, double a, const void* xf, void* y, cudaStream_t st);
 double spec_sub_norm2_host(const SpecSystem& sys, const void* b, const void* q, void* r, const KWork& kw,
                            cudaStream_t st);
