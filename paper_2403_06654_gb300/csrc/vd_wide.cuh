@@ -126,7 +126,8 @@ __device__ __forceinline__ T wide_kfac(const GridDesc& g, int a) {
 
 // Block: W = 2^lw lines side by side, tpl threads per line.  Shared memory: the twiddle table, one
 // (two stages) or two (more) tiles of W x n, and k~ of every index along the axis.
-template <typename T, int S>
+// PAD: rows of narrow tiles are padded (tiles of 128-byte rows need none).
+template <typename T, int S, bool PAD>
 __global__ void __launch_bounds__(kWideThreads, (sizeof(T) == 8 ? 2 : 3))
     k_axis_w(const __grid_constant__ AxisProg P, const __grid_constant__ GridDesc g, const cpx<T>* __restrict__ twg,
              int lw, int tpl, int ps, int cls) {
@@ -136,10 +137,10 @@ __global__ void __launch_bounds__(kWideThreads, (sizeof(T) == 8 ? 2 : 3))
   const int n = pl.n, nst = pl.nst, W = 1 << lw;
   cpx<T>* tw = reinterpret_cast<cpx<T>*>(smem_raw);
   cpx<T>* A = tw + n;
-  const int tile = W * (n + (n >> ps));
+  const int tile = W * (PAD ? n + (n >> ps) : n);
   cpx<T>* B = A + (nst > 2 ? tile : 0);
   T* katab = reinterpret_cast<T*>(B + tile);
-  auto at = [&](int j) { return (j + (j >> ps)) * W; };   // element j of a line (narrow tiles: padded rows)
+  auto at = [&](int j) { return (PAD ? j + (j >> ps) : j) << lw; };   // row of element j of the lines
   const T kfa = wide_kfac<T>(g, axis);
   for (int j = threadIdx.x; j < n; j += blockDim.x) {
     tw[j] = twg[pl.tw_off + j];
@@ -190,17 +191,6 @@ __global__ void __launch_bounds__(kWideThreads, (sizeof(T) == 8 ? 2 : 3))
       if (flags & MUL_SYM) c *= symarr[g0 + i * ls];
       if (flags & MUL_NEGK2) c *= -(ka * ka + kp2);
       return c;
-    };
-    auto put = [&](int i, cpx<T> v, cpx<T> prev) {   // row i of the output line
-      if (xf.post == MUL_IK && unit) {
-        v = mul_ik(v, katab[i]);
-      } else if (xf.post) {
-        v = scal(v, mult(xf.post, i, scale));
-        if (xf.post & MUL_IK) v = mul_i(v);
-      } else if (!unit) {
-        v = scal(v, scale);
-      }
-      dst[g0 + i * ls] = xf.first ? v : (prev + v);
     };
     if (xf.nofft) {
       if (ok)
@@ -275,20 +265,38 @@ __global__ void __launch_bounds__(kWideThreads, (sizeof(T) == 8 ? 2 : 3))
           }
         }
         dft_wide<T, S, R>(u);
-        if (ok) {
-          // partial sums (written by this thread) are read in batches ahead of the stores
+        if (!ok) continue;
+        // the multiplier of the output, the common cases (none, i k~, with a unit scale) in code of
+        // their own, then the stores; partial sums (written by this thread) are read in batches ahead of them
+        if (xf.post == MUL_IK && unit) {
+#pragma unroll
+          for (int r = 0; r < R; ++r) u[r] = mul_ik(u[r], katab[i + r * nb]);
+        } else if (xf.post) {
+#pragma unroll
+          for (int r = 0; r < R; ++r) {
+            u[r] = scal(u[r], mult(xf.post, i + r * nb, scale));
+            if (xf.post & MUL_IK) u[r] = mul_i(u[r]);
+          }
+        } else if (!unit) {
+#pragma unroll
+          for (int r = 0; r < R; ++r) u[r] = scal(u[r], scale);
+        }
+        cpx<T>* q = dst + g0 + i * ls;
+        const int qs = nb * ls;
+        if (xf.first) {
+#pragma unroll
+          for (int r = 0; r < R; ++r) q[r * qs] = u[r];
+        } else {
           constexpr int PB = R < 4 ? R : 4;
 #pragma unroll
           for (int r0 = 0; r0 < R; r0 += PB) {
             cpx<T> prev[PB];
-            if (!xf.first) {
-#pragma unroll
-              for (int b = 0; b < PB; ++b)
-                if (r0 + b < R) prev[b] = dst[g0 + (i + (r0 + b) * nb) * ls];
-            }
 #pragma unroll
             for (int b = 0; b < PB; ++b)
-              if (r0 + b < R) put(i + (r0 + b) * nb, u[r0 + b], prev[b]);
+              if (r0 + b < R) prev[b] = q[(r0 + b) * qs];
+#pragma unroll
+            for (int b = 0; b < PB; ++b)
+              if (r0 + b < R) q[(r0 + b) * qs] = prev[b] + u[r0 + b];
           }
         }
       }
@@ -573,8 +581,10 @@ static void wide_axis_launch(const AxisProg& P, const GridDesc& g, const cpx<T>*
   const long long lines = (long long)g.h0 * (P.axis == 2 ? g.n1 : g.n2);
   const int tpl = wide_tpl(pl, W);
   const size_t smem = wide_axis_smem(pl, W, sizeof(T));
-  ensure_smem(reinterpret_cast<const void*>(k_axis_w<T, S>), smem);
-  pdl_launch(k_axis_w<T, S>, dim3((unsigned)((lines + W - 1) / W), groups), W * tpl, smem, st, P, g, tw, wide_log2(W), tpl,
+  const bool pad = W * (int)sizeof(cpx<T>) < 128;
+  auto kernel = pad ? k_axis_w<T, S, true> : k_axis_w<T, S, false>;
+  ensure_smem(reinterpret_cast<const void*>(kernel), smem);
+  pdl_launch(kernel, dim3((unsigned)((lines + W - 1) / W), groups), W * tpl, smem, st, P, g, tw, wide_log2(W), tpl,
                                                                               wide_pad_shift(pl), cls);
 }
 
