@@ -4,7 +4,7 @@
 // blocks writes per-block partials, and the last block to finish (atomic ticket) adds them
 // in a fixed order and runs the scalar epilogue of the algorithm (step lengths, Givens
 // rotations, convergence tests) in one thread.  The scalars never leave the device; the
-// host only reads the `done` flag every `check_every` iterations, and (CG, RMR) one batch
+// host only reads the `done` flag every `check_every` iterations, one batch
 // behind: it waits for the flag of batch k-1 with batch k already queued.  Kernels of an
 // iteration return at once when the flag is set, so iterations enqueued ahead cost a launch
 // each and change nothing.
@@ -198,7 +198,6 @@ enum Epi : int {
   EPI_GM_BETA = 7,    // tot = [rr]
   EPI_GM_H1 = 8,      // tot[i] -> h1[off + i]
   EPI_GM_H2 = 9,      // tot[i] -> h2[off + i]
-  EPI_GM_NORM = 10,   // tot = [ww]
   EPI_NORM = 11,      // tot = [vv] -> ks->rr
 };
 
@@ -334,56 +333,75 @@ __device__ void epilogue(int epi, const double (&t)[NV], KState* ks, double* his
         if (off + i <= j) h[off + i] = t[i];
       return;
     }
-    case EPI_GM_NORM: {
-      const int m = ks->m;
-      const double hn = sqrt(t[0]);
-      double* __restrict__ col = ks->H + (size_t)j * (m + 1);
-      const double* __restrict__ h1 = ks->h1;
-      const double* __restrict__ h2 = ks->h2;
-      const double* __restrict__ cs = ks->cs;
-      const double* __restrict__ sn = ks->sn;
-      // the entry a rotation passes on stays in a register; the loads of the next rotations
-      // (unrolled) do not wait for it
-      double cur = h1[0] + h2[0];
-#pragma unroll 4
-      for (int i = 0; i < j; ++i) {
-        const double nx = h1[i + 1] + h2[i + 1], ci = cs[i], si = sn[i];
-        col[i] = ci * cur + si * nx;
-        cur = -si * cur + ci * nx;
-      }
-      double c = 1.0, s = 0.0;
-      if (hn != 0.0) {
-        const double h = hypot(cur, hn);
-        c = cur / h;
-        s = hn / h;
-      }
-      ks->cs[j] = c;
-      ks->sn[j] = s;
-      col[j] = c * cur + s * hn;
-      col[j + 1] = 0.0;
-      ks->gv[j + 1] = -s * ks->gv[j];
-      ks->gv[j] = c * ks->gv[j];
-      ks->iters += 1;
-      ks->k = j + 1;
-      const double est = fabs(ks->gv[j + 1]) / sqrt(ks->bb);
-      ks->relres = est;
-      record(ks, hist, est);
-      ks->ww = hn;
-      if (bad(est)) {
-        ks->status = VD_ERR_NONFINITE;
-        ks->cycle_done = 1;
-      } else if (est <= tol || hn == 0.0) {
-        ks->status = 0;   // converged (or invariant Krylov space): finished after the update
-        ks->cycle_done = 1;
-      } else if (j + 1 >= m || ks->iters >= ks->maxit) {
-        ks->cycle_done = 1;
-      }
-      return;
-    }
     case EPI_NORM: {
       ks->rr = t[0];
       return;
     }
+  }
+}
+
+// End of GMRES step j (tot = |w|^2): the new column of H through the rotations, the next rotation, the
+// residual estimate and the cycle's end; by one warp.  One thread's rotations were four FP64 operations of
+// 64 cycles each in a row, its square roots and quotients six of 600: 6 us of a step at j = 30.  Here
+// the products that do not pass from rotation to rotation are formed by a lane per rotation, leaving
+// one operation per rotation in the chain, and roots and quotients run side by side in lanes.
+__device__ void gm_norm_epilogue(double tot, KState* ks, double* hist, double tol, int j) {
+  if (tol < 0.0) tol = ks->dtol;
+  const int lane = threadIdx.x;
+  const int m = ks->m;
+  double* __restrict__ col = ks->H + (size_t)j * (m + 1);
+  constexpr int K = kMaxRestart / 32;
+  double c[K], sn[K], cn[K], sx[K], at[K];   // rotation i = lane + 32 k: c, s, c h_{i+1}, s h_{i+1}, entry passed on
+#pragma unroll
+  for (int k = 0; k < K; ++k) {
+    const int i = lane + 32 * k;
+    const bool in = i < j;
+    c[k] = in ? ks->cs[i] : 0.0;
+    sn[k] = in ? ks->sn[i] : 0.0;
+    const double h = in ? ks->h1[i + 1] + ks->h2[i + 1] : 0.0;
+    cn[k] = c[k] * h;
+    sx[k] = sn[k] * h;
+    at[k] = 0.0;
+  }
+  const double root = sqrt(lane == 1 ? ks->bb : tot);
+  const double hn = __shfl_sync(0xffffffffu, root, 0), bn = __shfl_sync(0xffffffffu, root, 1);
+  double cur = ks->h1[0] + ks->h2[0];
+#pragma unroll
+  for (int k = 0; k < K; ++k)
+    for (int l = 0; l < 32 && l + 32 * k < j; ++l) {
+      at[k] = lane == l ? cur : at[k];
+      cur = fma(-__shfl_sync(0xffffffffu, sn[k], l), cur, __shfl_sync(0xffffffffu, cn[k], l));
+    }
+#pragma unroll
+  for (int k = 0; k < K; ++k)
+    if (lane + 32 * k < j) col[lane + 32 * k] = fma(c[k], at[k], sx[k]);
+  const double h2 = fma(cur, cur, hn * hn);
+  const double h = (h2 > 1e-280 && h2 < 1e280) ? sqrt(h2) : hypot(cur, hn);
+  const double g = ks->gv[j];
+  const double q = (lane == 0 ? cur : (lane == 1 ? hn : g)) / (lane < 2 ? h : bn);
+  const bool turn = hn != 0.0;
+  const double cj = turn ? __shfl_sync(0xffffffffu, q, 0) : 1.0, sj = turn ? __shfl_sync(0xffffffffu, q, 1) : 0.0;
+  const double est = fabs(sj) * fabs(__shfl_sync(0xffffffffu, q, 2));
+  if (lane != 0) return;
+  ks->cs[j] = cj;
+  ks->sn[j] = sj;
+  col[j] = cj * cur + sj * hn;
+  col[j + 1] = 0.0;
+  ks->gv[j + 1] = -sj * g;
+  ks->gv[j] = cj * g;
+  ks->iters += 1;
+  ks->k = j + 1;
+  ks->relres = est;
+  record(ks, hist, est);
+  ks->ww = hn;
+  if (bad(est)) {
+    ks->status = VD_ERR_NONFINITE;
+    ks->cycle_done = 1;
+  } else if (est <= tol || hn == 0.0) {
+    ks->status = 0;   // converged (or invariant Krylov space): finished after the update
+    ks->cycle_done = 1;
+  } else if (j + 1 >= m || ks->iters >= ks->maxit) {
+    ks->cycle_done = 1;
   }
 }
 
@@ -807,7 +825,7 @@ __global__ void __launch_bounds__(kRedThreads) k_gm_step(Ix ix, cpx<T>* __restri
     epilogue<NB>(EPI_GM_H2, t, ra.ks, ra.hist, ra.tol, 0, nv - 1);
 }
 
-// GMRES: w -= sum_{i<=j} h_i V_i (h = h1 or h2); with_norm: reduce [(w,w)] -> EPI_GM_NORM
+// GMRES: w -= sum_{i<=j} h_i V_i (h = h1 or h2); with_norm: reduce [(w,w)] -> gm_norm_epilogue
 template <typename T>
 __global__ void __launch_bounds__(kRedThreads) k_gm_maxpy(Ix ix, cpx<T>* __restrict__ w,
                                                           const cpx<T>* __restrict__ V, int j, int which, int with_norm,
@@ -833,8 +851,8 @@ __global__ void __launch_bounds__(kRedThreads) k_gm_maxpy(Ix ix, cpx<T>* __restr
   if (!with_norm) return;
   const typename Acc<T>::Sum v[1] = {a0.total()};
   double t[1];
-  if (reduce_last(v, ra.partials, ra.counter, t) && threadIdx.x == 0)
-    epilogue<1>(EPI_GM_NORM, t, ra.ks, ra.hist, ra.tol, 0, j);
+  if (reduce_last(v, ra.partials, ra.counter, t) && threadIdx.x < 32)
+    gm_norm_epilogue(t[0], ra.ks, ra.hist, ra.tol, j);
 }
 
 static inline Ix mkix(long long len, int h0, long long nc, int blocks, int threads);
@@ -849,7 +867,7 @@ static inline Ix mkix(long long len, int h0, long long nc, int blocks, int threa
     else CALL(32);                  \
   } while (0)
 
-// the orthogonalisation of w against V_0..V_j on st: h1, h2, w and |w| (EPI_GM_NORM)
+// the orthogonalisation of w against V_0..V_j on st: h1, h2, w and |w| (gm_norm_epilogue)
 template <typename T>
 static void gm_orthogonalise(const SpecSystem& sys, cpx<T>* w, const cpx<T>* V, int j, const RedArgs& ra,
                              cudaStream_t st) {
@@ -1329,6 +1347,8 @@ vd_status krylov_solve(const SpecSystem& sys, const SolveOpts& o, const void* b,
   } else {
     cpx<T>* V = vb;
     cpx<T>* w = vb + (size_t)(m + 1) * len;
+    HeadPipeLease lease;
+    HeadPipe* hp = lease.get();
     { ProfScope ps_(sizeof(T) == 4 ? PC_VEC32 : PC_VEC64, st, (double)1 * len * sizeof(cpx<T>), 0.0); pdl_launch(k_norms<T, 1>, rb, kRedThreads, 0, st, ixr, nullptr, B, EPI_BB, ra, nullptr); }
     for (int cycle = 0;; ++cycle) {
       // r = b - A x into V_0 (unnormalised), then V_0 /= beta
@@ -1340,15 +1360,39 @@ vd_status krylov_solve(const SpecSystem& sys, const SolveOpts& o, const void* b,
       }
       { ProfScope ps_(sizeof(T) == 4 ? PC_VEC32 : PC_VEC64, st, (double)1 * len * sizeof(cpx<T>), 0.0); pdl_launch(k_norms<T, 1>, rb, kRedThreads, 0, st, ixr, nullptr, V, EPI_GM_BETA, ra, done); }
       { ProfScope ps_(sizeof(T) == 4 ? PC_VEC32 : PC_VEC64, st, (double)2 * len * sizeof(cpx<T>), 0.0); pdl_launch(k_gm_scale<T>, eb, 256, 0, st, ixe, V, V, kw.ks, 1); }
+      // the flag of step j is read with step j + check already queued (its kernels see the device's
+      // flag and return), so the device does not wait for the host between steps.  Not for three
+      // components: their step that comes to nothing is 25 launches, as long as the waits of a cycle
+      // (96^3 velocity solve 5.76 ms ahead, 5.66 not; 480 x 360 pressure 5.66 and 6.24, 320^2 velocity 2.56
+      // and 2.67).
+      const bool ahead = hp && sys.ncomp < 3;
+      int snaps = 0;
+      long long mark = 0;
       for (int j = 0; j < m; ++j) {
+        if (j % check == 0) mark = prof_mark();
         cpx<T>* Vj = V + (size_t)j * len;
         sys.apply(sys, Vj, w, true, cdone, st);
         gm_orthogonalise<T>(sys, w, V, j, ra, st);
         { ProfScope ps_(sizeof(T) == 4 ? PC_VEC32 : PC_VEC64, st, (double)2 * len * sizeof(cpx<T>), 0.0); pdl_launch(k_gm_scale<T>, eb, 256, 0, st, ixe, V + (size_t)(j + 1) * len, w, kw.ks, 0); }
         if ((j + 1) % check == 0 || j + 1 == m) {
-          vd_status e = read_head(kw, &hd, st);
+          vd_status e = VD_OK;
+          if (!ahead) {
+            e = read_head(kw, &hd, st);
+            if (e != VD_OK) return e;
+            if (hd.cycle_done || hd.done) break;
+            continue;
+          }
+          if (snaps > 0) {
+            e = hp->latest(&hd);
+            if (e != VD_OK) return e;
+            if (hd.cycle_done || hd.done) {
+              prof_discard(mark, st);
+              break;
+            }
+          }
+          e = hp->snapshot(kw, st);
           if (e != VD_OK) return e;
-          if (hd.cycle_done || hd.done) break;
+          ++snaps;
         }
       }
       { pdl_launch(k_gm_solve, 1, 32, 0, st, kw.ks); count_launch(); }
