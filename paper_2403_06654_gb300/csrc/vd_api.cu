@@ -773,7 +773,7 @@ vd_status enqueue_solve_graph(const vd_grid* G, vd_op op, vd_solver solver, cons
     si.check_every = 1;
     si.x_zero = 1;
     e = refine_enqueue_graph(sys64, sys32, &resid_cb, &rc, si, tol, auto_inner_tol(G), maxit, L.bh, L.xh, L.rh, L.bh_f, L.xh_f,
-                             L.vecs, kw, L.ost, info, st, body[0], body[1], body[2]);
+                             L.vecs, kw, L.ost, info, st, body[0], body[1], body[2], body[3]);
     if (e != VD_OK) return e;
     if (dd) inv_transform_dd(G, L.xh, x, L.tmp, st);
     else inv_all(G, ncomp, L.xh, x, L.tmp, st);
@@ -788,7 +788,7 @@ vd_status enqueue_solve_graph(const vd_grid* G, vd_op op, vd_solver solver, cons
   so.check_every = 1;
   so.x_zero = 1;
   SpecSystem sys = make_system<double>(G, op, opp, L.sym, L.tmp);
-  if ((e = krylov_enqueue_graph<double>(sys, so, L.bh, L.xh, L.vecs, kw, st, body_st)) != VD_OK) return e;
+  if ((e = krylov_enqueue_graph<double>(sys, so, L.bh, L.xh, L.vecs, kw, st, body_st, body[1])) != VD_OK) return e;
   inv_all(G, ncomp, L.xh, x, L.tmp, st);
   return krylov_graph_finish<double>(sys, L.bh, L.xh, L.vecs, kw, info, st);
 }

@@ -131,7 +131,7 @@ vd_status vd_batch_create(const vd_batch_item* items, int count, const vd_batch_
   VD_CUDA(cudaStreamSynchronize(st));
 
   // record: fork one branch per item from the capturing stream, join them at the end
-  cudaStream_t body[3] = {nullptr, nullptr, nullptr};
+  cudaStream_t body[4] = {nullptr, nullptr, nullptr, nullptr};
   cudaEvent_t fork = nullptr;
   std::vector<cudaEvent_t> joins(2 * count, nullptr);
   std::vector<cudaStream_t> branches(2 * count, nullptr);   // one capture stream per system

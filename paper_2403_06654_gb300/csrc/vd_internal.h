@@ -148,8 +148,8 @@ vd_status small_solve_1d(const vd_grid* G, int solver, const vd_solve_params* pr
                          double* x, vd_solve_info* info, void* out_dev, double* hist_dev, int hist_cap,
                          cudaStream_t st);
 
-// one solve recorded into the capture of st (see vd_api.cu); body: 3 streams for the
-// conditional bodies (one is enough in FP64)
+// one solve recorded into the capture of st (see vd_api.cu); body: 4 streams for the
+// conditional bodies (two are enough in FP64)
 vd_status enqueue_solve_graph(const vd_grid* G, vd_op op, vd_solver solver, const vd_op_params* opp, double tol,
                               int maxit, int restart, int precision, const double* b, double* x, void* ws,
                               size_t ws_bytes, double* info, cudaStream_t st, cudaStream_t const* body);

@@ -1461,6 +1461,45 @@ __global__ void k_ks_reset_dev(KState* ks, const OState* o, int m, cudaGraphCond
   ks->dtol = o->itol;
 }
 
+// The Arnoldi steps of a recorded GMRES cycle stand in groups, each the body of an IF node: a group that
+// ends before the cycle does sets the condition of the next, so the steps after convergence are
+// skipped (as kernels that return at once, 16 to 25 a step, they were half of a 64^3 velocity solve:
+// 5.0 ms recorded, 2.6 in groups).
+constexpr int kGmGroups = 8;
+constexpr int kGmGroupAt[kGmGroups + 1] = {0, 4, 8, 12, 16, 24, 32, 48, kMaxRestart};
+struct GmConds {
+  cudaGraphConditionalHandle h[kGmGroups];
+};
+// start of a cycle: the first group runs unless the residual already meets the tolerance
+__global__ void k_gm_arm(GmConds c, int n, const KState* ks) {
+  pdl_wait();
+  if (threadIdx.x < n) cudaGraphSetConditional(c.h[threadIdx.x], (threadIdx.x == 0 && !ks->cycle_done) ? 1u : 0u);
+}
+__global__ void k_gm_next(cudaGraphConditionalHandle h, const KState* ks) {
+  pdl_wait();
+  if (threadIdx.x == 0) cudaGraphSetConditional(h, ks->cycle_done ? 0u : 1u);
+}
+
+static vd_status open_cond(cudaStream_t st, cudaGraphConditionalNodeType type, cudaGraphConditionalHandle hnd,
+                           cudaGraph_t* body) {
+  cudaStreamCaptureStatus cs;
+  cudaGraph_t g = nullptr;
+  const cudaGraphNode_t* deps = nullptr;
+  size_t nd = 0;
+  VD_CUDA(cudaStreamGetCaptureInfo(st, &cs, nullptr, &g, &deps, nullptr, &nd));
+  if (cs != cudaStreamCaptureStatusActive) return fail(VD_ERR_INVALID_ARG, "graph solve needs a capturing stream");
+  cudaGraphNodeParams cp{};
+  cp.type = cudaGraphNodeTypeConditional;
+  cp.conditional.handle = hnd;
+  cp.conditional.type = type;
+  cp.conditional.size = 1;
+  cudaGraphNode_t node;
+  VD_CUDA(cudaGraphAddNode(&node, g, deps, nullptr, nd, &cp));
+  VD_CUDA(cudaStreamUpdateCaptureDependencies(st, &node, nullptr, 1, cudaStreamSetCaptureDependencies));
+  *body = cp.conditional.phGraph_out[0];
+  return VD_OK;
+}
+
 __global__ void k_graph_cond(cudaGraphConditionalHandle handle, const KState* ks) {
   pdl_wait();
   if (threadIdx.x == 0 && blockIdx.x == 0) cudaGraphSetConditional(handle, ks->done ? 0u : 1u);
@@ -1468,7 +1507,7 @@ __global__ void k_graph_cond(cudaGraphConditionalHandle handle, const KState* ks
 
 template <typename T>
 vd_status krylov_enqueue_graph(const SpecSystem& sys, const SolveOpts& o, const void* b, void* x, void* vecs,
-                               const KWork& kw, cudaStream_t st, cudaStream_t body_st) {
+                               const KWork& kw, cudaStream_t st, cudaStream_t body_st, cudaStream_t group_st) {
   const long long len = sys.len;
   const long long nc = sys.G->g.ncplx;
   const int h0 = sys.h0;
@@ -1582,12 +1621,34 @@ vd_status krylov_enqueue_graph(const SpecSystem& sys, const SolveOpts& o, const 
     count_launch();
     count_launch();
     count_launch();
-    for (int j = 0; j < m; ++j) {
-      cpx<T>* Vj = V + (size_t)j * len;
-      sys.apply(sys, Vj, w, true, cdone, body_st);
-      gm_orthogonalise<T>(sys, w, V, j, ra, body_st);
-      pdl_launch(k_gm_scale<T>, eb, 256, 0, body_st, ixe, V + (size_t)(j + 1) * len, w, kw.ks, 0);
-      count_launch();
+    int groups = 0;
+    while (kGmGroupAt[groups] < m) ++groups;
+    GmConds conds{};
+    {
+      cudaStreamCaptureStatus cs;
+      cudaGraph_t g = nullptr;
+      VD_CUDA(cudaStreamGetCaptureInfo(body_st, &cs, nullptr, &g, nullptr, nullptr, nullptr));
+      for (int k = 0; k < groups; ++k)
+        VD_CUDA(cudaGraphConditionalHandleCreate(&conds.h[k], g, 0, cudaGraphCondAssignDefault));
+    }
+    pdl_launch(k_gm_arm, 1, 32, 0, body_st, conds, groups, kw.ks);
+    count_launch();
+    for (int k = 0; k < groups; ++k) {
+      cudaGraph_t gb = nullptr;
+      if ((e = open_cond(body_st, cudaGraphCondTypeIf, conds.h[k], &gb)) != VD_OK) return e;
+      VD_CUDA(cudaStreamBeginCaptureToGraph(group_st, gb, nullptr, nullptr, 0, cudaStreamCaptureModeRelaxed));
+      for (int j = kGmGroupAt[k]; j < std::min(m, kGmGroupAt[k + 1]); ++j) {
+        cpx<T>* Vj = V + (size_t)j * len;
+        sys.apply(sys, Vj, w, true, cdone, group_st);
+        gm_orthogonalise<T>(sys, w, V, j, ra, group_st);
+        pdl_launch(k_gm_scale<T>, eb, 256, 0, group_st, ixe, V + (size_t)(j + 1) * len, w, kw.ks, 0);
+        count_launch();
+      }
+      if (k + 1 < groups) {
+        pdl_launch(k_gm_next, 1, 1, 0, group_st, conds.h[k + 1], kw.ks);
+        count_launch();
+      }
+      VD_CUDA(cudaStreamEndCapture(group_st, &gb));
     }
     pdl_launch(k_gm_solve, 1, 32, 0, body_st, kw.ks);
     pdl_launch(k_gm_update<T>, eb, 256, 0, body_st, ixe, X, V, sym, kw.ks);
@@ -1723,32 +1784,12 @@ __global__ void k_out_info(const OState* o, double* info) {
 
 // v *= 1/|r| and x += |r| d with the scalars read from the refinement state
 
-static vd_status open_cond(cudaStream_t st, cudaGraphConditionalNodeType type, cudaGraphConditionalHandle hnd,
-                           cudaGraph_t* body) {
-  cudaStreamCaptureStatus cs;
-  cudaGraph_t g = nullptr;
-  const cudaGraphNode_t* deps = nullptr;
-  size_t nd = 0;
-  VD_CUDA(cudaStreamGetCaptureInfo(st, &cs, nullptr, &g, &deps, nullptr, &nd));
-  if (cs != cudaStreamCaptureStatusActive) return fail(VD_ERR_INVALID_ARG, "graph solve needs a capturing stream");
-  cudaGraphNodeParams cp{};
-  cp.type = cudaGraphNodeTypeConditional;
-  cp.conditional.handle = hnd;
-  cp.conditional.type = type;
-  cp.conditional.size = 1;
-  cudaGraphNode_t node;
-  VD_CUDA(cudaGraphAddNode(&node, g, deps, nullptr, nd, &cp));
-  VD_CUDA(cudaStreamUpdateCaptureDependencies(st, &node, nullptr, 1, cudaStreamSetCaptureDependencies));
-  *body = cp.conditional.phGraph_out[0];
-  return VD_OK;
-}
-
 vd_status refine_enqueue_graph(const SpecSystem& sys64, const SpecSystem& sys32,
                                void (*resid)(const void* ctx, const void* x, void* y, cudaStream_t st),
                                const void* resid_ctx, const SolveOpts& inner, double tol, double itol0, int maxit,
                                void* bh, void* xh, void* rh, void* bh_f, void* xh_f, void* vecs, const KWork& kw,
                                OState* ost, double* info, cudaStream_t st, cudaStream_t s1, cudaStream_t s2,
-                               cudaStream_t s3) {
+                               cudaStream_t s3, cudaStream_t s4) {
   const long long len = sys64.len;
   const int rb = red_blocks(len);
   const int eb = ew_blocks(len);
@@ -1808,7 +1849,7 @@ vd_status refine_enqueue_graph(const SpecSystem& sys64, const SpecSystem& sys32,
   si.src64 = RH;
   si.x_zero = 1;
   si.dev_outer = ost;
-  if ((e = krylov_enqueue_graph<float>(sys32, si, bh_f, xh_f, vecs, kw, s2, s3)) != VD_OK) return e;
+  if ((e = krylov_enqueue_graph<float>(sys32, si, bh_f, xh_f, vecs, kw, s2, s3, s4)) != VD_OK) return e;
   pdl_launch(k_out_after_inner, 1, 1, 0, s2, ost, kw.ks);
   pdl_launch(k_axpy_f2d, eb, 256, 0, s2, len, 0.0, ost, (const cpx<float>*)xh_f, XH);
   resid(resid_ctx, XH, RH, s2);
@@ -1827,9 +1868,9 @@ vd_status refine_enqueue_graph(const SpecSystem& sys64, const SpecSystem& sys32,
 }
 
 template vd_status krylov_enqueue_graph<double>(const SpecSystem&, const SolveOpts&, const void*, void*, void*,
-                                                const KWork&, cudaStream_t, cudaStream_t);
+                                                const KWork&, cudaStream_t, cudaStream_t, cudaStream_t);
 template vd_status krylov_enqueue_graph<float>(const SpecSystem&, const SolveOpts&, const void*, void*, void*,
-                                               const KWork&, cudaStream_t, cudaStream_t);
+                                               const KWork&, cudaStream_t, cudaStream_t, cudaStream_t);
 
 template vd_status krylov_solve<double>(const SpecSystem&, const SolveOpts&, const void*, void*, void*, const KWork&,
                                         double*, int, SolveOut*, cudaStream_t);

@@ -107,21 +107,22 @@ template <typename T>
 size_t krylov_vec_bytes(const SpecSystem& sys, int solver, int restart);
 
 // The same solve as a capturable graph fragment: `st` must be capturing; the iteration loop
-// becomes a conditional WHILE node (its body captured on body_st).  No host synchronisation:
+// becomes a conditional WHILE node (its body captured on body_st, the groups of GMRES steps within it on
+// group_st).  No host synchronisation:
 // the result stays in the KState (iters, status, relres, done).
 template <typename T>
 vd_status krylov_enqueue_graph(const SpecSystem& sys, const SolveOpts& o, const void* b, void* x, void* vecs,
-                               const KWork& kw, cudaStream_t st, cudaStream_t body_st);
+                               const KWork& kw, cudaStream_t st, cudaStream_t body_st, cudaStream_t group_st);
 // Iterative refinement as a graph fragment (see vd_krylov.cu): x += |r| d with the inner
 // float solve A32 d = r/|r| and r = b - A x from `resid` (double or float-pair operator).
 // bh, xh, rh: double spectral vectors (bh holds the projected rhs; xh is zeroed here);
-// bh_f, xh_f, vecs: float inner vectors.  Streams: st capturing, s1..s3 for the bodies.
+// bh_f, xh_f, vecs: float inner vectors.  Streams: st capturing, s1..s4 for the bodies.
 vd_status refine_enqueue_graph(const SpecSystem& sys64, const SpecSystem& sys32,
                                void (*resid)(const void* ctx, const void* x, void* y, cudaStream_t st),
                                const void* resid_ctx, const SolveOpts& inner, double tol, double itol0, int maxit,
                                void* bh, void* xh, void* rh, void* bh_f, void* xh_f, void* vecs, const KWork& kw,
                                OState* ost, double* info, cudaStream_t st, cudaStream_t s1, cudaStream_t s2,
-                               cudaStream_t s3);
+                               cudaStream_t s3, cudaStream_t s4);
 
 // After a graph solve: true residual of x and the result record info[0..4] (iterations,
 // status, monitored relres, |b|^2, true relres), all on the device.  vecs: scratch.
