@@ -1510,12 +1510,26 @@ void ensure_smem(const void* func, size_t smem) {
   }
 }
 
+// The plan of radices up to 5 of a length, in the Stockham engine's form: float pairs of the lengths that
+// the packed engine does not take.  A radix-8 butterfly on float pairs is some 1200 instructions of one
+// thread, and a small field leaves a warp or two per block to run them (forward transform, radices up
+// to 8 and up to 5: 96^2 14.6 and 12.9 us, 320^2 23.6 and 17.4, 480 x 360 28.4 and 20.7, 80^3 33.6 and 31.2,
+// 96^3 38.1 and 37.7, 160^3 155 and 152).
+static FftPlan narrow_plan(const WidePlan& w) {
+  FftPlan p{};
+  p.n = w.n;
+  p.nst = w.nst;
+  for (int s = 0; s < w.nst; ++s) p.rad[s] = w.rad[s];
+  p.tw_off = w.tw_off;
+  return p;
+}
+
 template <typename T, int S, bool CV, bool PK>
 static void launch_k_axis(const AxisProg& P, const GridDesc& g, const cpx<T>* tw, int W, long long blocks,
-                          size_t smem, cudaStream_t st) {
-  // 8 elements per thread, whole lines' worth of warps
+                          size_t smem, cudaStream_t st, int per = 8) {
+  // `per` elements per thread, whole lines' worth of warps
   const int n = (P.axis == 2) ? g.pz.n : g.py.n;
-  const int threads = std::min(kThreads, std::max(32, W * std::max((n + 7) / 8, (31 + W) / W)));
+  const int threads = std::min(kThreads, std::max(32, W * std::max((n + per - 1) / per, (31 + W) / W)));
   ensure_smem(reinterpret_cast<const void*>(k_axis<T, S, CV, PK>), smem);
   pdl_launch(k_axis<T, S, CV, PK>, (unsigned)blocks, threads, smem, st, P, g, tw, ilog2(W));
 }
@@ -1722,10 +1736,16 @@ void launch_axis(const AxisProg& P0, int dir, const GridDesc& g, const void* tw,
       else launch_k_axis<T, +1, false, true>(P, g, twp, W, blocks, psmem, st);
       return;
     }
-    if (dir < 0 && cv) launch_k_axis<T, -1, true, false>(P, g, twp, W, blocks, smem, st);
-    else if (dir < 0) launch_k_axis<T, -1, false, false>(P, g, twp, W, blocks, smem, st);
-    else if (cv) launch_k_axis<T, +1, true, false>(P, g, twp, W, blocks, smem, st);
-    else launch_k_axis<T, +1, false, false>(P, g, twp, W, blocks, smem, st);
+    GridDesc gn = g;
+    int per = 8;
+    if (!p_plan_ok(pl, n)) {   // by the length alone: a shape never changes the bits
+      (P.axis == 2 ? gn.pz : gn.py) = narrow_plan((P.axis == 2 ? g.wz : g.wy)[0]);
+      per = 4;
+    }
+    if (dir < 0 && cv) launch_k_axis<T, -1, true, false>(P, gn, twp, W, blocks, smem, st, per);
+    else if (dir < 0) launch_k_axis<T, -1, false, false>(P, gn, twp, W, blocks, smem, st, per);
+    else if (cv) launch_k_axis<T, +1, true, false>(P, gn, twp, W, blocks, smem, st, per);
+    else launch_k_axis<T, +1, false, false>(P, gn, twp, W, blocks, smem, st, per);
   } else {
     wide_axis<T>(P, dir, g, tw, W, split_axis(P, (inner_n * outer_n + W - 1) / W), st);
   }
@@ -1733,10 +1753,10 @@ void launch_axis(const AxisProg& P0, int dir, const GridDesc& g, const void* tw,
 
 template <typename T, bool CV, bool PK, int MINB = 3>
 static void launch_k_xpass(const XProg& P, const GridDesc& g, const cpx<T>* tw, int L, long long blocks, size_t smem,
-                           cudaStream_t st) {
+                           cudaStream_t st, int per = 8) {
   ensure_smem(reinterpret_cast<const void*>(k_xpass<T, CV, PK, MINB>), smem);
-  // threads per line: a power of two, one radix-8 butterfly each, at least a warp per block
-  const int tpl = std::min(kThreads / L, std::max(pow2_at_least((g.px.n + 7) / 8), pow2_at_least((31 + L) / L)));
+  // threads per line: a power of two, `per` elements each, at least a warp per block
+  const int tpl = std::min(kThreads / L, std::max(pow2_at_least((g.px.n + per - 1) / per), pow2_at_least((31 + L) / L)));
   pdl_launch(k_xpass<T, CV, PK, MINB>, (unsigned)blocks, L * tpl, smem, st, P, g, tw, ilog2(L), ilog2(tpl));
 }
 
@@ -1828,8 +1848,14 @@ void launch_xpass(const XProg& P0, const GridDesc& g, const void* tw, cudaStream
       else launch_k_xpass<T, false, true, 3>(P, g, twp, L, blocks, psmem, st);
       return;
     }
-    if (cv) launch_k_xpass<T, true, false>(P, g, twp, L, blocks, smem, st);
-    else launch_k_xpass<T, false, false>(P, g, twp, L, blocks, smem, st);
+    GridDesc gn = g;
+    int per = 8;
+    if (!p_plan_ok(g.px, m)) {
+      gn.px = narrow_plan(g.wx[0]);
+      per = 4;
+    }
+    if (cv) launch_k_xpass<T, true, false>(P, gn, twp, L, blocks, smem, st, per);
+    else launch_k_xpass<T, false, false>(P, gn, twp, L, blocks, smem, st, per);
   } else {
     wide_xpass<T>(P, g, tw, L, split_xpass(P, (nlines + L - 1) / L), st);
   }
