@@ -897,19 +897,13 @@ vd_status vd_divergence(const vd_grid* G, const double* u, double* out, void* ws
   const GridDesc& g = G->g;
   const size_t need = align256((size_t)g.ncplx * 16 * 3);
   if (ws_bytes < need) return fail(VD_ERR_OOM, "workspace too small (3 spectral fields)");
+  // the sum over j of i k_j F u_j in spectral space, then one inverse transform (d forward transforms
+  // in one launch per pass; d inverse transforms summed in physical space took 22 launches in 3D)
   cpx<double>* a = (cpx<double>*)ws;
-  cpx<double>* acc = a + g.ncplx;
-  cpx<double>* tmp = acc + g.ncplx;
-  // out = sum_j F^-1(i k_j F u_j): accumulate i k_j u^_j in spectral space via derivative transforms
-  VD_CUDA(cudaMemsetAsync(out, 0, sizeof(double) * g.nreal, st));
-  for (int j = 0; j < g.ndim; ++j) {
-    fwd_transform<double>(G, u + (size_t)j * g.nreal, a, st);
-    Mult m;
-    m.deriv[j] = 1;
-    inv_transform<double>(G, a, m, reinterpret_cast<double*>(acc), tmp, st);
-    // out += acc (physical): reuse spectral axpy on reals viewed as complex pairs
-    spec_axpy<double>(g.nreal / 2, 1.0, acc, out, st);
-  }
+  fwd_transform_n<double>(G, g.ndim, u, a, st);
+  divergence_spec(G, a, st);
+  Mult m;
+  inv_transform<double>(G, a, m, out, a + g.ncplx, st);
   VD_CUDA(cudaGetLastError());
   return VD_OK;
 }
@@ -921,13 +915,10 @@ vd_status vd_gradient(const vd_grid* G, const double* phi, double* out, void* ws
   const size_t need = align256((size_t)g.ncplx * 16 * 3);
   if (ws_bytes < need) return fail(VD_ERR_OOM, "workspace too small (3 spectral fields)");
   cpx<double>* a = (cpx<double>*)ws;
-  cpx<double>* tmp = a + g.ncplx;
   fwd_transform<double>(G, phi, a, st);
-  for (int j = 0; j < g.ndim; ++j) {
-    Mult m;
-    m.deriv[j] = 1;
-    inv_transform<double>(G, a, m, out + (size_t)j * g.nreal, tmp, st);
-  }
+  double* grad[3];
+  for (int j = 0; j < 3; ++j) grad[j] = out + (size_t)j * g.nreal;
+  gradient_fields(G, a, grad, a + g.ncplx, st);
   VD_CUDA(cudaGetLastError());
   return VD_OK;
 }

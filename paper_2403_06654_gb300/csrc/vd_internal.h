@@ -122,6 +122,10 @@ int velocity_spec_tmps(int ndim);    // of which spectral scratch (the rest hold
 // grad[j] = F^-1(i k_j rh), hess[hidx(a, b)] = F^-1((i k_a)(i k_b) rh) in double; tmp: 3 spectral fields
 void derivative_fields(const vd_grid* G, const cpx<double>* rh, double* const grad[3], double* const hess[6],
                        cpx<double>* tmp, cudaStream_t st);
+// grad[j] = F^-1(i k_j a); t: two spectral fields; a is overwritten in 3D
+void gradient_fields(const vd_grid* G, cpx<double>* a, double* const grad[3], cpx<double>* t, cudaStream_t st);
+// a_0 <- sum_j i k_j a_j over ndim spectral fields back to back
+void divergence_spec(const vd_grid* G, cpx<double>* a, cudaStream_t st);
 int pressure_tmp_fields(int ndim);
 
 // K_rho operator in spectral space: out = K~ (S in) = Lap S in + F(c F^-1(S in)); with S the

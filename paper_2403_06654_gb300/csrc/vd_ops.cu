@@ -170,6 +170,80 @@ void inv_transform_n(const vd_grid* G, int ncomp, const cpx<T>* in, T* out, cpx<
   launch_xpass<T>(X, g, twtab<T>(G), st);
 }
 
+// grad[j] = F^-1(i k_j a) from the spectrum a; the inverse transforms share their passes (each output gets
+// its own transform's multipliers in the same passes: the bits of separate inverse transforms).  t: two
+// spectral fields; a is overwritten in 3D.
+void gradient_fields(const vd_grid* G, cpx<double>* a, double* const grad[3], cpx<double>* t, cudaStream_t st) {
+  const GridDesc& g = G->g;
+  const int d = g.ndim;
+  const size_t nc = (size_t)g.ncplx;
+  const void* tw = G->tw_d;
+  cpx<double>* T0 = t;
+  cpx<double>* T1 = t + nc;
+  AxisProg P{};
+  P.in[0] = a;
+  P.nxf = 2;
+  P.xf[0] = mkxf(0, 1, MUL_IK, 0, true, true);
+  P.xf[1] = mkxf(0, 0, 0, 0, true, true);
+  P.out[0] = T0;
+  P.out[1] = T1;
+  const cpx<double>* in[3] = {a, T1, T1};
+  if (d >= 2) {   // T0 = F^-1(a), T1 = F^-1(i k a) along the last axis
+    P.axis = d - 1;
+    launch_axis<double>(P, +1, g, tw, st);
+    in[0] = T0;
+  }
+  if (d == 3) {   // along y: a <- F^-1(i k T0), T0 and T1 in place
+    AxisProg Q{};
+    Q.nxf = 3;
+    Q.xf[0] = mkxf(0, 2, MUL_IK, 0, true, true);
+    Q.xf[1] = mkxf(0, 0, 0, 0, true, true);
+    Q.xf[2] = mkxf(1, 1, 0, 0, true, true);
+    Q.in[0] = T0;
+    Q.in[1] = T1;
+    Q.out[0] = T0;
+    Q.out[1] = T1;
+    Q.out[2] = a;
+    Q.axis = 1;
+    launch_axis<double>(Q, +1, g, tw, st);
+    in[1] = a;
+  }
+  XProg X{};
+  X.mode = 2;
+  X.ncomp = d;
+  for (int j = 0; j < d; ++j) {
+    X.in[j] = in[j];
+    X.out[j] = grad[j];
+  }
+  X.pre[0] = MUL_IK;
+  X.scale = 1.0 / (double)g.nreal;
+  launch_xpass<double>(X, g, tw, st);
+}
+
+// a_0 <- sum_j i k~_j a_j (d spectral fields back to back)
+__global__ void k_divergence(GridDesc g, cpx<double>* __restrict__ a) {
+  pdl_wait();
+  const int nc = (int)g.ncplx;
+  for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < nc; e += gridDim.x * blockDim.x) {
+    const int line = e / g.h0;
+    const int idx[3] = {e - line * g.h0, line % g.n1, line / g.n1};
+    const int n[3] = {g.n0, g.n1, g.n2};
+    cpx<double> s = mk<double>(0.0, 0.0);
+    for (int j = 0; j < g.ndim; ++j) {
+      const double k = g.kfac[j] * (double)freq_tilde(idx[j], n[j]);
+      const cpx<double> v = a[(size_t)j * g.ncplx + e];
+      s = mk<double>(fma(-k, v.y, s.x), fma(k, v.x, s.y));
+    }
+    a[e] = s;
+  }
+}
+
+void divergence_spec(const vd_grid* G, cpx<double>* a, cudaStream_t st) {
+  const int blocks = (int)std::min<long long>((G->g.ncplx + 255) / 256, 4096);
+  pdl_launch(k_divergence, blocks, 256, 0, st, G->g, a);
+  count_launch();
+}
+
 // First and second derivatives of a field from its spectrum rh (double): grad[j] = F^-1(i k_j rh),
 // hess[hidx(a, b)] = F^-1((i k_a)(i k_b) rh).  The inverse transforms sharing a z multiplier
 // share their z and y passes (each output gets its own transform's multipliers in the same

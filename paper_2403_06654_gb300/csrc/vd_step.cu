@@ -184,15 +184,12 @@ static int ewb(long long n) { return (int)std::max<long long>(1, std::min<long l
 
 static size_t a256(size_t x) { return (x + 255) & ~(size_t)255; }
 
-// physical gradient of a scalar field into d fields (spectral scratch: 2 fields)
-static void grad_phys(const vd_grid* G, const double* f, double* out, cpx<double>* s0, cpx<double>* s1,
-                      cudaStream_t st) {
-  fwd_transform<double>(G, f, s0, st);
-  for (int j = 0; j < G->g.ndim; ++j) {
-    Mult m;
-    m.deriv[j] = 1;
-    inv_transform<double>(G, s0, m, out + (size_t)j * G->g.nreal, s1, st);
-  }
+// physical gradient of a field, from its spectrum s0, into d fields (s0 is overwritten in 3D; t: two
+// spectral fields)
+static void grad_phys(const vd_grid* G, cpx<double>* s0, double* out, cpx<double>* t, cudaStream_t st) {
+  double* grad[3];
+  for (int j = 0; j < 3; ++j) grad[j] = out + (size_t)j * G->g.nreal;
+  gradient_fields(G, s0, grad, t, st);
 }
 
 }  // namespace vd
@@ -403,7 +400,8 @@ vd_status vd_flow_step(vd_flow* F, double dt, vd_step_info* info, vd_stream stre
   vd_status e;
 
   // 1. mass equation
-  grad_phys(G, F->rho, F->grad, s0, s1, st);
+  fwd_transform<double>(G, F->rho, s0, st);
+  grad_phys(G, s0, F->grad, s1, st);
   { pdl_launch(k_dotvec, b, 256, 0, st, n, d, F->u, F->grad, F->nrho); count_launch(); }
   const double* ab = F->nrho;
   if (F->have_prev) {
@@ -414,7 +412,7 @@ vd_status vd_flow_step(vd_flow* F, double dt, vd_step_info* info, vd_stream stre
     { pdl_launch(k_lin, b, 256, 0, st, n, 1.0, ab, -1.0, F->msrc, F->fphi); count_launch(); }
     ab = F->fphi;
   }
-  fwd_transform<double>(G, F->rho, s0, st);
+  if (d == 3) fwd_transform<double>(G, F->rho, s0, st);   // (else s0 still holds it)
   fwd_transform<double>(G, ab, s1, st);
   const double c = dt / (2.0 * p.Re * p.Sc);
   { pdl_launch(k_mass, ewb(g.ncplx), 256, 0, st, g, c, dt, s0, s1, s2); count_launch(); }
@@ -429,8 +427,9 @@ vd_status vd_flow_step(vd_flow* F, double dt, vd_step_info* info, vd_stream stre
   // 3. predictor
   const double a = dt / (2.0 * p.Re);
   const vd_op_params opp{a, 1.0 / p.Sc};
+  fwd_transform_n<double>(G, d, F->u, s0, st);   // (temporaries: the solve workspace, free here)
   for (int i = 0; i < d; ++i) {
-    grad_phys(G, F->u + i * n, F->grad, s0, s1, st);
+    grad_phys(G, s0 + (size_t)i * g.ncplx, F->grad, reinterpret_cast<cpx<double>*>(F->ws), st);
     { pdl_launch(k_dotvec, b, 256, 0, st, n, d, F->u, F->grad, F->nu + i * n); count_launch(); }
   }
   const double* abu = F->nu;
@@ -487,13 +486,9 @@ vd_status vd_flow_step(vd_flow* F, double dt, vd_step_info* info, vd_stream stre
   if (e != VD_OK) return e;
   { pdl_launch(k_lin, ewb(n * d), 256, 0, st, n * d, 1.0, F->w, -1.0, F->hz, F->hz); count_launch(); }
   { pdl_launch(k_mul_by, b, 256, 0, st, n, d, F->hz, F->rho_h, F->hz); count_launch(); }
-  for (int j = 0; j < d; ++j) fwd_transform<double>(G, F->hz + (size_t)j * n, s0 + (size_t)j * g.ncplx, st);
+  fwd_transform_n<double>(G, d, F->hz, s0, st);
   { pdl_launch(k_grad_part, ewb(g.ncplx), 256, 0, st, g, d, s0); count_launch(); }
-  for (int j = 0; j < d; ++j) {
-    Mult m;
-    inv_transform<double>(G, s0 + (size_t)j * g.ncplx, m, F->w + (size_t)j * n, reinterpret_cast<cpx<double>*>(F->ws),
-                          st);
-  }
+  inv_transform_n<double>(G, d, s0, F->w, reinterpret_cast<cpx<double>*>(F->ws), st);
   { pdl_launch(k_gradp, b, 256, 0, st, n, d, F->grad, F->w, F->gradp); count_launch(); }
   { pdl_launch(k_project, b, 256, 0, st, n, d, F->ustar, F->grad, F->rho_h, dt, F->u); count_launch(); }
   // history and new density
