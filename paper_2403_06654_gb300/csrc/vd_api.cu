@@ -65,6 +65,32 @@ static void wide_search(int n, int least, int most, WidePlan* cur, WidePlan* bes
       --cur->nst;
     }
 }
+// Threads per line for W lines per block: the fewest warp slots (a stage of nb butterflies takes
+// ceil(nb / t) rounds of its radix; a warp without butterflies costs nothing, a part-filled one all),
+// with a surcharge per extra round (the rounds are the latency of the block).
+static int wide_tpl(const WidePlan& pl, int W) {
+  const int most = std::max(1, kWideThreads / W);
+  int best = 1;
+  double cost = -1;
+  for (int t = 1; t <= most && t <= pl.n; ++t) {
+    double c = 0;
+    int extra = 0;
+    for (int s = 0; s < pl.nst; ++s) {
+      const int nb = pl.n / pl.rad[s];
+      for (int done = 0; done < nb; done += t) {
+        c += (double)((W * std::min(t, nb - done) + 31) / 32) * pl.rad[s];
+        extra += done > 0 ? 1 : 0;
+      }
+    }
+    c *= 1.0 + 0.08 * extra;
+    if (cost < 0 || c < cost) {
+      cost = c;
+      best = t;
+    }
+  }
+  return best;
+}
+
 bool make_wide_plans(int n, int tw_off, WidePlan p[kWideClasses]) {
   for (int k = 0; k < kWideClasses; ++k) {
     WidePlan cur{}, best{};
@@ -77,6 +103,7 @@ bool make_wide_plans(int n, int tw_off, WidePlan p[kWideClasses]) {
     p[k] = best;
     p[k].n = (int16_t)n;
     p[k].tw_off = tw_off;
+    for (int l = 0; l < 7; ++l) p[k].tpl[l] = (int16_t)wide_tpl(p[k], 1 << l);
   }
   return true;
 }

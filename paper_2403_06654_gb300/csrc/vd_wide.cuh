@@ -27,8 +27,6 @@
 
 namespace vd {
 
-constexpr int kWideThreads = 256;   // most threads per block
-
 // ---------------------------------------------------------------------------------------
 // codelets of the composite radices (S = -1 forward, +1 inverse)
 // ---------------------------------------------------------------------------------------
@@ -547,39 +545,13 @@ __global__ void __launch_bounds__(kWideThreads, (sizeof(T) == 8 ? 2 : 3))
 // launches
 // ---------------------------------------------------------------------------------------
 
-// Threads per line for W lines per block: the fewest warp slots (a stage of nb butterflies takes
-// ceil(nb / t) rounds of its radix; a warp without butterflies costs nothing, a part-filled one all),
-// with a surcharge per extra round (the rounds are the latency of the block).
-inline int wide_tpl(const WidePlan& pl, int W) {
-  const int most = std::max(1, kWideThreads / W);
-  int best = 1;
-  double cost = -1;
-  for (int t = 1; t <= most && t <= pl.n; ++t) {
-    double c = 0;
-    int extra = 0;
-    for (int s = 0; s < pl.nst; ++s) {
-      const int nb = pl.n / pl.rad[s];
-      for (int done = 0; done < nb; done += t) {
-        c += (double)((W * std::min(t, nb - done) + 31) / 32) * pl.rad[s];
-        extra += done > 0 ? 1 : 0;
-      }
-    }
-    c *= 1.0 + 0.08 * extra;
-    if (cost < 0 || c < cost) {
-      cost = c;
-      best = t;
-    }
-  }
-  return best;
-}
-
 template <typename T, int S>
 static void wide_axis_launch(const AxisProg& P, const GridDesc& g, const cpx<T>* tw, int W, int groups,
                              cudaStream_t st) {
   const int cls = wide_class(sizeof(T), (long long)g.ncplx);
   const WidePlan& pl = (P.axis == 2 ? g.wz : g.wy)[cls];
   const long long lines = (long long)g.h0 * (P.axis == 2 ? g.n1 : g.n2);
-  const int tpl = wide_tpl(pl, W);
+  const int tpl = pl.tpl[wide_log2(W)];
   const size_t smem = wide_axis_smem(pl, W, sizeof(T));
   const bool pad = W * (int)sizeof(cpx<T>) < 128;
   auto kernel = pad ? k_axis_w<T, S, true> : k_axis_w<T, S, false>;
