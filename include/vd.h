@@ -409,8 +409,9 @@ vd_status vd_batch_destroy(vd_batch* batch);
  * the solvers use (y and z passes in both directions; the x pass forward, inverse and fused)
  * is timed with CUDA events on `scratch` (device, vd_autotune_bytes(grid) bytes, caller-owned,
  * overwritten) for each candidate shape: the register-resident four-step kernel where one
- * exists, and the shared-memory Stockham engine with 1, 2, 4, ... lines per block up to the
- * shared-memory limit.  The fastest shape goes into a process-wide table keyed by (pass, type,
+ * exists, and the general kernel of the type (float and double: wide-radix Stockham stages from
+ * and to global memory; float pairs: the shared-memory Stockham engine) with 1, 2, 4, ... lines
+ * per block up to the shared-memory limit.  The fastest shape goes into a process-wide table keyed by (pass, type,
  * length, axis, direction or x-pass form) that every later launch on any grid consults; with
  * the environment variable VD_TUNE_FILE set the table is written to that file, and read from
  * it at the first launch or query of a later process.  Synchronises `stream`.  Shapes change

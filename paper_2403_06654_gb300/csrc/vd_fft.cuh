@@ -1,4 +1,5 @@
-// Shared-memory Stockham FFT engine (device side).
+// Shared-memory Stockham FFT engine (device side): the float-pair passes of vd_passes.cu.  Float and
+// double passes take its codelets into wide-radix stages of their own (vd_wide.cuh).
 //
 // A transform of length n = R_0 R_1 ... R_{s-1} runs s radix stages between two shared
 // memory buffers (ping-pong).  Stage with radix R and span p (product of the radices before
@@ -253,14 +254,5 @@ __device__ __forceinline__ double recip(double x) {
   return fma(r, e, r);
 }
 __device__ __forceinline__ float recip(float x) { return __frcp_rn(x); }
-
-// diagonal symbol value for |k~|^2 = k2 (corner modes have k2 == 0 exactly)
-template <typename T>
-__device__ __forceinline__ T symbol_value(int kind, T a, T k2) {
-  if (kind == SYM_PRESSURE) return (k2 == T(0)) ? T(0) : -recip(k2);
-  if (kind == SYM_VELOCITY) return recip(T(1) + a * k2);
-  if (kind == SYM_PROJECT) return (k2 == T(0)) ? T(0) : T(1);
-  return T(1);
-}
 
 }  // namespace vd

@@ -27,11 +27,6 @@ namespace vd {
 // reduction machinery
 // ---------------------------------------------------------------------------------------
 
-__device__ __forceinline__ double wgt(long long e, int h0) {
-  const int kx = (int)(e % h0);
-  return (kx == 0 || kx == h0 - 1) ? 1.0 : 2.0;
-}
-
 template <typename T>
 __device__ __forceinline__ cpx<double> ld(const cpx<T>* p, long long e) {
   const cpx<T> v = p[e];

@@ -4,12 +4,13 @@
 // passes in both directions, and the x pass in its three forms (forward real-to-half-spectrum,
 // inverse, and the fused inverse-weight-forward form of the operators) -- is timed with CUDA
 // events (median of seven launches) for each candidate shape: the register-resident four-step
-// kernel where one exists (float, lengths 128 and 256; x pass n0 = 128, 256, 512) and the
-// Stockham engine with 1, 2, 4, ... lines per block up to the shared-memory limit.  A shape
+// kernel where one exists (float, lengths 128 and 256; x pass n0 = 128, 256, 512) and the general
+// kernel of the type (float and double: the wide-radix passes of vd_wide.cuh; float pairs: the
+// Stockham engine) with 1, 2, 4, ... lines per block up to the shared-memory limit.  A shape
 // replaces the built-in choice only when it is at least 3% faster; the winner goes into the
 // process-wide launch table that every later launch consults (and, with VD_TUNE_FILE set, into
 // that file).  Shapes change only the work distribution, never the arithmetic of a line,
-// except that the register kernel and the Stockham engine round differently (both are
+// except that the register kernel and the general ones round differently (both are
 // complete transforms; the parity tests hold for either).
 #include "vd_internal.h"
 #include "vd_dd.cuh"
