@@ -1504,10 +1504,9 @@ void ensure_smem(const void* func, size_t smem) {
   static std::map<const void*, size_t> set;
   std::lock_guard<std::mutex> lk(mu);
   size_t& cur = set[func];
-  if (smem > cur) {
-    cudaFuncSetAttribute(func, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  // (a refused size is not recorded: smaller ones still have to be opted into)
+  if (smem > cur && cudaFuncSetAttribute(func, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) == cudaSuccess)
     cur = smem;
-  }
 }
 
 // The plan of radices up to 5 of a length, in the Stockham engine's form: float pairs of the lengths that
@@ -1662,6 +1661,19 @@ static int split_xpass(const XProg& P, long long blocks) {
   return P.ncomp;
 }
 
+// A table entry as this plan can run it: an entry of so many lines per block that they do not fit the
+// block's shared memory here counts as absent.  Entries are set by length alone (by hand, from a file),
+// but the bytes of a line also depend on the radix class, that is on the field's size: 32 double lines
+// of 256 points take 145 KB in radix 16 and 301 KB in radices up to 5.
+template <typename T>
+static int entry_for_plan(int choice, int kind, const FftPlan& pl, const WidePlan& wide) {
+  if (choice <= 0 || choice > 64) return choice;
+  size_t need = shape_smem(kind, type_code<T>(), pl, wide, choice);
+  if (std::is_same<T, dd>::value && !p_plan_ok(pl, kThreads / choice))   // without the packed tables
+    need -= sizeof(pdd) * (size_t)pl.n * (kind == 0 ? 1 : 3);
+  return need <= kSmemMost ? choice : -1;
+}
+
 template <typename T>
 void launch_axis(const AxisProg& P0, int dir, const GridDesc& g, const void* tw, cudaStream_t st) {
   AxisProg P = P0;
@@ -1675,10 +1687,10 @@ void launch_axis(const AxisProg& P0, int dir, const GridDesc& g, const void* tw,
     inner_n = g.h0;
     outer_n = g.n2;
   }
-  int choice = tune_get(0, type_code<T>(), n, P.axis, dir);
   const bool reg_ok = std::is_same<T, float>::value && (n == 256 || n == 128);
   const FftPlan& pl = P.axis == 2 ? g.pz : g.py;
   const WidePlan& wide = (P.axis == 2 ? g.wz : g.wy)[wide_class(sizeof(T), g.ncplx)];
+  int choice = entry_for_plan<T>(tune_get(0, type_code<T>(), n, P.axis, dir), 0, pl, wide);
   if (choice < 0) choice = default_shape(0, type_code<T>(), pl, wide, P.axis, inner_n * outer_n);
   if (choice == kChoiceStaged && !(reg_ok && tma_program_ok(P, g))) choice = 0;   // not applicable: register kernel
   const int W = (choice > 0 && choice <= 64) ? choice : axis_lines(type_code<T>(), pl, wide, inner_n * outer_n);
@@ -1784,10 +1796,11 @@ void launch_xpass(const XProg& P0, const GridDesc& g, const void* tw, cudaStream
   split_scale(P.scale, &P.scale_hi, &P.scale_lo);
   split_scale(P.aux_scale, &P.aux_scale_hi, &P.aux_scale_lo);
   const int m = g.n0 / 2;
-  int choice = tune_get(1, type_code<T>(), m, 0, P.mode);
   const long long nlines = (long long)g.n1 * g.n2;
-  if (choice < 0) choice = default_shape(1, type_code<T>(), g.px, g.wx[wide_class(sizeof(T), g.ncplx)], 0, nlines);
-  const int L = (choice > 0 && choice <= 64) ? choice : x_lines(type_code<T>(), g.px, g.wx[wide_class(sizeof(T), g.ncplx)], nlines);
+  const WidePlan& wide = g.wx[wide_class(sizeof(T), g.ncplx)];
+  int choice = entry_for_plan<T>(tune_get(1, type_code<T>(), m, 0, P.mode), 1, g.px, wide);
+  if (choice < 0) choice = default_shape(1, type_code<T>(), g.px, wide, 0, nlines);
+  const int L = (choice > 0 && choice <= 64) ? choice : x_lines(type_code<T>(), g.px, wide, nlines);
   const double fc = (double)g.ncplx * sizeof(cpx<T>), fr = (double)g.nreal * sizeof(T);
   double bytes = 0, flops = 0;
   const double real_fft = (double)g.nreal * 2.5 * std::log2((double)g.n0);   // one real transform of every line

@@ -106,6 +106,8 @@ int tune_table(int* out, int max);   // 6 ints per entry; returns the entry coun
 int default_shape(int kind, int type, const FftPlan& pl, const WidePlan& wide, int axis, long long lines);
 void tune_save();                    // write the table to $VD_TUNE_FILE (if set)
 
+// most dynamic shared memory of a block (227 KB)
+constexpr size_t kSmemMost = 227 * 1024;
 // opt a kernel into more than 48 KB of dynamic shared memory (once per size)
 void ensure_smem(const void* func, size_t smem);
 int sm_count();
