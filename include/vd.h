@@ -412,9 +412,10 @@ vd_status vd_batch_destroy(vd_batch* batch);
  * exists, and the general kernel of the type (float and double: wide-radix Stockham stages from
  * and to global memory; float pairs: the shared-memory Stockham engine) with 1, 2, 4, ... lines
  * per block up to the shared-memory limit.  The fastest shape goes into a process-wide table keyed by (pass, type,
- * length, axis, direction or x-pass form) that every later launch on any grid consults; with
- * the environment variable VD_TUNE_FILE set the table is written to that file, and read from
- * it at the first launch or query of a later process.  Synchronises `stream`.  Shapes change
+ * length, axis, direction or x-pass form) for later launches on fields of about this size (the same
+ * radices, a line count within the same power of two); with the environment variable
+ * VD_TUNE_FILE set the table is written to that file, and read from it at the first launch or
+ * query of a later process (files whose entries name no field size hold for every field).  Synchronises `stream`.  Shapes change
  * the work distribution only; results stay within the parity bounds.  The event profiler must
  * be off while tuning.
  */
@@ -427,7 +428,9 @@ vd_status vd_autotune(const vd_grid* grid, int precisions, void* scratch, size_t
  * engine gives the same bits); writes at most max entries to out (may be null) and returns the
  * total count */
 int vd_autotune_table(int* out, int max);
-/* set one entry by hand (choice < 0 erases it); INVALID_ARG on a bad key or choice */
+/* set one entry by hand, for every field size (choice < 0 erases it, and what the tuner found for
+ * that key); INVALID_ARG on a bad key or choice.  Lines per block beyond a field's shared-memory
+ * limit give the built-in shape there. */
 vd_status vd_autotune_set(int kind, int type, int n, int axis, int dir, int choice);
 
 /*

@@ -1400,9 +1400,10 @@ static void launch_xpass_r(const XProg& P, const GridDesc& g, const cpx<T>* tw, 
 
 // ---------------------------------------------------------------------------------------
 // launch-shape table, filled by the autotuner (vd_autotune) and consulted by every launch:
-// choice 0 = register-resident four-step kernel, > 0 = lines per block of the Stockham
-// engine; absent = the built-in heuristic.  Optionally persisted in the file named by the
-// environment variable VD_TUNE_FILE (one entry per line: kind type length axis dir choice).
+// choice 0 = register-resident four-step kernel, > 0 = lines per block of the type's general
+// kernel; absent = the built-in heuristic.  Optionally persisted in the file named by the
+// environment variable VD_TUNE_FILE, one entry per line: kind type length axis dir choice, and for
+// the tuner's entries their scope and whether the built-in shape won (0 / 1).
 // ---------------------------------------------------------------------------------------
 
 template <typename T>
@@ -1411,12 +1412,18 @@ constexpr int type_code() {
 }
 
 static std::mutex g_tune_mu;
-static std::map<long long, int> g_tune;
+struct TuneEntry {
+  int choice;
+  bool builtin;
+};
+static std::map<long long, TuneEntry> g_tune;
 static bool g_tune_loaded = false;
+constexpr int kTuneScopes = 1 + 32 * kWideClasses;
 
-static long long tune_key(int kind, int type, int n, int axis, int dir) {
-  return ((long long)kind << 48) | ((long long)type << 40) | ((long long)(axis & 0xff) << 32) |
-         ((long long)((dir + 4) & 0xff) << 24) | (long long)(n & 0xffffff);
+// (the scopes of a key are neighbours)
+static long long tune_key(int kind, int type, int n, int axis, int dir, int scope) {
+  return ((long long)kind << 56) | ((long long)type << 48) | ((long long)(axis & 0xff) << 40) |
+         ((long long)((dir + 4) & 0xff) << 32) | ((long long)(n & 0xffffff) << 8) | (long long)(scope & 0xff);
 }
 
 static void tune_load_locked() {
@@ -1426,24 +1433,38 @@ static void tune_load_locked() {
   if (!path) return;
   FILE* f = std::fopen(path, "r");
   if (!f) return;
-  int kind, type, n, axis, dir, choice;
-  while (std::fscanf(f, "%d %d %d %d %d %d", &kind, &type, &n, &axis, &dir, &choice) == 6)
-    g_tune[tune_key(kind, type, n, axis, dir)] = choice;
+  char line[256];
+  while (std::fgets(line, sizeof line, f)) {
+    int kind, type, n, axis, dir, choice, scope = 0, builtin = 0;
+    const int got = std::sscanf(line, "%d %d %d %d %d %d %d %d", &kind, &type, &n, &axis, &dir, &choice, &scope, &builtin);
+    if (got != 6 && got != 8) continue;
+    if (scope < 0 || scope >= kTuneScopes) continue;
+    g_tune[tune_key(kind, type, n, axis, dir, scope)] = {choice, builtin != 0};
+  }
   std::fclose(f);
 }
 
-int tune_get(int kind, int type, int n, int axis, int dir) {
+int tune_get(int kind, int type, int n, int axis, int dir, int scope) {
   std::lock_guard<std::mutex> lk(g_tune_mu);
   tune_load_locked();
-  auto it = g_tune.find(tune_key(kind, type, n, axis, dir));
-  return it == g_tune.end() ? -1 : it->second;
+  if (g_tune.empty()) return -1;
+  auto it = g_tune.find(tune_key(kind, type, n, axis, dir, scope));
+  if (it == g_tune.end()) it = g_tune.find(tune_key(kind, type, n, axis, dir, 0));
+  return it == g_tune.end() || it->second.builtin ? -1 : it->second.choice;
 }
 
 void tune_set(int kind, int type, int n, int axis, int dir, int choice) {
   std::lock_guard<std::mutex> lk(g_tune_mu);
   tune_load_locked();
-  if (choice < 0) g_tune.erase(tune_key(kind, type, n, axis, dir));
-  else g_tune[tune_key(kind, type, n, axis, dir)] = choice;
+  g_tune.erase(g_tune.lower_bound(tune_key(kind, type, n, axis, dir, 0)),
+               g_tune.upper_bound(tune_key(kind, type, n, axis, dir, 0xff)));
+  if (choice >= 0) g_tune[tune_key(kind, type, n, axis, dir, 0)] = {choice, false};
+}
+
+void tune_put(int kind, int type, int n, int axis, int dir, int scope, int choice, bool builtin) {
+  std::lock_guard<std::mutex> lk(g_tune_mu);
+  tune_load_locked();
+  g_tune[tune_key(kind, type, n, axis, dir, scope)] = {choice, builtin};
 }
 
 int default_shape(int kind, int type, const FftPlan& pl, const WidePlan& wide, int axis, long long lines) {
@@ -1469,12 +1490,12 @@ int tune_table(int* out, int max) {
     if (out && k < max) {
       const long long key = kv.first;
       int* e = out + 6 * k;
-      e[0] = (int)(key >> 48);
-      e[1] = (int)((key >> 40) & 0xff);
-      e[2] = (int)(key & 0xffffff);
-      e[3] = (int)((key >> 32) & 0xff);
-      e[4] = (int)((key >> 24) & 0xff) - 4;
-      e[5] = kv.second;
+      e[0] = (int)(key >> 56);
+      e[1] = (int)((key >> 48) & 0xff);
+      e[2] = (int)((key >> 8) & 0xffffff);
+      e[3] = (int)((key >> 40) & 0xff);
+      e[4] = (int)((key >> 32) & 0xff) - 4;
+      e[5] = kv.second.choice;
     }
     ++k;
   }
@@ -1489,8 +1510,10 @@ void tune_save() {
   if (!f) return;
   for (const auto& kv : g_tune) {
     const long long key = kv.first;
-    std::fprintf(f, "%d %d %d %d %d %d\n", (int)(key >> 48), (int)((key >> 40) & 0xff), (int)(key & 0xffffff),
-                 (int)((key >> 32) & 0xff), (int)((key >> 24) & 0xff) - 4, kv.second);
+    std::fprintf(f, "%d %d %d %d %d %d", (int)(key >> 56), (int)((key >> 48) & 0xff), (int)((key >> 8) & 0xffffff),
+                 (int)((key >> 40) & 0xff), (int)((key >> 32) & 0xff) - 4, kv.second.choice);
+    if (key & 0xff) std::fprintf(f, " %d %d", (int)(key & 0xff), kv.second.builtin ? 1 : 0);
+    std::fprintf(f, "\n");
   }
   std::fclose(f);
 }
@@ -1662,8 +1685,8 @@ static int split_xpass(const XProg& P, long long blocks) {
 }
 
 // A table entry as this plan can run it: an entry of so many lines per block that they do not fit the
-// block's shared memory here counts as absent.  Entries are set by length alone (by hand, from a file),
-// but the bytes of a line also depend on the radix class, that is on the field's size: 32 double lines
+// block's shared memory here counts as absent.  Entries set by hand or read from an older file go by length
+// alone, but the bytes of a line also depend on the radix class, that is on the field's size: 32 double lines
 // of 256 points take 145 KB in radix 16 and 301 KB in radices up to 5.
 template <typename T>
 static int entry_for_plan(int choice, int kind, const FftPlan& pl, const WidePlan& wide) {
@@ -1689,8 +1712,10 @@ void launch_axis(const AxisProg& P0, int dir, const GridDesc& g, const void* tw,
   }
   const bool reg_ok = std::is_same<T, float>::value && (n == 256 || n == 128);
   const FftPlan& pl = P.axis == 2 ? g.pz : g.py;
-  const WidePlan& wide = (P.axis == 2 ? g.wz : g.wy)[wide_class(sizeof(T), g.ncplx)];
-  int choice = entry_for_plan<T>(tune_get(0, type_code<T>(), n, P.axis, dir), 0, pl, wide);
+  const int cls = wide_class(sizeof(T), g.ncplx);
+  const WidePlan& wide = (P.axis == 2 ? g.wz : g.wy)[cls];
+  int choice = entry_for_plan<T>(
+      tune_get(0, type_code<T>(), n, P.axis, dir, tune_scope(cls, inner_n * outer_n)), 0, pl, wide);
   if (choice < 0) choice = default_shape(0, type_code<T>(), pl, wide, P.axis, inner_n * outer_n);
   if (choice == kChoiceStaged && !(reg_ok && tma_program_ok(P, g))) choice = 0;   // not applicable: register kernel
   const int W = (choice > 0 && choice <= 64) ? choice : axis_lines(type_code<T>(), pl, wide, inner_n * outer_n);
@@ -1797,8 +1822,9 @@ void launch_xpass(const XProg& P0, const GridDesc& g, const void* tw, cudaStream
   split_scale(P.aux_scale, &P.aux_scale_hi, &P.aux_scale_lo);
   const int m = g.n0 / 2;
   const long long nlines = (long long)g.n1 * g.n2;
-  const WidePlan& wide = g.wx[wide_class(sizeof(T), g.ncplx)];
-  int choice = entry_for_plan<T>(tune_get(1, type_code<T>(), m, 0, P.mode), 1, g.px, wide);
+  const int cls = wide_class(sizeof(T), g.ncplx);
+  const WidePlan& wide = g.wx[cls];
+  int choice = entry_for_plan<T>(tune_get(1, type_code<T>(), m, 0, P.mode, tune_scope(cls, nlines)), 1, g.px, wide);
   if (choice < 0) choice = default_shape(1, type_code<T>(), g.px, wide, 0, nlines);
   const int L = (choice > 0 && choice <= 64) ? choice : x_lines(type_code<T>(), g.px, wide, nlines);
   const double fc = (double)g.ncplx * sizeof(cpx<T>), fr = (double)g.nreal * sizeof(T);

@@ -93,14 +93,25 @@ void launch_xpass(const XProg& P, const GridDesc& g, const void* tw, cudaStream_
 // launch-shape table (vd_passes.cu).  kind 0: y/z pass (key: type, length, axis, direction);
 // kind 1: x pass (key: type, n0/2, axis 0, mode).  type: 0 double, 1 float, 2 float-pair.
 // choice: 0 register four-step kernel, > 0 lines per block, < 0 (get) absent / (set) erase.
+// Entries set by hand (tune_set) hold for every field; the tuner's (tune_put) for fields of the tuned one's
+// scope: the same radix class and a line count within the same power of two.  The bytes of a shape
+// depend on the class and the better shape on the line count: the 16-line blocks and register kernels
+// that win on 256^3 leave most SMs idle on a 256^2 field.  A scoped entry goes before one set by hand.
 // kind 0 choice kChoiceStaged: the register kernel with TMA-staged input (float y/z passes of
 // length 128 / 256).  Type 2 choice kChoiceUnpacked (either kind): the Stockham engine on
 // unpacked float pairs with the default lines per block, instead of the packed engine that the
 // float-pair passes use for lengths whose radices are 2, 4 and 8 (same results, bit for bit).
 constexpr int kChoiceStaged = 128;
 constexpr int kChoiceUnpacked = 256;
-int tune_get(int kind, int type, int n, int axis, int dir);
-void tune_set(int kind, int type, int n, int axis, int dir, int choice);
+int tune_get(int kind, int type, int n, int axis, int dir, int scope);
+void tune_set(int kind, int type, int n, int axis, int dir, int choice);   // replaces the scoped ones too
+// builtin: the built-in shape is the best of this scope (choice: which one that was, for the listing)
+void tune_put(int kind, int type, int n, int axis, int dir, int scope, int choice, bool builtin);
+inline int tune_scope(int cls, long long lines) {
+  int l = 0;
+  while ((lines >> (l + 1)) > 0) ++l;
+  return 1 + 32 * cls + l;   // 0: every field
+}
 int tune_table(int* out, int max);   // 6 ints per entry; returns the entry count
 // the built-in choice for a pass of `lines` lines in all (kind 1: n = n0/2)
 int default_shape(int kind, int type, const FftPlan& pl, const WidePlan& wide, int axis, long long lines);

@@ -8,8 +8,8 @@
 // kernel of the type (float and double: the wide-radix passes of vd_wide.cuh; float pairs: the
 // Stockham engine) with 1, 2, 4, ... lines per block up to the shared-memory limit.  A shape
 // replaces the built-in choice only when it is at least 3% faster; the winner goes into the
-// process-wide launch table that every later launch consults (and, with VD_TUNE_FILE set, into
-// that file).  Shapes change only the work distribution, never the arithmetic of a line,
+// process-wide launch table for the launches of fields of this one's scope (radix class and, within a
+// power of two, line count) and, with VD_TUNE_FILE set, into that file.  Shapes change only the work distribution, never the arithmetic of a line,
 // except that the register kernel and the general ones round differently (both are
 // complete transforms; the parity tests hold for either).
 #include "vd_internal.h"
@@ -100,14 +100,18 @@ vd_status tune_type(const vd_grid* G, const void* tw, void* a, void* b, cudaStre
       P.in[0] = a;
       P.out[0] = b;
       P.axis = axis;
-      // the built-in shape first: the register kernel, else the heuristic tile width
-      tune_set(0, type, n, axis, dir, -1);
+      // the built-in shape first
+      const FftPlan& pl = axis == 2 ? g.pz : g.py;
+      const WidePlan& wide = (axis == 2 ? g.wz : g.wy)[cls];
+      const long long lines = inner * (axis == 2 ? 1 : g.n2);
+      const int scope = tune_scope(cls, lines), own = default_shape(0, type, pl, wide, axis, lines);
+      tune_put(0, type, n, axis, dir, scope, own, true);
       float tdef = time_it([&] { launch_axis<T>(P, dir, g, tw, st); }, st, tm);
       VD_CUDA(cudaGetLastError());
       int best = -1;
       float tbest = tdef * kSwitchGain;
       for (int c : cand) {
-        tune_set(0, type, n, axis, dir, c);
+        tune_put(0, type, n, axis, dir, scope, c, false);
         const float ms = time_it([&] { launch_axis<T>(P, dir, g, tw, st); }, st, tm);
         VD_CUDA(cudaGetLastError());
         if (ms < tbest) {
@@ -115,9 +119,7 @@ vd_status tune_type(const vd_grid* G, const void* tw, void* a, void* b, cudaStre
           best = c;
         }
       }
-      (void)reg;
-      tune_set(0, type, n, axis, dir, best >= 0 ? best : default_shape(0, type, axis == 2 ? g.pz : g.py, (axis == 2 ? g.wz : g.wy)[cls], axis,
-                                                                        inner * (axis == 2 ? 1 : g.n2)));
+      tune_put(0, type, n, axis, dir, scope, best >= 0 ? best : own, best < 0);
     }
   }
   // x pass: forward (mode 1), inverse (mode 2), fused (mode 0 with a weight field)
@@ -141,13 +143,14 @@ vd_status tune_type(const vd_grid* G, const void* tw, void* a, void* b, cudaStre
     X.out[0] = (mode == 2) ? a : b;
     X.wfield = (mode == 0) ? a : nullptr;
     X.scale = (mode == 2) ? 1.0 / (double)g.nreal : 0.5;
-    tune_set(1, type, m, 0, mode, -1);
+    const int scope = tune_scope(cls, nlines), own = default_shape(1, type, g.px, g.wx[cls], 0, nlines);
+    tune_put(1, type, m, 0, mode, scope, own, true);
     const float tdef = time_it([&] { launch_xpass<T>(X, g, tw, st); }, st, tm);
     VD_CUDA(cudaGetLastError());
     int best = -1;
     float tbest = tdef * kSwitchGain;
     for (int c : cm) {
-      tune_set(1, type, m, 0, mode, c);
+      tune_put(1, type, m, 0, mode, scope, c, false);
       const float ms = time_it([&] { launch_xpass<T>(X, g, tw, st); }, st, tm);
       VD_CUDA(cudaGetLastError());
       if (ms < tbest) {
@@ -155,7 +158,7 @@ vd_status tune_type(const vd_grid* G, const void* tw, void* a, void* b, cudaStre
         best = c;
       }
     }
-    tune_set(1, type, m, 0, mode, best >= 0 ? best : default_shape(1, type, g.px, g.wx[cls], 0, nlines));
+    tune_put(1, type, m, 0, mode, scope, best >= 0 ? best : own, best < 0);
   }
   return VD_OK;
 }
