@@ -536,6 +536,18 @@ vd_status vd_density_set(vd_grid* G, vd_op op, const double* rho, void* ws, size
       }
     derivative_fields(G, rh, grad, hess, tmp, st);
     VD_CUDA(cudaGetLastError());
+    // The float bracket may split the data into float pairs where 1/(N rho), rho and its derivatives (at
+    // most k^2 sqrt(N) max rho by Cauchy-Schwarz, k the largest wavenumber) stay below 2^90, so that a
+    // product with a float field below 2^37 is a float, and no value that counts (a derivative of rho
+    // over the longest wavelength) is so small, 2^-60, that its pair loses bits of the low part.
+    double kmax = 0.0, kmin = 1.0;
+    for (int j = 0; j < d; ++j) {
+      kmax = std::max(kmax, G->g.kfac[j] * (j == 0 ? g.n0 : (j == 1 ? g.n1 : g.n2)) / 2.0);
+      kmin = std::min(kmin, G->g.kfac[j]);
+    }
+    const double most = std::max(1.0, kmax * kmax) * std::sqrt((double)nr) * mx;
+    const double least = kmin * kmin * mn;
+    G->bracket_pairs = most < 0x1p90 && (double)nr * mx < 0x1p90 && least > 0x1p-60;
     G->has_velocity_data = 1;
   }
   G->has_krho_data = 0;

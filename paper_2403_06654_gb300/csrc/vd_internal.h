@@ -30,6 +30,7 @@ struct vd_grid {
   const void* kc_dd = nullptr;
   const void* kw_hat = nullptr;      // cpx<double>, ncplx
   double rho_min = 0, rho_max = 0;
+  int bracket_pairs = 0;   // the velocity data lie well inside the range of floats (see vd_density_set)
   int has_density = 0;
   int has_velocity_data = 0;
   int has_krho_data = 0;

@@ -11,6 +11,7 @@
 #include "vd_dd.cuh"
 
 #include <algorithm>
+#include <cmath>
 #include <type_traits>
 
 namespace vd {
@@ -1064,24 +1065,25 @@ __device__ constexpr int packed_index(int i, int j) {   // i <= j
   return i * D - i * (i - 1) / 2 + (j - i);
 }
 
-// The bracket on double fields, written over lap.
-template <int D>
-__global__ void k_vel_combine(long long nreal, const double* __restrict__ u, const double* __restrict__ du,
-                              double* __restrict__ lap, const double* __restrict__ rho, DensPtrs dp, double inv_sc,
+// The bracket in double, written over lap: double fields, and float fields of densities outside the range
+// of k_vel_combine_f.
+template <typename T, int D>
+__global__ void k_vel_combine(long long nreal, const T* __restrict__ u, const T* __restrict__ du,
+                              T* __restrict__ lap, const double* __restrict__ rho, DensPtrs dp, double inv_sc,
                               const int* done) {
   pdl_wait();
   if (done && *done) return;
   for (long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x; e < nreal;
        e += (long long)gridDim.x * blockDim.x) {
     const double rinv = 1.0 / rho[e];
-    double out[D];
+    T out[D];
 #pragma unroll
     for (int i = 0; i < D; ++i) {
       double t = 0.0;
 #pragma unroll
       for (int j = 0; j < D; ++j)
-        t += u[j * nreal + e] * dp.h[pair_index(i, j)][e] + dp.g[j][e] * du[(i * D + j) * nreal + e];
-      out[i] = rinv * (lap[i * nreal + e] + inv_sc * t);
+        t += (double)u[j * nreal + e] * dp.h[pair_index(i, j)][e] + dp.g[j][e] * (double)du[(i * D + j) * nreal + e];
+      out[i] = (T)(rinv * ((double)lap[i * nreal + e] + inv_sc * t));
     }
 #pragma unroll
     for (int i = 0; i < D; ++i) lap[i * nreal + e] = out[i];
@@ -1140,9 +1142,14 @@ void velocity_combine_launch(const vd_grid* G, int sz, const void* u, const void
   for (int j = 0; j < 6; ++j) dp.h[j] = G->hrho[j];
   const int blocks = (int)std::min<long long>((n + 255) / 256, 4096);
   const int d = G->g.ndim;
+  // (the pairs of inv_sc have the same range)
+  const bool pairs = G->bracket_pairs && (inv_sc == 0.0 || (std::fabs(inv_sc) > 0x1p-30 && std::fabs(inv_sc) < 0x1p30));
   if (sz == 8) {
-    auto k = d == 1 ? k_vel_combine<1> : (d == 2 ? k_vel_combine<2> : k_vel_combine<3>);
+    auto k = d == 1 ? k_vel_combine<double, 1> : (d == 2 ? k_vel_combine<double, 2> : k_vel_combine<double, 3>);
     pdl_launch(k, blocks, 256, 0, st, n, (const double*)u, (const double*)du, (double*)lap, G->rho, dp, inv_sc, done);
+  } else if (!pairs) {
+    auto k = d == 1 ? k_vel_combine<float, 1> : (d == 2 ? k_vel_combine<float, 2> : k_vel_combine<float, 3>);
+    pdl_launch(k, blocks, 256, 0, st, n, (const float*)u, (const float*)du, (float*)lap, G->rho, dp, inv_sc, done);
   } else {
     auto k = d == 1 ? k_vel_combine_f<1> : (d == 2 ? k_vel_combine_f<2> : k_vel_combine_f<3>);
     pdl_launch(k, blocks, 256, 0, st, n, (const float*)u, (const float*)du, (float*)lap, (const dd*)G->rinv_s_dd,
