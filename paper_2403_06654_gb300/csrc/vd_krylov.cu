@@ -502,13 +502,15 @@ struct Acc<float> {
 
 // float(v * s) on the integer and FP32 pipes: v scaled by the power of two in s (exponent bits), split
 // into a float pair, times the rest of s in [1, 2), rounded to float once.  A double multiply and a
-// conversion per value kept k_d2f_scaled at 64 us of 256^3 points against 30 us of memory.  Results
-// below the normal floats are zero.  An s that is no normal double takes the double arithmetic.
+// conversion per value kept k_d2f_scaled at 64 us of 256^3 points against 30 us of memory.  Zeros pass;
+// scaled values outside [2^-74, 2^126), whose pairs or products would lose bits, and an s that is no
+// normal double take the double arithmetic.
 struct Narrow {
   double s;
   float sh, sl;
   int k;   // s = (sh + sl) 2^k
   bool plain;
+  static constexpr int kLeast = 1023 - 74, kEnd = 1023 + 126;   // exponent fields of the float arithmetic
   __device__ __forceinline__ explicit Narrow(double scale) : s(scale) {
     const int hi = __double2hiint(scale), ef = (hi >> 20) & 0x7ff;
     plain = ef == 0 || ef == 0x7ff;
@@ -519,8 +521,11 @@ struct Narrow {
   }
   __device__ __forceinline__ float operator()(double v) const {
     const int hi = __double2hiint(v), ef = (hi >> 20) & 0x7ff, en = ef + k;
-    if (plain || ef == 0x7ff || en >= 0x7ff) return (float)(v * s);
-    if (ef == 0 || en <= 0) return 0.0f;
+    if (plain || ef == 0 || ef == 0x7ff || en < kLeast || en >= kEnd) {
+      if (!plain && ((hi & 0x7fffffff) | __double2loint(v)) == 0)   // a zero with the product's sign
+        return __int_as_float((hi ^ __double2hiint(s)) & (int)0x80000000);
+      return (float)(v * s);
+    }
     const dd d = dd_from_double(__hiloint2double(hi + (k << 20), __double2loint(v)));
     return mul_pair_dd(d, sh, sl);
   }
