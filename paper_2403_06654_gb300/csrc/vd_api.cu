@@ -68,21 +68,18 @@ static void wide_search(int n, int least, int most, WidePlan* cur, WidePlan* bes
 // Threads per line for W lines per block: the fewest warp slots (a stage of nb butterflies takes
 // ceil(nb / t) rounds of its radix; a warp without butterflies costs nothing, a part-filled one all),
 // with a surcharge per extra round (the rounds are the latency of the block).
-static int wide_tpl(const WidePlan& pl, int W) {
+int wide_threads(const WidePlan& pl, int W) {
   const int most = std::max(1, kWideThreads / W);
   int best = 1;
   double cost = -1;
   for (int t = 1; t <= most && t <= pl.n; ++t) {
-    double c = 0;
-    int extra = 0;
+    int slots = 0, extra = 0;
     for (int s = 0; s < pl.nst; ++s) {
-      const int nb = pl.n / pl.rad[s];
-      for (int done = 0; done < nb; done += t) {
-        c += (double)((W * std::min(t, nb - done) + 31) / 32) * pl.rad[s];
-        extra += done > 0 ? 1 : 0;
-      }
+      const int nb = pl.n / pl.rad[s], full = nb / t, rest = nb - full * t;
+      slots += (full * ((W * t + 31) / 32) + (W * rest + 31) / 32) * pl.rad[s];
+      extra += full - (rest > 0 ? 0 : 1);
     }
-    c *= 1.0 + 0.08 * extra;
+    const double c = (double)slots * (1.0 + 0.08 * extra);
     if (cost < 0 || c < cost) {
       cost = c;
       best = t;
@@ -91,19 +88,23 @@ static int wide_tpl(const WidePlan& pl, int W) {
   return best;
 }
 
-bool make_wide_plans(int n, int tw_off, WidePlan p[kWideClasses]) {
+bool make_wide_plan(int n, int tw_off, int cls, WidePlan* p) {
+  WidePlan cur{}, best{};
+  wide_search(n, 2, kWideMost[cls], &cur, &best);
+  if (best.nst == 0) return false;
+  std::sort(best.rad, best.rad + best.nst, [](int a, int b) {
+    const bool pa = (a & (a - 1)) == 0, pb = (b & (b - 1)) == 0;
+    return pa != pb ? pa : a > b;
+  });
+  *p = best;
+  p->n = (int16_t)n;
+  p->tw_off = tw_off;
+  return true;
+}
+static bool make_wide_plans(int n, WidePlan p[kWideClasses]) {
   for (int k = 0; k < kWideClasses; ++k) {
-    WidePlan cur{}, best{};
-    wide_search(n, 2, kWideMost[k], &cur, &best);
-    if (best.nst == 0) return false;
-    std::sort(best.rad, best.rad + best.nst, [](int a, int b) {
-      const bool pa = (a & (a - 1)) == 0, pb = (b & (b - 1)) == 0;
-      return pa != pb ? pa : a > b;
-    });
-    p[k] = best;
-    p[k].n = (int16_t)n;
-    p[k].tw_off = tw_off;
-    for (int l = 0; l < 7; ++l) p[k].tpl[l] = (int16_t)wide_tpl(p[k], 1 << l);
+    if (!make_wide_plan(n, 0, k, &p[k])) return false;
+    for (int l = 0; l < 7; ++l) p[k].tpl[l] = (int16_t)wide_threads(p[k], 1 << l);
   }
   return true;
 }
@@ -169,9 +170,10 @@ bool grid_desc_only(int ndim, const int n[3], const double L[3], vd_grid* G) {
   g.nreal = (long long)nn[0] * nn[1] * nn[2];
   g.ncplx = (long long)g.h0 * nn[1] * nn[2];
   for (int j = 0; j < 3; ++j) G->L[j] = (j < ndim) ? L[j] : 1.0;
-  bool ok = make_plan(nn[0] / 2, &g.px) && make_wide_plans(nn[0] / 2, 0, g.wx);
-  if (ndim >= 2) ok = ok && make_plan(nn[1], &g.py) && make_wide_plans(nn[1], 0, g.wy);
-  if (ndim == 3) ok = ok && make_plan(nn[2], &g.pz) && make_wide_plans(nn[2], 0, g.wz);
+  // (no plans for the wide passes: nothing is launched on this description)
+  bool ok = make_plan(nn[0] / 2, &g.px);
+  if (ndim >= 2) ok = ok && make_plan(nn[1], &g.py);
+  if (ndim == 3) ok = ok && make_plan(nn[2], &g.pz);
   return ok && g.ncplx * 3 < (1ll << 31);
 }
 }  // namespace vd
@@ -209,10 +211,10 @@ vd_status vd_grid_create(int ndim, const int n[3], const double L[3], vd_grid** 
     split_ld(kl, &g.kfac_dd[j][0], &g.kfac_dd[j][1]);
     g.kfac_f[j] = (float)g.kfac[j];
   }
-  bool ok = make_plan(nn[0] / 2, &g.px) && make_wide_plans(nn[0] / 2, 0, g.wx);
-  if (ndim >= 2) ok = ok && make_plan(nn[1], &g.py) && make_wide_plans(nn[1], 0, g.wy);
+  bool ok = make_plan(nn[0] / 2, &g.px) && make_wide_plans(nn[0] / 2, g.wx);
+  if (ndim >= 2) ok = ok && make_plan(nn[1], &g.py) && make_wide_plans(nn[1], g.wy);
   else g.py = g.px;
-  if (ndim == 3) ok = ok && make_plan(nn[2], &g.pz) && make_wide_plans(nn[2], 0, g.wz);
+  if (ndim == 3) ok = ok && make_plan(nn[2], &g.pz) && make_wide_plans(nn[2], g.wz);
   else g.pz = g.py;
   if (!ok) {
     delete G;

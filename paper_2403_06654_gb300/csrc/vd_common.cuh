@@ -79,7 +79,7 @@ struct FftPlan {
 struct WidePlan {
   int16_t n, nst;
   int8_t rad[8];
-  int16_t tpl[8];   // y/z passes: threads per line for 1, 2, 4, ... 64 lines per block
+  int16_t tpl[8];   // y/z passes: threads per line for 1, 2, 4, ... 64 lines per block (0: not formed)
   int tw_off;
 };
 constexpr int kWideThreads = 256;   // most threads per block of those passes

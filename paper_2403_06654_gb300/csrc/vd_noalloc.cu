@@ -112,7 +112,7 @@ extern "C" vd_status vd_apply_pressure_noalloc(int ndim, const int n[3], const d
   if (ndim < 1 || ndim > 3) return fail(VD_ERR_INVALID_ARG, "ndim must be 1, 2 or 3");
   if (in == out) return fail(VD_ERR_INVALID_ARG, "in and out must not alias");
   // grid description on the stack (same plans and layout as vd_grid_create)
-  vd_grid G;
+  vd_grid G{};
   GridDesc& g = G.g;
   int nn[3] = {1, 1, 1};
   for (int j = 0; j < ndim; ++j) {
@@ -156,8 +156,10 @@ extern "C" vd_status vd_apply_pressure_noalloc(int ndim, const int n[3], const d
   // the transform passes' plans, on the same twiddle tables
   const FftPlan* narrow[3] = {&g.px, &g.py, &g.pz};
   WidePlan* wide[3] = {g.wx, g.wy, g.wz};
-  for (int j = 0; j < ndim; ++j) ok = ok && make_wide_plans(narrow[j]->n, narrow[j]->tw_off, wide[j]);
+  const int cls = wide_class(sizeof(double), g.ncplx);
+  for (int j = 0; j < ndim; ++j) ok = ok && make_wide_plan(narrow[j]->n, narrow[j]->tw_off, cls, &wide[j][cls]);
   if (!ok) return fail(VD_ERR_INVALID_ARG, "axis lengths must factor into 2, 3 and 5");
+  wide_axis_threads(&g);
   g.pk_off = off;
   const size_t ntw = (size_t)off + g.n0 / 2 + 1;
   // scratch layout: flag | twiddles | 1/(N rho) | b^ | x^ | 3 temporaries

@@ -1697,6 +1697,33 @@ static int entry_for_plan(int choice, int kind, const FftPlan& pl, const WidePla
   return need <= kSmemMost ? choice : -1;
 }
 
+// the table's or the built-in choice of a y/z pass
+template <typename T>
+static int axis_choice(const GridDesc& g, int axis, int dir, int cls, long long lines) {
+  const FftPlan& pl = axis == 2 ? g.pz : g.py;
+  const WidePlan& wide = (axis == 2 ? g.wz : g.wy)[cls];
+  const int choice =
+      entry_for_plan<T>(tune_get(0, type_code<T>(), pl.n, axis, dir, tune_scope(cls, lines)), 0, pl, wide);
+  return choice >= 0 ? choice : default_shape(0, type_code<T>(), pl, wide, axis, lines);
+}
+template <typename T>
+static int axis_width(const GridDesc& g, int axis, int choice, int cls, long long lines) {
+  if (choice > 0 && choice <= 64) return choice;
+  return axis_lines(type_code<T>(), axis == 2 ? g.pz : g.py, (axis == 2 ? g.wz : g.wy)[cls], lines);
+}
+
+void wide_axis_threads(GridDesc* g) {
+  const int cls = wide_class(sizeof(double), g->ncplx);
+  for (int axis = 1; axis < g->ndim; ++axis)
+    for (int dir = -1; dir <= 1; dir += 2) {
+      const long long lines = (long long)g->h0 * (axis == 2 ? g->n1 : g->n2);
+      WidePlan& pl = (axis == 2 ? g->wz : g->wy)[cls];
+      const int W = axis_width<double>(*g, axis, axis_choice<double>(*g, axis, dir, cls, lines), cls, lines);
+      int16_t& t = pl.tpl[ilog2(W)];
+      if (t == 0) t = (int16_t)wide_threads(pl, W);
+    }
+}
+
 template <typename T>
 void launch_axis(const AxisProg& P0, int dir, const GridDesc& g, const void* tw, cudaStream_t st) {
   AxisProg P = P0;
@@ -1713,12 +1740,9 @@ void launch_axis(const AxisProg& P0, int dir, const GridDesc& g, const void* tw,
   const bool reg_ok = std::is_same<T, float>::value && (n == 256 || n == 128);
   const FftPlan& pl = P.axis == 2 ? g.pz : g.py;
   const int cls = wide_class(sizeof(T), g.ncplx);
-  const WidePlan& wide = (P.axis == 2 ? g.wz : g.wy)[cls];
-  int choice = entry_for_plan<T>(
-      tune_get(0, type_code<T>(), n, P.axis, dir, tune_scope(cls, inner_n * outer_n)), 0, pl, wide);
-  if (choice < 0) choice = default_shape(0, type_code<T>(), pl, wide, P.axis, inner_n * outer_n);
+  int choice = axis_choice<T>(g, P.axis, dir, cls, inner_n * outer_n);
   if (choice == kChoiceStaged && !(reg_ok && tma_program_ok(P, g))) choice = 0;   // not applicable: register kernel
-  const int W = (choice > 0 && choice <= 64) ? choice : axis_lines(type_code<T>(), pl, wide, inner_n * outer_n);
+  const int W = axis_width<T>(g, P.axis, choice, cls, inner_n * outer_n);
   // algorithmic traffic: every distinct input and output field once, the symbol array once
   unsigned inmask = 0, outmask = 0;
   int nfft = 0;

@@ -129,8 +129,13 @@ template <typename T>
 void wide_axis(const AxisProg& P, int dir, const GridDesc& g, const void* tw, int W, int groups, cudaStream_t st);
 template <typename T>
 void wide_xpass(const XProg& P, const GridDesc& g, const void* tw, int L, int groups, cudaStream_t st);
-// the plans of length n in every radix class, their tables at tw_off
-bool make_wide_plans(int n, int tw_off, WidePlan p[kWideClasses]);
+// the plan of length n in a radix class, its table at tw_off, without threads per line
+bool make_wide_plan(int n, int tw_off, int cls, WidePlan* p);
+// threads per line of a y/z pass with W lines per block
+int wide_threads(const WidePlan& pl, int W);
+// the threads per line of the shapes that launches of double y/z passes on g take: descriptions made
+// for a single call form no others (all of a length's, 21 searches, take up to 114 us)
+void wide_axis_threads(GridDesc* g);
 // The radix class of a pass over a field of ncplx points.  Wide radices make fewer trips through
 // shared memory, narrow ones more and shorter threads.  Double: a warp issues one FP64 instruction
 // per 64 cycles however independent, four warps per SM saturate the pipe, so a small field wants

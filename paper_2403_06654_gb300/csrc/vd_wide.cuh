@@ -551,13 +551,13 @@ static void wide_axis_launch(const AxisProg& P, const GridDesc& g, const cpx<T>*
   const int cls = wide_class(sizeof(T), (long long)g.ncplx);
   const WidePlan& pl = (P.axis == 2 ? g.wz : g.wy)[cls];
   const long long lines = (long long)g.h0 * (P.axis == 2 ? g.n1 : g.n2);
-  const int tpl = pl.tpl[wide_log2(W)];
+  const int l = wide_log2(W), tpl = pl.tpl[l] > 0 ? pl.tpl[l] : wide_threads(pl, W);
   const size_t smem = wide_axis_smem(pl, W, sizeof(T));
   const bool pad = W * (int)sizeof(cpx<T>) < 128;
   auto kernel = pad ? k_axis_w<T, S, true> : k_axis_w<T, S, false>;
   ensure_smem(reinterpret_cast<const void*>(kernel), smem);
-  pdl_launch(kernel, dim3((unsigned)((lines + W - 1) / W), groups), W * tpl, smem, st, P, g, tw, wide_log2(W), tpl,
-                                                                              wide_pad_shift(pl), cls);
+  pdl_launch(kernel, dim3((unsigned)((lines + W - 1) / W), groups), W * tpl, smem, st, P, g, tw, l, tpl,
+             wide_pad_shift(pl), cls);
 }
 
 template <typename T>
