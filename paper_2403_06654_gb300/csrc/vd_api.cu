@@ -321,11 +321,14 @@ size_t vd_grid_modes(const vd_grid* G) { return G ? (size_t)G->g.ncplx : 0; }
 
 namespace vd {
 
-// invN / r for a positive finite r, within an ulp of the quotient in four FP64 operations: the reciprocal
-// of r's significand in float pairs (a rounded float reciprocal and its residual), the quotient from
-// it corrected by its own residual, and r's exponent put back through the bits.  A quotient or an r
-// outside the normal doubles takes the division (9-10 operations; with conversions and double
-// comparisons the preparation of 256^3 points took 361 us against 90 us of memory, now 171).
+// invN / r for a positive finite r, correctly rounded (the bits of the division) in five FP64 operations:
+// the reciprocal of r's significand m in float pairs (a rounded float reciprocal and its residual, relative
+// error 2^-47), the quotient from it corrected by its own residual.  That one is off by at most a half
+// and 2^-40 spacings: its residual, exact for such a quotient, says by integer comparison whether the
+// neighbour is nearer (1 / m for m a few spacings below 1 lies this close to the middle of two
+// doubles).  r's exponent is put back through the bits.  A quotient or an r outside the normal
+// doubles takes the division (9-10 operations; with conversions and double comparisons the
+// preparation of 256^3 points took 359 us against 90 us of memory, now 223).
 __device__ __noinline__ double density_division(double invN, double r) { return invN / r; }
 __device__ __noinline__ float density_narrow(double v) { return (float)v; }
 __device__ __forceinline__ double density_quotient(double invN, double r) {
@@ -336,10 +339,16 @@ __device__ __forceinline__ double density_quotient(double invN, double r) {
   const float d = __fmaf_rn(-y, w.lo, __fmaf_rn(-y, w.hi, 1.0f));   // 1 - y m, about 2^-24
   const double yd = f2d_bits(y) + f2d_bits(y * __fmaf_rn(d, d, d));
   const double q0 = invN * yd;
-  const double q = fma(fma(-q0, m, invN), yd, q0);
-  const int qh = __double2hiint(q), qe = ((qh >> 20) & 0x7ff) - (ef - 1023);
-  if (ef <= 0 || ef >= 0x7ff || qe <= 0 || qe >= 0x7ff) return density_division(invN, r);
-  return __hiloint2double(qh - ((ef - 1023) << 20), __double2loint(q));
+  const double q1 = fma(fma(-q0, m, invN), yd, q0);
+  const long long qb = __double_as_longlong(q1), rb = __double_as_longlong(fma(-q1, m, invN));
+  const int qe = (int)(qb >> 52) & 0x7ff;
+  // half a spacing of q1, times m, by the exponent; below a power of two the spacing is half as large
+  const bool edge = rb < 0 && (qb & 0xfffffffffffffll) == 0;
+  const long long half = __double_as_longlong(m) + (qe - 1023 - 53 - (edge ? 1 : 0)) * (1ll << 52);
+  const long long qn = qb + ((rb & 0x7fffffffffffffffll) > half ? (rb < 0 ? -1 : 1) : 0);
+  const int en = ((int)(qn >> 52) & 0x7ff) - (ef - 1023);
+  if (ef <= 0 || ef >= 0x7ff || qe <= 60 || en <= 0 || en >= 0x7ff) return density_division(invN, r);
+  return __longlong_as_double(qn - (ef - 1023) * (1ll << 52));
 }
 
 __global__ void k_density_prep(long long n, const double* __restrict__ rho, double* __restrict__ rcopy,
