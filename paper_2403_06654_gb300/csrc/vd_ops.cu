@@ -16,17 +16,14 @@
 
 namespace vd {
 
-static inline Xf mkxf(int src, int dst, int pre, int post, bool first, bool last, double scale = 1.0,
-                      bool nofft = false) {
-  Xf x;
+static inline Xf mkxf(int src, int dst, int pre, int post, bool first, bool last, double scale = 1.0) {
+  Xf x{};
   x.src = (int8_t)src;
   x.dst = (int8_t)dst;
   x.pre = (int8_t)pre;
   x.post = (int8_t)post;
   x.first = first ? 1 : 0;
   x.last = last ? 1 : 0;
-  x.nofft = nofft ? 1 : 0;
-  x.pad = 0;
   x.scale = scale;
   return x;
 }

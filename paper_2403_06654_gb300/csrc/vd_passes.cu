@@ -49,20 +49,18 @@ __device__ __forceinline__ void st_el(void* p, int conv, int go, cpx<T> v, bool 
   *q = first ? v : (*q + v);
 }
 
-// kfac[axis] and a scale factor in the arithmetic type.  Float-pair and float values come
-// converted from the host (hi = the double rounded to float), so float kernels issue no
+// kfac[axis] and a scale factor in the arithmetic type, float or float pair.  They come
+// converted from the host (hi = the double rounded to float), so these kernels issue no
 // double -> float conversions: those run on the FP64 pipe, ~1/64 of the float rate on GB300.
 template <typename T>
 __device__ __forceinline__ T kfac_t(const GridDesc& g, int a) {
   if constexpr (std::is_same<T, dd>::value) return dd(g.kfac_dd[a][0], g.kfac_dd[a][1]);
-  else if constexpr (std::is_same<T, float>::value) return g.kfac_f[a];
-  else return g.kfac[a];
+  else return g.kfac_f[a];
 }
 template <typename T>
-__device__ __forceinline__ T scale_t(double s, float hi, float lo) {
+__device__ __forceinline__ T scale_t(float hi, float lo) {
   if constexpr (std::is_same<T, dd>::value) return dd(hi, lo);
-  else if constexpr (std::is_same<T, float>::value) return hi;
-  else return s;
+  else return hi;
 }
 
 // Hint: bring [p, p + bytes) into L2 (p and bytes multiples of 16), in pieces of at most 32 KB.
@@ -136,9 +134,10 @@ size_t shape_smem(int kind, int type, const FftPlan& pl, const WidePlan& wide, i
 // PK (float pairs, radices 2 / 4 / 8 only): the shared-memory transform runs on packed
 // complex float pairs (vd_pdd.cuh), bit-identical to the unpacked engine; its twiddle table
 // holds two entries per twiddle.
-template <typename T, int S, bool CV, bool PK = false>
+template <int S, bool CV, bool PK>
 __global__ void __launch_bounds__(kThreads, 4) k_axis(const AxisProg P, const GridDesc g,
-                                                   const cpx<T>* __restrict__ twg, int lw) {
+                                                   const cpx<dd>* __restrict__ twg, int lw) {
+  using T = dd;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int axis = P.axis;
   const FftPlan& pl = (axis == 2) ? g.pz : g.py;
@@ -217,20 +216,7 @@ __global__ void __launch_bounds__(kThreads, 4) k_axis(const AxisProg P, const Gr
     const void* src = P.in[xf.src];
     void* dst = P.out[xf.dst];
     const int cin = (P.conv_in >> xf.src) & 1, cout = (P.conv_out >> xf.dst) & 1;
-    const T scale = scale_t<T>(xf.scale, xf.scale_hi, xf.scale_lo);
-    if (xf.nofft) {
-      if (colok) {
-#pragma unroll 4
-        for (int q = 0; q < nq; ++q) {
-          const int i = ib + q * istep;
-          const int go = g0 + q * gstep;
-          cpx<T> v = scal(ld_el<T, CV>(src, cin, go), mult(xf.pre, i, go, scale));
-          if (xf.pre & MUL_IK) v = mul_i(v);
-          st_el<T, CV>(dst, cout, go, v, xf.first);
-        }
-      }
-      continue;
-    }
+    const T scale = scale_t<T>(xf.scale_hi, xf.scale_lo);
     __syncthreads();
 #pragma unroll 4
     for (int q = 0; q < nq; ++q) {
@@ -248,7 +234,7 @@ __global__ void __launch_bounds__(kThreads, 4) k_axis(const AxisProg P, const Gr
     // PK: the rows of the next transform's input tile are prefetched into L2 (one thread per
     // row: a row of the tile is W elements of 16 bytes) while this one is transformed
     if constexpr (PK) {
-      if (w == 0 && t + 1 < P.nxf && !P.xf[t + 1].nofft) {
+      if (w == 0 && t + 1 < P.nxf) {
         const cpx<T>* nsrc = reinterpret_cast<const cpx<T>*>(P.in[P.xf[t + 1].src]);   // 16-byte elements
         for (int q = 0; q < nq; ++q) prefetch_line_l2(nsrc + g0 + q * gstep);
       }
@@ -446,20 +432,7 @@ __global__ void __launch_bounds__(kRLines * N2, (N2 == 16 ? 3 : 2)) k_axis_r(con
     const void* src = P.in[xf.src];
     void* dst = P.out[xf.dst];
     const int cin = (P.conv_in >> xf.src) & 1, cout = (P.conv_out >> xf.dst) & 1;
-    const T scale = scale_t<T>(xf.scale, xf.scale_hi, xf.scale_lo);
-    if (xf.nofft) {
-      if (colok) {
-#pragma unroll
-        for (int j = 0; j < N1; ++j) {
-          const int i = N2 * j + t;
-          const int go = gbase + i * line_stride;
-          cpx<T> v = scal(ld_el<T>(src, cin, go), mult(xf.pre, i, go, scale));
-          if (xf.pre & MUL_IK) v = mul_i(v);
-          st_el<T>(dst, cout, go, v, xf.first);
-        }
-      }
-      continue;
-    }
+    const T scale = scale_t<T>(xf.scale_hi, xf.scale_lo);
     cpx<T> u[N1];
 #pragma unroll
     for (int j = 0; j < N1; ++j) {
@@ -709,7 +682,7 @@ __global__ void __launch_bounds__(kRLines * N2, (N2 == 16 ? 3 : 6))
       return;
     }
     void* dst = P.out[xf.dst];
-    const T scale = scale_t<T>(xf.scale, xf.scale_hi, xf.scale_lo);
+    const T scale = scale_t<T>(xf.scale_hi, xf.scale_lo);
     cpx<T> u[N1];
 #pragma unroll
     for (int j = 0; j < N1; ++j) {
@@ -785,9 +758,10 @@ __global__ void __launch_bounds__(kRLines * N2, (N2 == 16 ? 3 : 6))
 // PK (float pairs, radices 2 / 4 / 8 only): the transforms and the (un)packing of the real
 // transform run on packed complex float pairs (vd_pdd.cuh), bit-identical to the unpacked
 // code, with packed twiddle tables for both directions and the packing twiddles W_{n0}^k.
-template <typename T, bool CV, bool PK = false, int MINB = 3>
+template <bool CV, bool PK, int MINB>
 __global__ void __launch_bounds__(kThreads, MINB) k_xpass(const XProg P, const GridDesc g,
-                                                    const cpx<T>* __restrict__ twg, int llpc, int ltpl) {
+                                                    const cpx<dd>* __restrict__ twg, int llpc, int ltpl) {
+  using T = dd;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int m = g.n0 / 2;
   const int h0 = g.h0;
@@ -831,13 +805,12 @@ __global__ void __launch_bounds__(kThreads, MINB) k_xpass(const XProg P, const G
   const bool lok = line < nl;
   const int lofs = line * ls;
   const T kfx = kfac_t<T>(g, 0);
-  const T scale = scale_t<T>(P.scale, P.scale_hi, P.scale_lo);
+  const T scale = scale_t<T>(P.scale_hi, P.scale_lo);
   const T* __restrict__ symarr = reinterpret_cast<const T*>(P.symarr) + (line0 + line) * h0;
-  // float pairs: the block's lines of a component are one contiguous chunk (16 bytes per
-  // element, float pairs and doubles alike); the weights and each next component's input are
-  // prefetched into L2 while the current component is transformed
-  constexpr bool kPrefetch = std::is_same<T, dd>::value;
-  if (kPrefetch && tid == 0 && P.mode == 0 && P.wfield)
+  // the block's lines of a component are one contiguous chunk (16 bytes per element, float pairs
+  // and doubles alike); the weights and each next component's input are prefetched into L2
+  // while the current component is transformed
+  if (tid == 0 && P.mode == 0 && P.wfield)
     prefetch_l2(reinterpret_cast<const cpx<T>*>(P.wfield) + line0 * m, (unsigned)(nl * m) * 16u);
   // the transforms and element conversions of the engine in use
   auto fft_fwd = [&](E* a, E* b) -> E* {
@@ -860,7 +833,7 @@ __global__ void __launch_bounds__(kThreads, MINB) k_xpass(const XProg P, const G
     const int mode = aux ? 2 : P.mode;
     E* res;
     __syncthreads();
-    if (kPrefetch && tid == 0 && c + 1 < P.ncomp) {
+    if (tid == 0 && c + 1 < P.ncomp) {
       const int per = (P.mode == 1) ? m : h0;   // elements per line of the next input
       prefetch_l2(reinterpret_cast<const cpx<T>*>(P.in[c + 1]) + line0 * per, (unsigned)(nl * per) * 16u);
     }
@@ -913,7 +886,7 @@ __global__ void __launch_bounds__(kThreads, MINB) k_xpass(const XProg P, const G
       if (mode == 2) {
         void* o = aux ? P.aux_out : P.out[c];
         const int cout = aux ? P.aux_conv : ((P.conv_out >> c) & 1);
-        const T sc = aux ? scale_t<T>(P.aux_scale, P.aux_scale_hi, P.aux_scale_lo) : scale;
+        const T sc = aux ? scale_t<T>(P.aux_scale_hi, P.aux_scale_lo) : scale;
         const int rbase = (int)((line0 + line) * m);
         if (lok)
           for (int j = t0; j < m; j += TPL) {
@@ -923,23 +896,15 @@ __global__ void __launch_bounds__(kThreads, MINB) k_xpass(const XProg P, const G
         continue;
       }
       if (P.wfield && lok) {
-        bool done_pair = false;
-        if constexpr (PK) {
-          // lane by lane the float-pair products z.x wv.x and z.y wv.y
-          const cpx<T>* __restrict__ wf = reinterpret_cast<const cpx<T>*>(P.wfield) + (line0 + line) * m;
+        const cpx<T>* __restrict__ wf = reinterpret_cast<const cpx<T>*>(P.wfield) + (line0 + line) * m;
 #pragma unroll 4
-          for (int j = t0; j < m; j += TPL) res[lofs + j] = p_scal(res[lofs + j], pdd_of(wf[j]));
-          done_pair = true;
-        }
-        if constexpr (!PK) {
-          if (!done_pair) {
-            const cpx<T>* __restrict__ wf = reinterpret_cast<const cpx<T>*>(P.wfield) + (line0 + line) * m;
-#pragma unroll 4
-            for (int j = t0; j < m; j += TPL) {
-              const cpx<T> z = res[lofs + j];
-              const cpx<T> wv = wf[j];
-              res[lofs + j] = mk<T>(z.x * wv.x, z.y * wv.y);
-            }
+        for (int j = t0; j < m; j += TPL) {
+          if constexpr (PK) {   // lane by lane the float-pair products z.x wv.x and z.y wv.y
+            res[lofs + j] = p_scal(res[lofs + j], pdd_of(wf[j]));
+          } else {
+            const cpx<T> z = res[lofs + j];
+            const cpx<T> wv = wf[j];
+            res[lofs + j] = mk<T>(z.x * wv.x, z.y * wv.y);
           }
         }
       }
@@ -1100,7 +1065,7 @@ __global__ void __launch_bounds__(256, (sizeof(T) == 4 ? 4 : 1)) k_xpass_r(const
   const bool lok = line0 + line < nlines;
   cpx<T>* Yl = buf + line * LS;
   const T kfx = kfac_t<T>(g, 0);
-  const T scale = scale_t<T>(P.scale, P.scale_hi, P.scale_lo);
+  const T scale = scale_t<T>(P.scale_hi, P.scale_lo);
   const int lb = (int)((line0 + line) * h0);      // spectral line base
   const int rb = (int)((line0 + line) * M);       // real line base (complex pairs)
   const T* __restrict__ symarr = reinterpret_cast<const T*>(P.symarr);
@@ -1272,7 +1237,7 @@ __global__ void __launch_bounds__(256, 3) k_xpass_tma(const XProg P, const GridD
   cpx<T>* Yl = buf + line * LS;
   const cpx<T>* Sl = stage + line * pitch;
   const T kfx = kfac_t<T>(g, 0);
-  const T scale = scale_t<T>(P.scale, P.scale_hi, P.scale_lo);
+  const T scale = scale_t<T>(P.scale_hi, P.scale_lo);
 
   for (int it = 0; it < nitems; ++it) {
     const long long line0 = (long long)((int)blockIdx.x + (it / nc) * (int)gridDim.x) * LINES;
@@ -1546,14 +1511,14 @@ static FftPlan narrow_plan(const WidePlan& w) {
   return p;
 }
 
-template <typename T, int S, bool CV, bool PK>
-static void launch_k_axis(const AxisProg& P, const GridDesc& g, const cpx<T>* tw, int W, long long blocks,
+template <int S, bool CV, bool PK>
+static void launch_k_axis(const AxisProg& P, const GridDesc& g, const cpx<dd>* tw, int W, long long blocks,
                           size_t smem, cudaStream_t st, int per = 8) {
   // `per` elements per thread, whole lines' worth of warps
   const int n = (P.axis == 2) ? g.pz.n : g.py.n;
   const int threads = std::min(kThreads, std::max(32, W * std::max((n + per - 1) / per, (31 + W) / W)));
-  ensure_smem(reinterpret_cast<const void*>(k_axis<T, S, CV, PK>), smem);
-  pdl_launch(k_axis<T, S, CV, PK>, (unsigned)blocks, threads, smem, st, P, g, tw, ilog2(W));
+  ensure_smem(reinterpret_cast<const void*>(k_axis<S, CV, PK>), smem);
+  pdl_launch(k_axis<S, CV, PK>, (unsigned)blocks, threads, smem, st, P, g, tw, ilog2(W));
 }
 
 template <typename T, int S, int N1, int N2>
@@ -1635,7 +1600,7 @@ static bool tma_program_ok(const AxisProg& P, const GridDesc& g) {
   if (P.conv_in || P.conv_out || P.nxf <= 0) return false;
   if (P.axis == 1 && (g.n1 & 1)) return false;
   for (int t = 0; t < P.nxf; ++t)
-    if (P.xf[t].nofft || P.xf[t].src >= kTmaMaxIn) return false;
+    if (P.xf[t].src >= kTmaMaxIn) return false;
   for (int b = 1; b < P.nxf; ++b)
     for (int a = 0; a < b; ++a)
       if (P.in[P.xf[b].src] == P.out[P.xf[a].dst]) return false;
@@ -1745,17 +1710,15 @@ void launch_axis(const AxisProg& P0, int dir, const GridDesc& g, const void* tw,
   const int W = axis_width<T>(g, P.axis, choice, cls, inner_n * outer_n);
   // algorithmic traffic: every distinct input and output field once, the symbol array once
   unsigned inmask = 0, outmask = 0;
-  int nfft = 0;
   bool sym = false;
   for (int t = 0; t < P.nxf; ++t) {
     inmask |= 1u << P.xf[t].src;
     outmask |= 1u << P.xf[t].dst;
-    nfft += P.xf[t].nofft ? 0 : 1;
     sym = sym || ((P.xf[t].pre | P.xf[t].post) & MUL_SYM);
   }
   const double fb = (double)g.ncplx * sizeof(cpx<T>);
   const double bytes = (__builtin_popcount(inmask) + __builtin_popcount(outmask)) * fb + (sym ? g.ncplx * sizeof(T) : 0);
-  const double flops = (double)nfft * (double)g.ncplx * 5.0 * std::log2((double)n);
+  const double flops = (double)P.nxf * (double)g.ncplx * 5.0 * std::log2((double)n);
   ProfScope ps(std::is_same<T, dd>::value ? PC_AXISDD : (sizeof(T) == 8 ? PC_AXIS64 : PC_AXIS32), st, bytes,
                flops);
   if constexpr (std::is_same<T, float>::value) {
@@ -1791,10 +1754,10 @@ void launch_axis(const AxisProg& P0, int dir, const GridDesc& g, const void* tw,
     const size_t smem = sizeof(cpx<T>) * (size_t)(n + 2 * W * n);
     if (choice != kChoiceUnpacked && p_plan_ok(pl, kThreads / W)) {
       const size_t psmem = smem + sizeof(pdd) * (size_t)n;   // the second twiddle table
-      if (dir < 0 && cv) launch_k_axis<T, -1, true, true>(P, g, twp, W, blocks, psmem, st);
-      else if (dir < 0) launch_k_axis<T, -1, false, true>(P, g, twp, W, blocks, psmem, st);
-      else if (cv) launch_k_axis<T, +1, true, true>(P, g, twp, W, blocks, psmem, st);
-      else launch_k_axis<T, +1, false, true>(P, g, twp, W, blocks, psmem, st);
+      if (dir < 0 && cv) launch_k_axis<-1, true, true>(P, g, twp, W, blocks, psmem, st);
+      else if (dir < 0) launch_k_axis<-1, false, true>(P, g, twp, W, blocks, psmem, st);
+      else if (cv) launch_k_axis<+1, true, true>(P, g, twp, W, blocks, psmem, st);
+      else launch_k_axis<+1, false, true>(P, g, twp, W, blocks, psmem, st);
       return;
     }
     GridDesc gn = g;
@@ -1803,22 +1766,22 @@ void launch_axis(const AxisProg& P0, int dir, const GridDesc& g, const void* tw,
       (P.axis == 2 ? gn.pz : gn.py) = narrow_plan((P.axis == 2 ? g.wz : g.wy)[0]);
       per = 4;
     }
-    if (dir < 0 && cv) launch_k_axis<T, -1, true, false>(P, gn, twp, W, blocks, smem, st, per);
-    else if (dir < 0) launch_k_axis<T, -1, false, false>(P, gn, twp, W, blocks, smem, st, per);
-    else if (cv) launch_k_axis<T, +1, true, false>(P, gn, twp, W, blocks, smem, st, per);
-    else launch_k_axis<T, +1, false, false>(P, gn, twp, W, blocks, smem, st, per);
+    if (dir < 0 && cv) launch_k_axis<-1, true, false>(P, gn, twp, W, blocks, smem, st, per);
+    else if (dir < 0) launch_k_axis<-1, false, false>(P, gn, twp, W, blocks, smem, st, per);
+    else if (cv) launch_k_axis<+1, true, false>(P, gn, twp, W, blocks, smem, st, per);
+    else launch_k_axis<+1, false, false>(P, gn, twp, W, blocks, smem, st, per);
   } else {
     wide_axis<T>(P, dir, g, tw, W, split_axis(P, (inner_n * outer_n + W - 1) / W), st);
   }
 }
 
-template <typename T, bool CV, bool PK, int MINB = 3>
-static void launch_k_xpass(const XProg& P, const GridDesc& g, const cpx<T>* tw, int L, long long blocks, size_t smem,
+template <bool CV, bool PK, int MINB>
+static void launch_k_xpass(const XProg& P, const GridDesc& g, const cpx<dd>* tw, int L, long long blocks, size_t smem,
                            cudaStream_t st, int per = 8) {
-  ensure_smem(reinterpret_cast<const void*>(k_xpass<T, CV, PK, MINB>), smem);
+  ensure_smem(reinterpret_cast<const void*>(k_xpass<CV, PK, MINB>), smem);
   // threads per line: a power of two, `per` elements each, at least a warp per block
   const int tpl = std::min(kThreads / L, std::max(pow2_at_least((g.px.n + per - 1) / per), pow2_at_least((31 + L) / L)));
-  pdl_launch(k_xpass<T, CV, PK, MINB>, (unsigned)blocks, L * tpl, smem, st, P, g, tw, ilog2(L), ilog2(tpl));
+  pdl_launch(k_xpass<CV, PK, MINB>, (unsigned)blocks, L * tpl, smem, st, P, g, tw, ilog2(L), ilog2(tpl));
 }
 
 template <typename T>
@@ -1905,10 +1868,10 @@ void launch_xpass(const XProg& P0, const GridDesc& g, const void* tw, cudaStream
       const size_t psmem = smem + sizeof(pdd) * (size_t)(3 * m);
       // four blocks per SM (64 registers) where their shared memory fits, else three
       const bool four = 4 * (psmem + 1024) <= 228 * 1024;
-      if (cv && four) launch_k_xpass<T, true, true, 4>(P, g, twp, L, blocks, psmem, st);
-      else if (cv) launch_k_xpass<T, true, true, 3>(P, g, twp, L, blocks, psmem, st);
-      else if (four) launch_k_xpass<T, false, true, 4>(P, g, twp, L, blocks, psmem, st);
-      else launch_k_xpass<T, false, true, 3>(P, g, twp, L, blocks, psmem, st);
+      if (cv && four) launch_k_xpass<true, true, 4>(P, g, twp, L, blocks, psmem, st);
+      else if (cv) launch_k_xpass<true, true, 3>(P, g, twp, L, blocks, psmem, st);
+      else if (four) launch_k_xpass<false, true, 4>(P, g, twp, L, blocks, psmem, st);
+      else launch_k_xpass<false, true, 3>(P, g, twp, L, blocks, psmem, st);
       return;
     }
     GridDesc gn = g;
@@ -1917,8 +1880,8 @@ void launch_xpass(const XProg& P0, const GridDesc& g, const void* tw, cudaStream
       gn.px = narrow_plan(g.wx[0]);
       per = 4;
     }
-    if (cv) launch_k_xpass<T, true, false>(P, gn, twp, L, blocks, smem, st, per);
-    else launch_k_xpass<T, false, false>(P, gn, twp, L, blocks, smem, st, per);
+    if (cv) launch_k_xpass<true, false, 3>(P, gn, twp, L, blocks, smem, st, per);
+    else launch_k_xpass<false, false, 3>(P, gn, twp, L, blocks, smem, st, per);
   } else {
     wide_xpass<T>(P, g, tw, L, split_xpass(P, (nlines + L - 1) / L), st);
   }

@@ -34,8 +34,6 @@ struct Xf {
   int8_t src, dst, pre, post;
   int8_t first;   // start a new accumulation for dst
   int8_t last;    // write dst after this transform
-  int8_t nofft;   // skip the transform (pure diagonal multiply)
-  int8_t pad;
   double scale;
   float scale_hi, scale_lo;   // float-pair split of scale (set on the host)
 };

@@ -190,16 +190,6 @@ __global__ void __launch_bounds__(kWideThreads, (sizeof(T) == 8 ? 2 : 3))
       if (flags & MUL_NEGK2) c *= -(ka * ka + kp2);
       return c;
     };
-    if (xf.nofft) {
-      if (ok)
-        for (int i = ib; i < n; i += tpl) {
-          cpx<T> v = scal(src[g0 + i * ls], mult(xf.pre, i, scale));
-          if (xf.pre & MUL_IK) v = mul_i(v);
-          cpx<T>* q = dst + g0 + i * ls;
-          *q = xf.first ? v : (*q + v);
-        }
-      continue;
-    }
     // an even number of stages ends reading A, which the next transform's first stage writes
     if (t >= (int)gridDim.y && !(nst & 1)) __syncthreads();
     auto first_stage = [&](auto rc) {
@@ -526,7 +516,7 @@ __global__ void __launch_bounds__(kWideThreads, (sizeof(T) == 8 ? 2 : 3))
 #pragma unroll 2
     for (; it.l < nl; it.next()) {
       const int k = it.k, go = (line0 + it.l) * h0;
-      const cpx<T> Z = cur[at(it.l, k == m ? 0 : k)], Y = conjg(cur[at(it.l, k == 0 ? 0 : m - k)]);
+      const cpx<T> Z = cur[at(it.l, k)], Y = conjg(cur[at(it.l, k == 0 ? 0 : m - k)]);
       const cpx<T> s = Z + Y, ic = mul_i(cmul(Z - Y, pk[k]));
       cpx<T> lo = s - ic, hi = conjg(s + ic);
       lo = scal(lo, factor(post, k, go + k, scale));
