@@ -75,9 +75,10 @@ typedef enum { VD_OP_PRESSURE = 0, VD_OP_VELOCITY = 1, VD_OP_KRHO = 2 } vd_op;
 typedef enum { VD_SOLVER_CG = 0, VD_SOLVER_GMRES = 1, VD_SOLVER_RMR = 2 } vd_solver;
 typedef enum {
   VD_PREC_FP64 = 0,  /* every transform, product and reduction in IEEE double */
-  VD_PREC_MIXED = 1, /* inner Krylov solve with float transforms and preconditioner, double
-                        dot products, inside a double iterative-refinement loop whose true
-                        residual uses the double operator */
+  VD_PREC_MIXED = 1, /* inner Krylov solve with float transforms, preconditioner and vectors, dot
+                        products of float terms summed in float pairs and double, inside a
+                        double iterative-refinement loop whose true residual uses the
+                        double operator */
   VD_PREC_MIXED_DD = 2 /* as VD_PREC_MIXED, but the refinement residual b - A x is formed with
                         float-pair transforms (two floats per value, ~2^-48 relative rounding,
                         on the FP32 pipes; storage stays double; the velocity operator's

@@ -703,7 +703,7 @@ constexpr double kPairRatio = 10.0;
 static double auto_inner_tol(const vd_grid*) { return 1e-5; }
 
 static bool coef_in_pairs(const vd_grid* G, vd_op op, int coef_pair) {
-  if (op == VD_OP_VELOCITY) return false;   // the velocity bracket multiplies by 1/rho in double
+  if (op == VD_OP_VELOCITY) return false;   // the velocity bracket multiplies by 1/rho as a pair or in double
   if (coef_pair != 0) return coef_pair > 0;
   return G->rho_max > kPairRatio * G->rho_min;
 }

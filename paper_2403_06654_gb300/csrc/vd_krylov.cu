@@ -1,9 +1,10 @@
 // Krylov solvers: CG, restarted GMRES (CGS2 Arnoldi) and Richardson Minimal Residual.
 //
-// Every reduction is a two-level deterministic sum in double precision: a fixed number of
-// blocks writes per-block partials, and the last block to finish (atomic ticket) adds them
-// in a fixed order and runs the scalar epilogue of the algorithm (step lengths, Givens
-// rotations, convergence tests) in one thread.  The scalars never leave the device; the
+// Every reduction is a deterministic sum in a fixed order: threads, then lanes and warps of a block,
+// then blocks (as many as the vector's length asks for) whose double partials the last block to
+// finish (atomic ticket) adds; it runs the scalar epilogue of the algorithm (step lengths, convergence
+// tests in one thread, the Givens rotations of a GMRES step in one warp).  Double vectors are summed in
+// double throughout, float vectors in float pairs up to the warp (Acc).  The scalars never leave the device; the
 // host only reads the `done` flag every `check_every` iterations, one batch
 // behind: it waits for the flag of batch k-1 with batch k already queued.  Kernels of an
 // iteration return at once when the flag is set, so iterations enqueued ahead cost a launch
@@ -476,8 +477,11 @@ __device__ __forceinline__ cpx<T> weighted(cpx<T> v, int kx, int h0) {
 // with a compensated float sum (Knuth's two-sum carries the rounding error of every addition
 // in a second float), about as accurate as a double accumulation of the float terms but
 // without FP64 work per element: the FP64 pipe of GB300 is ~1/64 of the float rate and was
-// the limiter of these memory-bound kernels.  The cross-thread sum of the per-thread totals
-// is done in double (reduce_last).
+// the limiter of these memory-bound kernels.  The per-thread totals stay float pairs until one value per
+// warp is left, which is widened; warps and blocks add in double (block_sums, reduce_last).  Dots of
+// 2^12 to 2^20 terms, orthogonal vectors among them, err by 4e-10 to 2e-11 of the sum of their
+// terms' magnitudes either way (the products are rounded to float); the pairs differ from double
+// sums by less than 1e-18 of it.
 template <typename T>
 struct Acc {
   double a = 0.0;
@@ -1362,9 +1366,11 @@ vd_status krylov_solve(const SpecSystem& sys, const SolveOpts& o, const void* b,
       { ProfScope ps_(sizeof(T) == 4 ? PC_VEC32 : PC_VEC64, st, (double)2 * len * sizeof(cpx<T>), 0.0); pdl_launch(k_gm_scale<T>, eb, 256, 0, st, ixe, V, V, kw.ks, 1); }
       // the flag of step j is read with step j + check already queued (its kernels see the device's
       // flag and return), so the device does not wait for the host between steps.  Not for three
-      // components: their step that comes to nothing is 25 launches, as long as the waits of a cycle
-      // (96^3 velocity solve 5.76 ms ahead, 5.66 not; 480 x 360 pressure 5.66 and 6.24, 320^2 velocity 2.56
-      // and 2.67).
+      // components: the step that comes to nothing at the end of their cycle is 25 launches, more than the
+      // waits it saves.  Solves ahead and not, us: pressure 64^2 mixed 1729 and 1850, 512^2 fp64 5147 and
+      // 5297, 32^3 mixed 1870 and 2047, 128^3 mixed_dd 5969 and 6170; velocity 64^2 mixed 962 and 986, 512^2
+      // 3005 and 3096; three components 32^3 mixed 1416 and 1420, 48^3 1700 and 1656, 96^3 5708 and
+      // 5627, 128^3 fp64 37390 and 36880 (nine sizes in all, no exception).
       const bool ahead = hp && sys.ncomp < 3;
       int snaps = 0;
       long long mark = 0;

@@ -13,7 +13,7 @@
 namespace vd {
 
 constexpr int kMaxRestart = 64;
-constexpr int kRedBlocks = 608;   // fixed block count of every reduction (deterministic; 4 per SM on 152 SMs)
+constexpr int kRedBlocks = 608;   // most blocks of a reduction (4 per SM on 152 SMs); fewer for short vectors, by length alone
 constexpr int kRedThreads = 256;
 constexpr int kInnerGuard = 100;  // divergence guard of the inner float CG solves (see KState::guard)
 constexpr int kStallWindow = 8;   // iterations without a halving of the residual that count as a stall

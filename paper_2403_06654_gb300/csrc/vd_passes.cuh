@@ -137,9 +137,10 @@ void wide_axis_threads(GridDesc* g);
 // The radix class of a pass over a field of ncplx points.  Wide radices make fewer trips through
 // shared memory, narrow ones more and shorter threads.  Double: a warp issues one FP64 instruction
 // per 64 cycles however independent, four warps per SM saturate the pipe, so a small field wants
-// many threads of few operations (96 x 96 double apply: 8 radix-5-and-below stages 78 us, radix 8
-// 96, radix 16 127; 320 x 320: 127, 135; 512 x 1024: 312, 302; 80^3: 411, 393, 16: 504).  Float: latency
-// until the field is large (512 x 1024 forward: radix 8 14.4 us, 16 18.6; 320 x 256 x 160: 145, 108).
+// many threads of few operations (pressure apply in radices up to 5, 8 and 16, us: 96 x 96 59, 70, 85;
+// 320 x 320 103, 108, 138; 512 x 1024 281, 277, 275; 80^3 366, 335, 342; 128^3 1351, 1292, 1148).  Float:
+// latency until the field is large (forward transform in radices up to 8 and 16: 512 x 1024 13.8 and
+// 14.7, 128 x 120 x 128 20.6 and 16.9, 320 x 256 x 160 137 and 92).
 inline int wide_class(size_t el, long long ncplx) {
   if (el == sizeof(float)) return ncplx >= (1 << 20) ? 2 : 1;
   return ncplx >= (1 << 21) ? 2 : (ncplx >= (1 << 17) ? 1 : 0);

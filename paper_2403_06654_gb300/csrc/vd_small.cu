@@ -18,9 +18,9 @@
 // they are added, and a quotient or square root that only reports is formed when it is asked for.
 // N = 256 CG: 19 us per iteration before, 9 now (a solve of 22 iterations 460 -> 243 us).
 //
-// The recurrences are the library's own: the real-transform packing of the x pass, the same recurrences (PCG, right-preconditioned RMR, right-preconditioned
-// GMRES(m) with classical Gram-Schmidt applied twice and Givens rotations), the same tests
-// and statuses as the pass-by-pass solve (vd_krylov.cu).  Eligible: the pressure operator in
+// The arithmetic is the library's own: the real-transform packing of the x pass, the recurrences (PCG,
+// right-preconditioned RMR and GMRES(m) with classical Gram-Schmidt applied twice and Givens rotations), tests
+// and statuses of the pass-by-pass solve (vd_krylov.cu).  Eligible: the pressure operator in
 // FP64 on a 1D grid whose vectors fit in shared memory (GMRES: (m + 7) half spectra).
 #include "vd_internal.h"
 #include "vd_fft.cuh"

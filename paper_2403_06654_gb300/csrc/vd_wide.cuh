@@ -1,8 +1,8 @@
 // Transform passes of any supported length in float and double: Stockham stages of radices up to
 // 16 whose first stage loads from global memory and whose last one stores to it.
 //
-// A line of length n = R_0 ... R_{s-1} (two stages up to 256, three up to 1024) makes one
-// shared-memory round trip per stage boundary only.  A thread transforms whole butterflies: in
+// A line of length n = R_0 ... R_{s-1} (radices up to 5, 8 or 16 by the size of the field, wide_class;
+// 256 points in four, three or two stages) makes one shared-memory round trip per stage boundary only.  A thread transforms whole butterflies: in
 // the first stage butterfly i of radix R reads elements i + r n/R, in the last one it writes
 // elements i + r n/R, so both stages' rows are the thread's own registers.  In the fused x pass
 // the forward transform runs its radices in reverse order: the last inverse butterfly's outputs

@@ -3,6 +3,9 @@ lengths keeps its built-in shapes.  Shown by the bits: on the large float field 
 kernels win or are the built-in choice, on the small one the general kernel, which rounds differently."""
 
 import math
+import os
+import subprocess
+import sys
 
 import pytest
 import torch
@@ -52,3 +55,21 @@ def test_tuning_a_large_field_leaves_small_ones():
     finally:
         _erase()
     assert vd.vd_autotune_table() == []
+
+
+def test_tuned_table_survives_its_file(tmp_path, monkeypatch):
+    """A later process reads the tuner's file into the same entries."""
+    _erase()
+    f = tmp_path / "tune.txt"
+    monkeypatch.setenv("VD_TUNE_FILE", str(f))
+    try:
+        vd.vd_autotune(vd.Grid((24, 20, 18), (2 * math.pi,) * 3), ("fp64", "mixed_dd"))
+        table = sorted(vd.vd_autotune_table())
+    finally:
+        _erase()
+    code = "import paper_2403_06654_gb300 as vd; print(sorted(vd.vd_autotune_table()))"
+    env = dict(os.environ, PYTHONPATH=os.path.dirname(os.path.dirname(os.path.abspath(__file__))))
+    out = subprocess.run([sys.executable, "-c", code], env=env, capture_output=True, text=True, check=True).stdout
+    assert table and out.strip() == str(table)
+    # scope and built-in flag follow the six numbers of an entry
+    assert all(len(line.split()) == 8 for line in f.read_text().splitlines())
